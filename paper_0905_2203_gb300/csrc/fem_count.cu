@@ -947,32 +947,47 @@ int scan_exclusive(cudaStream_t st, int32_t *data, int64_t m, int32_t *tmp, int3
 // between consecutive event times within +-w events of it (a quiet spot, so
 // few occurrences span the boundary and few entry classes are needed); a
 // boundary always falls where the time changes.
-__global__ void k_segments(const int32_t *__restrict__ tm, int64_t n, int P, int64_t *__restrict__ seg) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > P) return;
-    int64_t b;
-    if (p == 0) {
-        b = 0;
-    } else if (p == P) {
-        b = n;
-    } else {
-        const int64_t nom = (int64_t)((__int128)n * p / P);
-        const int64_t seg_len = n / P;
-        const int64_t w = seg_len / 4 < 4096 ? seg_len / 4 : 4096;
-        const int64_t lo = nom - w > 1 ? nom - w : 1;
-        const int64_t hi = nom + w < n - 1 ? nom + w : n - 1;
-        b = nom;
-        int64_t best = -1;
-        for (int64_t i = lo; i <= hi; ++i) {
-            const int64_t gap = (int64_t)tm[i] - tm[i - 1];
-            if (gap > best) {
-                best = gap;
-                b = i;
-            }
-        }
-        if (best <= 0)
-            while (b < n && b > 0 && tm[b] == tm[b - 1]) ++b;
+//
+// One block per boundary: its threads take the up to 8193 places side by side
+// (coalesced reads) and reduce to the largest gap, the first place among
+// equal ones.  One thread per boundary walked them one after another, a chain
+// of 8193 loads that held the whole launch: 360-560 us for a 1M-event
+// recording cut into 130 segments.
+constexpr int kSegThreads = 256;
+
+__global__ void __launch_bounds__(kSegThreads) k_segments(const int32_t *__restrict__ tm, int64_t n, int P,
+                                                          int64_t *__restrict__ seg) {
+    __shared__ unsigned long long s_best[kSegThreads / 32];
+    const int p = blockIdx.x;
+    if (p == 0 || p == P) {
+        if (threadIdx.x == 0) seg[p] = p == 0 ? 0 : n;
+        return;
     }
+    const int64_t nom = (int64_t)((__int128)n * p / P);
+    const int64_t seg_len = n / P;
+    const int64_t w = seg_len / 4 < 4096 ? seg_len / 4 : 4096;
+    const int64_t lo = nom - w > 1 ? nom - w : 1;
+    const int64_t hi = nom + w < n - 1 ? nom + w : n - 1;
+    // (gap, places before the end of the range): the maximum is the largest
+    // gap at its first place; 0 = no place (gaps are never negative)
+    unsigned long long best = 0;
+#pragma unroll 4
+    for (int64_t i = lo + threadIdx.x; i <= hi; i += kSegThreads) {
+        const uint32_t gap = (uint32_t)(tm[i] - tm[i - 1]);
+        const unsigned long long v = ((unsigned long long)gap << 32) | (uint32_t)(hi - i + 1);
+        best = v > best ? v : best;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        best = y > best ? y : best;
+    }
+    if ((threadIdx.x & 31) == 0) s_best[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int q = 1; q < kSegThreads / 32; ++q) best = s_best[q] > best ? s_best[q] : best;
+    int64_t b = best ? hi + 1 - (int64_t)(uint32_t)best : nom;
+    if ((best >> 32) == 0)
+        while (b < n && b > 0 && tm[b] == tm[b - 1]) ++b;
     seg[p] = b;
 }
 
@@ -989,7 +1004,7 @@ int stream_segments(fem_ctx *ctx, fem_stream *s, int P, const int64_t **seg) {
     }
     void *p = nullptr;
     FEM_TRY(dev_alloc(ctx, &p, sizeof(int64_t) * (P + 1)));
-    k_segments<<<(P + 1 + 127) / 128, 128, 0, ctx->stream>>>(s->d_time, s->n, P, static_cast<int64_t *>(p));
+    k_segments<<<P + 1, kSegThreads, 0, ctx->stream>>>(s->d_time, s->n, P, static_cast<int64_t *>(p));
     FEM_CUDA_TRY(cudaGetLastError());
     s->segs[P] = static_cast<int64_t *>(p);
     *seg = static_cast<int64_t *>(p);
@@ -997,7 +1012,7 @@ int stream_segments(fem_ctx *ctx, fem_stream *s, int P, const int64_t **seg) {
 }
 
 int launch_segments(cudaStream_t st, const int32_t *time, int64_t n, int P, int64_t *seg) {
-    k_segments<<<(P + 1 + 127) / 128, 128, 0, st>>>(time, n, P, seg);
+    k_segments<<<P + 1, kSegThreads, 0, st>>>(time, n, P, seg);
     FEM_CUDA_TRY(cudaGetLastError());
     return FEM_OK;
 }
