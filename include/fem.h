@@ -105,10 +105,11 @@ typedef struct {
                              CTA, tile size, segment count, kernel) the first
                              time a workload signature is seen and keep the
                              fastest in the context's tuning cache */
-    int kernel;           /* 0 = choose per launch (grid-wide local
-                             tracking (4) for at most 256 episodes over a
-                             recording of at least 2^20 events, otherwise
-                             warp-per-item local tracking (7)), 1 = always the tiled
+    int kernel;           /* 0 = choose per launch (warp-per-item local
+                             tracking (7); grid-wide local tracking (4) for
+                             at most 256 episodes over a recording of at
+                             least 2^20 events whose spans are too wide to
+                             cut it into segments), 1 = always the tiled
                              shared-memory broadcast kernel, 2 = the sparse
                              per-type-list kernel where it applies, 3 = the
                              sparse kernel with per-node branching instead of

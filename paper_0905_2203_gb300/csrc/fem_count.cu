@@ -1784,11 +1784,19 @@ struct CountCall {
     int mode = 0;                        // 0 exact, 1 plain, 2 relaxed
     double seg_div = 1.0;                // fallback rounds divide the segment count
     bool force_tiled = false;            // last fallback round: tiled kernel, one segment
+    int64_t sumhi = -1;                  // largest sum of an episode's upper bounds (-1: not known)
+    bool plt_ok = false;                 // grid-wide local tracking may count this call (or its recounts)
     fem_stats stats{};
     float count_ms = 0.f;
 };
 
 static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int force_segments);
+static int count_grid_wide(CountCall &cc, std::vector<int32_t> &work, int variant);
+
+// Automatic grid-wide local tracking (fem_plt.cu): at most this many episodes
+// over a recording of at least this many events (see run_count).
+constexpr int64_t kPltMaxCands = 256;
+constexpr int64_t kPltMinEvents = 1 << 20;
 
 // Builds the per-recording RecInfo table and the density table.
 static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int force_segments) {
@@ -1822,6 +1830,17 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
         while (track_nblocks > 1 && track_buf_bytes(track_nblocks, track_cap) > free_b / 4)
             track_nblocks = track_nblocks > ctx->n_sm ? track_nblocks - ctx->n_sm : track_nblocks / 2;
         if (track_buf_bytes(track_nblocks, track_cap) > free_b / 4) track = false;
+    }
+    // few episodes over a long recording, and no room for the warp-per-item
+    // kernel: grid-wide local tracking needs no more than the lists
+    if (!track && cc.plt_ok && force_segments == 0) {
+        std::vector<int32_t> work(n_work);
+        std::iota(work.begin(), work.end(), 0);
+        if (subset) {
+            FEM_CUDA_TRY(cudaMemcpyAsync(work.data(), subset, 4 * n_work, cudaMemcpyDeviceToHost, ctx->stream));
+            FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        }
+        return count_grid_wide(cc, work, 0);
     }
     const int n_keys = kBuckets * n_recs;
     // --- density tables and per-recording tables
@@ -2491,6 +2510,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
         std::vector<int32_t> hsub(fbc);
         FEM_CUDA_TRY(cudaMemcpyAsync(hsub.data(), p_sub, sizeof(int32_t) * fbc, cudaMemcpyDeviceToHost, ctx->stream));
         FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if (cc.plt_ok) return count_grid_wide(cc, hsub, 0);
         void *p_keep = nullptr;
         FEM_TRY(dev_alloc(ctx, &p_keep, sizeof(int32_t) * fbc));
         cudaMemcpyAsync(p_keep, hsub.data(), sizeof(int32_t) * fbc, cudaMemcpyHostToDevice, ctx->stream);
@@ -2515,25 +2535,58 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     return FEM_OK;
 }
 
-constexpr int64_t kPltMaxCands = 256;        // automatic local tracking: at most this many episodes
-constexpr int64_t kPltMinEvents = 1 << 20;   // ... over a recording of at least this many events
+// Counts the candidates `work` by grid-wide local tracking (fem_plt.cu).
+static int count_grid_wide(CountCall &cc, std::vector<int32_t> &work, int variant) {
+    FEM_TRY(count_plt(cc.ctx, cc.recs, cc.offs, cc.types, cc.lo, cc.hi, cc.cand_rec, work, cc.mode == 2, cc.counts,
+                      &cc.stats, &cc.count_ms, variant));
+    return sync_status(cc.ctx);
+}
+
+// Few episodes over a long recording: grid-wide local tracking (parallel over
+// the events of an episode's node types, about 70 dependent launches) or the
+// warp-per-item kernel with the recording cut into segments (three launches).
+// Measured on recordings of 1.1M to 11M events (64 types at 20 Hz), 4-8 nodes:
+// edges of up to 20 ms: 1 episode 320 / 200 us, 16 episodes 1050-1500 /
+// 190-250 us, 256 episodes 1.9-10.3 / 0.28-0.85 ms (grid-wide / segments).
+// Segments stop paying in two cases, which the spans of the episodes tell:
+//   * too few of them (a segment is at least 8 halos long): one warp then
+//     walks 1/P of every list, and needs P >= 32 to stay ahead (11M events,
+//     16 episodes: P = 8 2.3 ms, 16 1.2 ms, 32 0.7 ms against 1.5 ms);
+//   * many events of a type inside one span: occurrences that straddle a
+//     boundary need an entry class each, and an episode with more than
+//     kClasses of them is counted again (up to 14 events of a type in the
+//     longest span no episode overflowed; at 28, 12-25 of 256 did, and cutting
+//     less finely then costs more than counting grid-wide at once: 16
+//     episodes, 11M events 12.4 against 1.6 ms).
+// An episode that overflows all the same is recounted grid-wide.
+constexpr double kFewMinSegments = 32.0;
+constexpr double kFewMaxPerSpan = 16.0;  // mean events of one type in the longest span
+
+static bool few_by_segments(const CountCall &cc) {
+    if (cc.sumhi < 0) return false;
+    for (auto *r : cc.recs) {
+        if (r->n < kPltMinEvents) continue;
+        const double span = std::max(1.0, (double)r->t_last - (double)r->t_first);
+        const double in_span = (double)r->n * (double)cc.sumhi / span;
+        if ((double)r->n / std::max((double)kTrackMinSeg, 8.0 * in_span) < kFewMinSegments) return false;
+        if (in_span / (double)r->n_types > kFewMaxPerSpan) return false;
+    }
+    return true;
+}
 
 static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int force_segments) {
-    // node-by-node local tracking (fem_plt.cu): when asked for, or for few
-    // episodes over long recordings (its steps are parallel over the events
-    // of the episodes' node types; the per-episode kernels need many
-    // episodes, or many segments with their halos and records, to fill the
-    // GPU)
     const int kern = cc.ctx->tuning.kernel;
-    bool plt = kern >= 4;
-    if (cc.ctx->tuning.kernel == 0 && n_sub <= kPltMaxCands) {
+    bool plt = kern >= 4 && kern <= 6;
+    cc.plt_ok = false;
+    if (kern == 0 && n_sub <= kPltMaxCands && cc.mode != 1 && force_segments == 0) {
         int64_t nmax = 0;
         bool lists = true;
         for (auto *r : cc.recs) {
             nmax = std::max(nmax, r->n);
             lists = lists && r->n_types <= 8192 && r->n <= INT32_MAX / 2;
         }
-        plt = lists && nmax >= kPltMinEvents;
+        cc.plt_ok = lists && nmax >= kPltMinEvents;
+        plt = cc.plt_ok && !few_by_segments(cc);
     }
     if (cc.mode != 1 && force_segments == 0 && plt) {
         std::vector<int32_t> work(n_sub);
@@ -2543,9 +2596,7 @@ static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int fo
         } else {
             for (int64_t i = 0; i < n_sub; ++i) work[i] = (int32_t)i;
         }
-        FEM_TRY(count_plt(cc.ctx, cc.recs, cc.offs, cc.types, cc.lo, cc.hi, cc.cand_rec, work, cc.mode == 2,
-                          cc.counts, &cc.stats, &cc.count_ms, kern >= 5 ? kern - 4 : 0));
-        return sync_status(cc.ctx);
+        return count_grid_wide(cc, work, kern >= 5 ? kern - 4 : 0);
     }
     return count_core(cc, subset, n_sub, force_segments);
 }
@@ -2556,9 +2607,16 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
                             int n_recs) {
     const int64_t n = c->n_cand;
     int64_t n_nodes = 0;
+    const bool few = n <= kPltMaxCands;  // their spans choose the path (few_by_segments)
+    std::vector<int64_t> offs_h(few ? n + 1 : 0);
+    std::vector<int32_t> hi_h;
     if (c->ptr_is_device) {
-        FEM_CUDA_TRY(cudaMemcpyAsync(&n_nodes, c->offs + n, 8, cudaMemcpyDeviceToHost, ctx->stream));
+        if (few)
+            FEM_CUDA_TRY(cudaMemcpyAsync(offs_h.data(), c->offs, 8 * (n + 1), cudaMemcpyDeviceToHost, ctx->stream));
+        else
+            FEM_CUDA_TRY(cudaMemcpyAsync(&n_nodes, c->offs + n, 8, cudaMemcpyDeviceToHost, ctx->stream));
         FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if (few) n_nodes = offs_h[n];
     } else {
         if (c->offs[0] != 0) return FEM_ERR_INVAL;
         for (int64_t i = 0; i < n; ++i)
@@ -2576,6 +2634,10 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
         lo_h.resize(n_edges);
         if (n_edges > 0) {
             FEM_CUDA_TRY(cudaMemcpyAsync(lo_h.data(), c->lo, 4 * n_edges, cudaMemcpyDeviceToHost, ctx->stream));
+            if (few) {
+                hi_h.resize(n_edges);
+                FEM_CUDA_TRY(cudaMemcpyAsync(hi_h.data(), c->hi, 4 * n_edges, cudaMemcpyDeviceToHost, ctx->stream));
+            }
             FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
         }
         if (rec_id) cc.cand_rec = rec_id;
@@ -2605,6 +2667,17 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
     }
     std::set<int32_t> los(lo_h.begin(), lo_h.end());
     cc.lo_vals.assign(los.begin(), los.end());
+    if (few) {
+        const int64_t *o = c->ptr_is_device ? offs_h.data() : c->offs;
+        const int32_t *h = c->ptr_is_device ? hi_h.data() : c->hi;
+        bool sound = o[0] == 0;  // device offsets are checked later, on the path taken
+        for (int64_t i = 0; i < n && sound; ++i) sound = o[i + 1] > o[i] && o[i + 1] <= n_nodes;
+        for (int64_t i = 0; i < n && sound; ++i) {
+            int64_t sum = 0;
+            for (int64_t e = o[i] - i; e < o[i + 1] - i - 1; ++e) sum += h[e];
+            cc.sumhi = std::max(cc.sumhi, sum);
+        }
+    }
     return FEM_OK;
 }
 
@@ -2643,11 +2716,12 @@ static int count_entry(fem_ctx *ctx, const fem_stream *const *recs, int n_recs, 
     return FEM_OK;
 }
 
-// Counting of device-resident candidates (used by the level-wise miner).
+// Counting of device-resident candidates (used by the level-wise miner); no
+// episode's upper bounds add up to more than sumhi.
 int count_device(fem_ctx *ctx, const std::vector<fem_stream *> &recs, int64_t n_cand, const int64_t *offs,
                  const uint16_t *types, const int32_t *lo, const int32_t *hi, const uint32_t *cand_rec,
-                 const std::vector<int32_t> &lo_vals, const int32_t *order, int64_t n_order, uint32_t *counts,
-                 fem_stats *stats) {
+                 const std::vector<int32_t> &lo_vals, int64_t sumhi, const int32_t *order, int64_t n_order,
+                 uint32_t *counts, fem_stats *stats) {
     CountCall cc;
     cc.ctx = ctx;
     cc.recs = recs;
@@ -2660,6 +2734,7 @@ int count_device(fem_ctx *ctx, const std::vector<fem_stream *> &recs, int64_t n_
     cc.cand_rec = cand_rec;
     cc.counts = counts;
     cc.lo_vals = lo_vals;
+    cc.sumhi = sumhi;
     // `order` (optional) lists every candidate once, in the order the
     // counting kernels should hold them (lane neighbours share types).
     const int64_t n_work = order ? n_order : n_cand;

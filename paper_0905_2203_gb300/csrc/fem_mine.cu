@@ -318,8 +318,8 @@ __global__ void k_rec_offsets(const uint32_t *rec, int64_t n, int n_recs, int64_
 // Counting entry shared with fem_count.cu (mode 0, device candidate arrays).
 int count_device(fem_ctx *ctx, const std::vector<fem_stream *> &recs, int64_t n_cand, const int64_t *offs,
                  const uint16_t *types, const int32_t *lo, const int32_t *hi, const uint32_t *cand_rec,
-                 const std::vector<int32_t> &lo_vals, const int32_t *order, int64_t n_order, uint32_t *counts,
-                 fem_stats *stats);
+                 const std::vector<int32_t> &lo_vals, int64_t sumhi, const int32_t *order, int64_t n_order,
+                 uint32_t *counts, fem_stats *stats);
 
 namespace {
 
@@ -425,6 +425,12 @@ struct MineGroup {
     std::vector<int64_t> c_off;         // host copy of d_coff_rec
 
     int nrec() const { return (int)recs.size(); }
+    // no candidate's upper bounds add up to more than this
+    int64_t span_max() const {
+        int32_t h = 0;
+        for (int32_t b : bhi) h = std::max(h, b);
+        return (int64_t)h * std::max(cand.N - 1, 0);
+    }
 
     int begin();
     int advance();
@@ -847,7 +853,7 @@ int MineGroup::graph_tail() {
 static int count_group(MineGroup &g) {
     fem_stats cs{};
     FEM_TRY(count_device(g.ctx, g.recs, g.cand.n, g.d_coffs, g.cand.types, g.cand.lo, g.cand.hi, g.cand.rec, g.lo_vals,
-                         g.d_order, g.n_order, g.cand.counts, &cs));
+                         g.span_max(), g.d_order, g.n_order, g.cand.counts, &cs));
     g.S.kernel_launches += cs.kernel_launches;
     g.S.sparse_launches += cs.sparse_launches;
     g.S.candidates_counted += cs.candidates_counted;
@@ -879,9 +885,10 @@ int mg_count_batch(fem_ctx *ctx, const std::vector<MineGroup *> &gs) {
     cudaStream_t st = ctx->stream;
     std::vector<fem_stream *> recs;
     std::vector<int32_t> lo_vals;
-    int64_t C = 0, nodes = 0, edges = 0, norder = 0;
+    int64_t C = 0, nodes = 0, edges = 0, norder = 0, sumhi = 0;
     for (MineGroup *g : gs) {
         if (g->done || g->cand.n == 0) continue;
+        sumhi = std::max(sumhi, g->span_max());
         recs.insert(recs.end(), g->recs.begin(), g->recs.end());
         lo_vals.insert(lo_vals.end(), g->lo_vals.begin(), g->lo_vals.end());
         C += g->cand.n;
@@ -931,7 +938,7 @@ int mg_count_batch(fem_ctx *ctx, const std::vector<MineGroup *> &gs) {
     k_set_last_offs<<<1, 1, 0, st>>>(offs, C, nodes);
     FEM_CUDA_TRY(cudaGetLastError());
     fem_stats cs{};
-    FEM_TRY(count_device(ctx, recs, C, offs, types, lo, hi, rec, lo_vals, order, norder, counts, &cs));
+    FEM_TRY(count_device(ctx, recs, C, offs, types, lo, hi, rec, lo_vals, sumhi, order, norder, counts, &cs));
     cb = 0;
     for (MineGroup *g : gs) {
         if (g->done || g->cand.n == 0) continue;
