@@ -1530,58 +1530,80 @@ __global__ void k_toff(const int32_t *__restrict__ keyoff, int n_types, int64_t 
     if (a == n_types) toff[a] = n;
 }
 
-// Temporary device allocations freed together (after the stream drains).
-int stream_bytype(fem_ctx *ctx, fem_stream *s) {
-    if (s->d_ttime) return FEM_OK;
+// The lists and (with pos) their stream positions: what is there already is
+// kept.  The positions are the partition's permutation; without pos it is
+// released with the other temporaries.
+int stream_bytype(fem_ctx *ctx, fem_stream *s, bool pos) {
+    if (s->d_ttime && (!pos || s->d_tpos)) return FEM_OK;
     if (s->n_types > 8192 || s->n > INT32_MAX / 2) return FEM_ERR_INVAL;
     const int64_t n = s->n;
-    void *p1 = nullptr, *p2 = nullptr;
-    FEM_TRY(dev_alloc(ctx, &p1, sizeof(int64_t) * (s->n_types + 1)));
-    const int st2 = dev_alloc(ctx, &p2, sizeof(int32_t) * std::max<int64_t>(n, 1));
-    if (st2 != FEM_OK) {
-        dev_free(ctx, p1, sizeof(int64_t) * (s->n_types + 1));
-        return st2;
-    }
+    const bool lists = !s->d_ttime;
+    const size_t toff_b = sizeof(int64_t) * (s->n_types + 1), list_b = sizeof(int32_t) * std::max<int64_t>(n, 1);
+    void *p1 = nullptr, *p2 = nullptr, *p3 = nullptr;
+    auto drop = [&](int code) {
+        dev_free(ctx, p1, toff_b);
+        dev_free(ctx, p2, list_b);
+        dev_free(ctx, p3, list_b);
+        return code;
+    };
+    int st = FEM_OK;
+    if (lists) st = dev_alloc(ctx, &p1, toff_b);
+    if (st == FEM_OK && lists) st = dev_alloc(ctx, &p2, list_b);
+    if (st == FEM_OK && pos) st = dev_alloc(ctx, &p3, list_b);
+    if (st != FEM_OK) return drop(st);
     int64_t *toff = static_cast<int64_t *>(p1);
     int32_t *ttime = static_cast<int32_t *>(p2);
     const int n_keys = (int)s->n_types;
     const int64_t nblk = std::max<int64_t>(1, (n + kPartBlock - 1) / kPartBlock);
     const int64_t tab_n = (int64_t)n_keys * nblk;
     TmpDev tmp(ctx);
-    int32_t *key, *perm, *blk, *stmp, *koff;
-    int st = tmp.get(&key, std::max<int64_t>(n, 1));
-    if (st == FEM_OK) st = tmp.get(&perm, std::max<int64_t>(n, 1));
+    int32_t *key, *perm = static_cast<int32_t *>(p3), *blk, *stmp, *koff;
+    st = tmp.get(&key, std::max<int64_t>(n, 1));
+    if (st == FEM_OK && !pos) st = tmp.get(&perm, std::max<int64_t>(n, 1));
     if (st == FEM_OK) st = tmp.get(&blk, tab_n);
     if (st == FEM_OK) st = tmp.get(&stmp, tab_n / kScanBlock + 2);
     if (st == FEM_OK) st = tmp.get(&koff, n_keys + 1);
-    if (st != FEM_OK) {
-        dev_free(ctx, p1, sizeof(int64_t) * (s->n_types + 1));
-        dev_free(ctx, p2, sizeof(int32_t) * std::max<int64_t>(n, 1));
-        return st;
-    }
+    if (st != FEM_OK) return drop(st);
     cudaStream_t cs = ctx->stream;
-    if (n > 0) {
-        const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 8 * ctx->n_sm);
-        k_widen_types<<<g, 256, 0, cs>>>(s->d_type, n, key);
-        k_part_count<<<(unsigned)nblk, 256, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk);
-        FEM_TRY(scan_exclusive(cs, blk, tab_n, stmp, nullptr, nullptr));
-        k_part_scatter<<<(unsigned)nblk, 32, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk, nullptr, perm, nullptr);
-        k_gather_keyoff<<<(n_keys + 255) / 256, 256, 0, cs>>>(blk, n_keys, nblk, koff);
-        k_gather_ttime<<<g, 256, 0, cs>>>(perm, s->d_time, n, ttime);
-        k_toff<<<(n_keys + 1 + 255) / 256, 256, 0, cs>>>(koff, n_keys, n, toff);
-    } else {
-        FEM_CUDA_TRY(cudaMemsetAsync(toff, 0, sizeof(int64_t) * (s->n_types + 1), cs));
+    auto build = [&]() -> int {
+        if (n > 0) {
+            const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 8 * ctx->n_sm);
+            k_widen_types<<<g, 256, 0, cs>>>(s->d_type, n, key);
+            k_part_count<<<(unsigned)nblk, 256, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk);
+            FEM_TRY(scan_exclusive(cs, blk, tab_n, stmp, nullptr, nullptr));
+            k_part_scatter<<<(unsigned)nblk, 32, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk, nullptr, perm, nullptr);
+            if (lists) {
+                k_gather_keyoff<<<(n_keys + 255) / 256, 256, 0, cs>>>(blk, n_keys, nblk, koff);
+                k_gather_ttime<<<g, 256, 0, cs>>>(perm, s->d_time, n, ttime);
+                k_toff<<<(n_keys + 1 + 255) / 256, 256, 0, cs>>>(koff, n_keys, n, toff);
+            }
+        } else if (lists) {
+            FEM_CUDA_TRY(cudaMemsetAsync(toff, 0, toff_b, cs));
+        }
+        FEM_CUDA_TRY(cudaGetLastError());
+        if (!lists) return FEM_OK;
+        // longest per-type list (sizes the per-warp buffers of local tracking)
+        std::vector<int64_t> toff_h(s->n_types + 1, 0);
+        FEM_CUDA_TRY(cudaMemcpyAsync(toff_h.data(), toff, toff_b, cudaMemcpyDeviceToHost, cs));
+        FEM_CUDA_TRY(cudaStreamSynchronize(cs));
+        s->max_list = 0;
+        for (uint32_t a = 0; a < s->n_types; ++a) s->max_list = std::max(s->max_list, toff_h[a + 1] - toff_h[a]);
+        return FEM_OK;
+    };
+    st = build();
+    if (st != FEM_OK) {
+        cudaStreamSynchronize(cs);
+        return drop(st);
     }
-    FEM_CUDA_TRY(cudaGetLastError());
-    // longest per-type list (sizes the per-warp buffers of local tracking)
-    std::vector<int64_t> toff_h(s->n_types + 1, 0);
-    FEM_CUDA_TRY(cudaMemcpyAsync(toff_h.data(), toff, sizeof(int64_t) * (s->n_types + 1), cudaMemcpyDeviceToHost, cs));
-    FEM_CUDA_TRY(cudaStreamSynchronize(cs));
-    s->max_list = 0;
-    for (uint32_t a = 0; a < s->n_types; ++a) s->max_list = std::max(s->max_list, toff_h[a + 1] - toff_h[a]);
-    s->d_toff = toff;
-    s->d_ttime = ttime;
-    s->bytes += sizeof(int64_t) * (s->n_types + 1) + sizeof(int32_t) * n;
+    if (lists) {
+        s->d_toff = toff;
+        s->d_ttime = ttime;
+        s->bytes += toff_b + sizeof(int32_t) * n;
+    }
+    if (pos) {
+        s->d_tpos = perm;
+        s->bytes += sizeof(int32_t) * n;
+    }
     return FEM_OK;
 }
 

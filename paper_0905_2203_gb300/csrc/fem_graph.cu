@@ -147,103 +147,6 @@ __global__ void k_g_gen2(const uint16_t *ft1, const int64_t *foff1, const int64_
     }
 }
 
-// Upper-bound pre-pass over all recordings (anti-monotonicity, "Temporal Data
-// Mining"): the non-overlapped occurrences of a -(lo,hi]-> b end at distinct
-// b-events, each with an a-event inside its window, so
-//     count(a, b, bin) <= UB = #{ b-events with an a-event in the window }.
-// A block takes a tile of kUbTile consecutive events of one recording and
-// stages the tile plus the events up to hi_max before it (at most kUbHalo) in
-// shared memory; one thread per event scans back over its window there (in
-// global memory beyond the staged halo), marks each (type, bin) once in its
-// bitset and adds one to UB for it.  The bins a time difference d falls in
-// come from a table of bin masks indexed by d (when hi_max < kUbLut), else
-// from a loop over the bins.  Word w of thread t's bitset sits at
-// bits[w * blockDim + t], so the lanes of a warp touch distinct banks.
-constexpr int kUbMaxBins = 8;
-constexpr int kUbLut = 65536;
-constexpr int kUbTile = 1024;
-constexpr int kUbHalo = 1024;
-
-__global__ void k_g_pair_ub(const RecInfo *ri, const int64_t *tpre, int n_recs, const uint32_t *nt,
-                            const int64_t *ub_off, const int32_t *blo, const int32_t *bhi, int nb, int32_t hi_max,
-                            int words, const uint8_t *lut_g, uint32_t *ub) {
-    extern __shared__ uint32_t sm[];
-    const int bd = blockDim.x;
-    const int lut_words = lut_g ? (hi_max + 4) / 4 : 0;
-    uint8_t *lut = reinterpret_cast<uint8_t *>(sm);
-    int32_t *s_tm = reinterpret_cast<int32_t *>(sm + lut_words);
-    uint16_t *s_ty = reinterpret_cast<uint16_t *>(s_tm + kUbTile + kUbHalo);
-    uint32_t *my = sm + lut_words + (kUbTile + kUbHalo) + (kUbTile + kUbHalo) / 2 + threadIdx.x;
-    __shared__ int64_t s_h0;
-    if (lut_g) {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(lut_g);
-        for (int w = threadIdx.x; w < lut_words; w += bd) sm[w] = src[w];
-    }
-    const int64_t tiles = tpre[n_recs];
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int r = seg_of(tpre, n_recs, tile);
-        const int64_t j0 = (tile - tpre[r]) * kUbTile;
-        const int64_t n = ri[r].n;
-        const int64_t j1 = min(n, j0 + kUbTile);
-        const uint16_t *ty = ri[r].type;
-        const int32_t *tm = ri[r].time;
-        const uint32_t ntr = nt[r];
-        const int wr = (int)((ntr * (uint32_t)nb + 31) / 32);
-        uint32_t *u = ub + ub_off[r];
-        if (threadIdx.x == 0) {
-            // first event within hi_max of the tile's first event (capped)
-            const int64_t lim = (int64_t)tm[j0] - hi_max;
-            int64_t lo = max((int64_t)0, j0 - kUbHalo), hi = j0;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if ((int64_t)tm[mid] < lim) lo = mid + 1; else hi = mid;
-            }
-            s_h0 = lo;
-        }
-        __syncthreads();
-        const int64_t h0 = s_h0;
-        for (int64_t i = h0 + threadIdx.x; i < j1; i += bd) {
-            s_tm[i - h0] = tm[i];
-            s_ty[i - h0] = ty[i];
-        }
-        __syncthreads();
-        for (int64_t j = j0 + threadIdx.x; j < j1; j += bd) {
-            for (int w = 0; w < wr; ++w) my[w * bd] = 0;
-            const int32_t t = s_tm[j - h0];
-            const uint32_t b = s_ty[j - h0];
-            const int64_t lim = (int64_t)t - hi_max;
-            for (int64_t i = j - 1; i >= 0; --i) {
-                const bool st = i >= h0;
-                const int32_t ti = st ? s_tm[i - h0] : tm[i];
-                if ((int64_t)ti < lim) break;
-                const int32_t d = t - ti;
-                if (d <= 0) continue;
-                const uint32_t a = st ? s_ty[i - h0] : ty[i];
-                if (a == b) continue;
-                uint32_t mask = 0;
-                if (lut_g) {
-                    mask = lut[d];
-                } else {
-                    for (int k = 0; k < nb; ++k)
-                        if (blo[k] < d && d <= bhi[k]) mask |= 1u << k;
-                }
-                while (mask) {
-                    const int k = __ffs(mask) - 1;
-                    mask &= mask - 1;
-                    const uint32_t bit = a * (uint32_t)nb + (uint32_t)k;
-                    const uint32_t m = 1u << (bit & 31);
-                    uint32_t &wd = my[(bit >> 5) * bd];
-                    if (!(wd & m)) {
-                        wd |= m;
-                        atomicAdd(&u[((size_t)a * ntr + b) * nb + k], 1u);
-                    }
-                }
-            }
-        }
-        __syncthreads();  // the staged events are replaced by the next tile's
-    }
-}
-
 __device__ __forceinline__ bool g_keep2(int64_t c, const uint16_t *gt, const int32_t *glo, const int32_t *ghi,
                                         const uint32_t *grec, const uint32_t *ub, const int64_t *ub_off,
                                         const uint32_t *nt, const int32_t *blo, const int32_t *bhi, int nb,
@@ -836,7 +739,8 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     std::vector<const uint32_t *> dens_h(need_dens ? (size_t)n_recs * lo_vals.size() : 0);
     for (int r = 0; r < n_recs; ++r) {
         fem_stream *s = g->recs[r];
-        FEM_TRY(!need_dens ? stream_tindex(ctx, s) : stream_bytype(ctx, s));
+        FEM_TRY(stream_bytype(ctx, s, g->prepass && first <= 2));  // the pair bound reads list positions
+        if (!need_dens) FEM_TRY(stream_tindex(ctx, s));
         if (need_dens) {
             FEM_TRY(stream_densities(ctx, s, lo_vals));
             for (size_t j = 0; j < lo_vals.size(); ++j) {
@@ -927,23 +831,11 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     // segment): room for four segments per candidate where the budget has it
     if (g->track && (size_t)(g->target + 4 * cap) * kRecWords * 4 <= free_b / 4) g->cap_threads = g->target + 4 * cap;
     if ((size_t)g->cap_threads * kRecWords * 4 > free_b / 4) return FEM_ERR_NOMEM;
-    // pre-pass launch shape: the bin-mask table (when hi_max < kUbLut), the
-    // staged events and a per-thread bitset of n_types x bins bits
-    const int ub_words = (int)((nt_max * (uint32_t)std::max(nb, 1) + 31) / 32);
-    const bool ub_lut = hi_max < kUbLut;
-    const size_t ub_lut_bytes = ub_lut ? (size_t)((hi_max + 4) / 4) * 4 : 0;
-    const size_t ub_stage = (size_t)(kUbTile + kUbHalo) * 4 + (size_t)(kUbTile + kUbHalo) / 2 * 4;
-    const int64_t ub_room = (int64_t)ctx->smem_optin - 1024 - (int64_t)ub_lut_bytes - (int64_t)ub_stage;
-    const int ub_threads =
-        ub_room > 0 ? (int)std::min<int64_t>(256, ub_room / (4 * (int64_t)ub_words) / 32 * 32) : 0;
-    const size_t ub_smem = ub_lut_bytes + ub_stage + (size_t)std::max(ub_threads, 0) * ub_words * 4;
-    if (ub_threads < 32 || nb > kUbMaxBins) g->prepass = false;
-    std::vector<int64_t> tpre(n_recs + 1, 0);
-    for (int r = 0; r < n_recs; ++r) tpre[r + 1] = tpre[r] + (g->recs[r]->n + kUbTile - 1) / kUbTile;
-    std::vector<uint8_t> lut_h(ub_lut ? (size_t)((hi_max + 4) / 4) * 4 : 0, 0);
-    for (int32_t d = 0; ub_lut && d <= hi_max; ++d)
-        for (int k = 0; k < nb; ++k)
-            if (blo[k] < d && d <= bhi[k]) lut_h[d] |= (uint8_t)(1u << k);
+    // pair bound: items of `ub_chunk` list positions per recording
+    if (nb > kPairBoundMaxBins || nt_max > kPairBoundMaxTypes) g->prepass = false;
+    const int ub_chunk = pair_bound_chunk(ctx->n_sm, evpre[n_recs]);
+    std::vector<int64_t> cpre(n_recs + 1, 0);
+    for (int r = 0; r < n_recs; ++r) cpre[r + 1] = cpre[r] + (g->recs[r]->n + ub_chunk - 1) / ub_chunk;
 
     RecInfo *d_ri;
     const uint32_t **d_dens;
@@ -1008,8 +900,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
         FEM_TRY(g->get(&f.foff, n_recs + 1));
     }
     // level-1 / level-2 inputs
-    int64_t *d_ntpre = nullptr, *d_evpre = nullptr, *d_uboff = nullptr, *d_tpre = nullptr;
-    uint8_t *d_lut = nullptr;
+    int64_t *d_ntpre = nullptr, *d_evpre = nullptr, *d_uboff = nullptr, *d_cpre = nullptr;
     uint32_t *d_nt = nullptr, *ub = nullptr;
     uint16_t *gt = nullptr;
     int32_t *glo = nullptr, *ghi = nullptr;
@@ -1019,8 +910,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
         FEM_TRY(g->get(&d_evpre, n_recs + 1));
         FEM_TRY(g->get(&d_uboff, n_recs + 1));
         FEM_TRY(g->get(&d_nt, n_recs));
-        FEM_TRY(g->get(&d_tpre, n_recs + 1));
-        if (ub_lut) FEM_TRY(g->get(&d_lut, lut_h.size()));
+        FEM_TRY(g->get(&d_cpre, n_recs + 1));
         FEM_TRY(g->get(&gt, (size_t)2 * std::max<int64_t>(cap2, 1)));
         FEM_TRY(g->get(&glo, std::max<int64_t>(cap2, 1)));
         FEM_TRY(g->get(&ghi, std::max<int64_t>(cap2, 1)));
@@ -1030,8 +920,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
         FEM_CUDA_TRY(cudaMemcpyAsync(d_evpre, evpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
         FEM_CUDA_TRY(cudaMemcpyAsync(d_uboff, ub_off.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
         FEM_CUDA_TRY(cudaMemcpyAsync(d_nt, nt_h.data(), 4 * n_recs, cudaMemcpyHostToDevice, st));
-        FEM_CUDA_TRY(cudaMemcpyAsync(d_tpre, tpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
-        if (ub_lut) FEM_CUDA_TRY(cudaMemcpyAsync(d_lut, lut_h.data(), lut_h.size(), cudaMemcpyHostToDevice, st));
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_cpre, cpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
     }
     FEM_CUDA_TRY(cudaMemcpyAsync(d_ri, ri_h.data(), sizeof(RecInfo) * n_recs, cudaMemcpyHostToDevice, st));
     FEM_CUDA_TRY(cudaMemcpyAsync(d_dens, dens_h.data(), sizeof(void *) * dens_h.size(), cudaMemcpyHostToDevice, st));
@@ -1133,14 +1022,6 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     const unsigned gb = (unsigned)std::min<int64_t>((cap + 256) / 256, 4 * ctx->n_sm);
     const unsigned gb2 = (unsigned)std::max<int64_t>(1, std::min<int64_t>((cap2 + 256) / 256, 8 * ctx->n_sm));
     const unsigned gb1 = (unsigned)std::max<int64_t>(1, std::min<int64_t>((tot1 + 256) / 256, 4 * ctx->n_sm));
-    const unsigned gbe = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tpre[n_recs], 8 * ctx->n_sm));
-    if (g->prepass && ub_smem > 48 * 1024) {
-        if (cudaFuncSetAttribute((const void *)k_g_pair_ub, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ub_smem) != cudaSuccess) {
-            cudaGetLastError();
-            g->prepass = false;
-        }
-    }
     cudaGraph_t graph = nullptr;
     FEM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     int cst = FEM_OK;
@@ -1200,8 +1081,11 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
                                           grec);
             if (g->prepass) {
                 ok(cudaMemsetAsync(ub, 0, sizeof(uint32_t) * std::max<int64_t>(ub_off[n_recs], 1), st));
-                k_g_pair_ub<<<gbe, ub_threads, ub_smem, st>>>(d_ri, d_tpre, n_recs, d_nt, d_uboff, d_blo, d_bhi, nb,
-                                                              hi_max, ub_words, d_lut, ub);
+                const PairBoundArgs pb{d_ri, n_recs, d_cpre, cpre[n_recs], ub_chunk, d_nt, g->d_thr,
+                                       d_uboff, d_blo, d_bhi, nb, hi_max, ub, 0, 0};
+                if (cst == FEM_OK)
+                    cst = pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, mean_window(g->recs, hi_max),
+                                     last_time(g->recs));
             }
             const uint32_t *ubp = g->prepass ? ub : nullptr;
             k_g_prune_flags<<<gb2, 256, 0, st>>>(gt, glo, ghi, grec, cn, cap2, ubp, d_uboff, d_nt, d_blo, d_bhi, nb,

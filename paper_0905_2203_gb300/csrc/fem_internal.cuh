@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <unordered_map>
@@ -71,6 +72,7 @@ struct RecInfo {
     int tshift;
     int32_t tbase;
     int64_t tcells;
+    const int32_t *tpos;  // stream position of every list entry (null where not built)
 };
 
 // Node-by-node local tracking with one warp per (episode, segment) work item
@@ -221,6 +223,7 @@ struct fem_stream {
     int32_t t_first = 0, t_last = 0;  // first and last event time (n > 0)
     int64_t *d_toff = nullptr;    // per-type event lists (built on first use): offsets [n_types + 1]
     int32_t *d_ttime = nullptr;   // times grouped by type, ascending within a type [n]
+    int32_t *d_tpos = nullptr;    // stream position of every list entry [n] (built on request)
     int64_t max_list = 0;         // longest per-type list (set with the lists)
     // Per-type time index (built on first use, after the lists): cells of
     // 2^tshift ticks from t_first; d_tidx[a * (tcells + 1) + c] is the
@@ -263,8 +266,9 @@ int copy_in(fem_ctx *ctx, void *dst_dev, const void *src, size_t bytes, int src_
 int copy_out(fem_ctx *ctx, void *dst, const void *src_dev, size_t bytes, int dst_is_device);
 // Segment boundaries of a stream cut into P segments (cached per P).
 int stream_segments(fem_ctx *ctx, fem_stream *s, int P, const int64_t **seg);
-// Per-type event lists of a stream (built on first use, kept in the stream).
-int stream_bytype(fem_ctx *ctx, fem_stream *s);
+// Per-type event lists of a stream (built on first use, kept in the stream);
+// with `pos` also the stream position of every list entry.
+int stream_bytype(fem_ctx *ctx, fem_stream *s, bool pos = false);
 // Per-type time index of a stream (after its lists; built on first use).
 int stream_tindex(fem_ctx *ctx, fem_stream *s);
 // The stream's per-type lists and time index in a RecInfo.
@@ -275,6 +279,7 @@ inline void recinfo_lists(RecInfo &ri, const fem_stream *s) {
     ri.tshift = s->tshift;
     ri.tbase = s->t_first;
     ri.tcells = s->tcells;
+    ri.tpos = s->d_tpos;
 }
 // Density table for one lo (computed on first use, cached in the stream).
 int stream_density(fem_ctx *ctx, fem_stream *s, int32_t lo, uint32_t **d_dens);
@@ -391,6 +396,46 @@ struct JoinBoundArgs {
     unsigned long long *skipc;  // per recording: skipped candidates
 };
 int join_bound_level3(cudaStream_t st, int n_sm, const JoinBoundArgs &a);
+
+// Level-2 upper bounds of all pairs of types (fem_pairbound.cu): ub[ub_off[r]
+// + (a * nt[r] + b) * nb + k] += for every frequent type a of recording r, the
+// b-events with an a-event inside bin k (entries a = b hold no bound).
+struct PairBoundArgs {
+    const RecInfo *ri;      // per recording: stream, lists and list positions
+    int n_recs;
+    const int64_t *cpre;    // per recording: first item (n_recs + 1)
+    int64_t n_items;        // chunks of `chunk` list positions
+    int chunk;
+    const uint32_t *nt;     // types per recording (at most 1024)
+    const uint32_t *thr;    // threshold per recording
+    const int64_t *ub_off;
+    const int32_t *blo, *bhi;
+    int nb;                 // bins (at most 8)
+    int32_t hi_max;
+    uint32_t *ub;           // zeroed by the caller
+    uint32_t width, magic;  // set by pair_bound (adjacent bins of one width)
+};
+constexpr int kPairBoundMaxBins = 8;
+constexpr uint32_t kPairBoundMaxTypes = 1024;
+int pair_bound_chunk(int n_sm, int64_t events);
+int pair_bound(cudaStream_t st, int n_sm, PairBoundArgs a, const std::vector<int32_t> &blo,
+               const std::vector<int32_t> &bhi, uint32_t nt_max, double window, int64_t t_last);
+inline int64_t last_time(const std::vector<fem_stream *> &recs) {
+    int64_t t = 0;
+    for (const fem_stream *s : recs) t = std::max<int64_t>(t, s->t_last);
+    return t;
+}
+// Events within `hi` ticks after an event, on average over the recordings'
+// events.
+inline double mean_window(const std::vector<fem_stream *> &recs, int64_t hi) {
+    double w = 0, n = 0;
+    for (const fem_stream *s : recs) {
+        const double span = std::max(1.0, (double)s->t_last - (double)s->t_first);
+        w += (double)s->n * ((double)s->n * (double)hi / span);
+        n += (double)s->n;
+    }
+    return n > 0 ? w / n : 0.0;
+}
 
 // Prefix groups of the slots (flags, scan, first slot of each group, and,
 // if in.gmax is set, each recording's largest group) without the item

@@ -148,7 +148,8 @@ __global__ void k_perm2_write(const int32_t *pos, const int64_t *f_off, const in
 // b-events, each with an a-event inside (t - hi, ... t - lo] before it, so
 //     count(a, b, bin) <= UB(a, b, bin) = #{ b-events with an a-event in the
 //                                            bin's window }.
-// One pass over the stream: every event j looks back over the widest bin
+// For streams whose per-type lists have no room (fem_pairbound.cu reads
+// those).  One pass over the stream: every event j looks back over the widest bin
 // window and marks, per bin, which types occur (a per-thread bitset in shared
 // memory dedupes repeated types; word w of thread t at bits[w * blockDim + t]
 // so a warp's lanes touch distinct banks), then adds one to UB(a, type_j,
@@ -573,21 +574,78 @@ int MineGroup::gen_level2() {
     int32_t hi_max = 0;
     for (int k = 0; k < nb; ++k) hi_max = std::max(hi_max, bhi[k]);
     std::vector<const uint32_t *> ubp(n_recs);
+    std::vector<uint32_t> nth(n_recs);
+    std::vector<int64_t> ub_off(n_recs + 1, 0);
+    uint32_t nt_max = 1;
+    int64_t events = 0;
     for (int r = 0; r < n_recs; ++r) {
-        const uint32_t nt = recs[r]->n_types;
-        uint32_t *u;
-        FEM_TRY(tmp.get(&u, (size_t)nt * nt * nb));
-        FEM_CUDA_TRY(cudaMemsetAsync(u, 0, sizeof(uint32_t) * (size_t)nt * nt * nb, st));
-        const int words = (int)((nt * (uint32_t)nb + 31) / 32);
-        int threads = std::min(256, (int)(48 * 1024 / (4 * words)) / 32 * 32);
-        threads = std::max(threads, 32);
-        if (recs[r]->n > 0 && (prev.h_off[r + 1] - prev.h_off[r]) >= 2) {
-            const int64_t blocks = std::min<int64_t>((recs[r]->n + threads - 1) / threads, 8 * ctx->n_sm);
-            k_pair_ub<<<(unsigned)blocks, threads, (size_t)threads * words * 4, st>>>(
-                recs[r]->d_type, recs[r]->d_time, recs[r]->n, nt, d_blo, d_bhi, nb, hi_max, words, u);
-            S.kernel_launches++;
+        nth[r] = recs[r]->n_types;
+        nt_max = std::max(nt_max, nth[r]);
+        events += recs[r]->n;
+        ub_off[r + 1] = ub_off[r] + (int64_t)nth[r] * nth[r] * nb;
+    }
+    uint32_t *ub;
+    FEM_TRY(tmp.get(&ub, std::max<int64_t>(ub_off[n_recs], 1)));
+    FEM_CUDA_TRY(cudaMemsetAsync(ub, 0, sizeof(uint32_t) * std::max<int64_t>(ub_off[n_recs], 1), st));
+    for (int r = 0; r < n_recs; ++r) ubp[r] = ub + ub_off[r];
+    // by the per-type lists; without room for them (or over 2^30 events) each
+    // event looks back over the stream
+    int by_lists = FEM_OK;
+    for (int r = 0; r < n_recs && by_lists == FEM_OK; ++r) by_lists = stream_bytype(ctx, recs[r], true);
+    if (by_lists != FEM_OK && by_lists != FEM_ERR_NOMEM && by_lists != FEM_ERR_INVAL) return by_lists;
+    if (by_lists == FEM_OK) {
+        PairBoundArgs pb{};
+        pb.chunk = pair_bound_chunk(ctx->n_sm, events);
+        std::vector<int64_t> cpre(n_recs + 1, 0);
+        std::vector<RecInfo> ri(n_recs);
+        for (int r = 0; r < n_recs; ++r) {
+            const bool any = prev.h_off[r + 1] - prev.h_off[r] >= 2;
+            cpre[r + 1] = cpre[r] + (any ? (recs[r]->n + pb.chunk - 1) / pb.chunk : 0);
+            ri[r] = RecInfo{};
+            ri[r].type = recs[r]->d_type;
+            ri[r].time = recs[r]->d_time;
+            ri[r].n = recs[r]->n;
+            ri[r].freq = recs[r]->d_freq;
+            recinfo_lists(ri[r], recs[r]);
         }
-        ubp[r] = u;
+        RecInfo *d_ri;
+        int64_t *d_cpre, *d_uboff;
+        uint32_t *d_ntp;
+        FEM_TRY(tmp.get(&d_ri, n_recs));
+        FEM_TRY(tmp.get(&d_cpre, n_recs + 1));
+        FEM_TRY(tmp.get(&d_uboff, n_recs + 1));
+        FEM_TRY(tmp.get(&d_ntp, n_recs));
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_ri, ri.data(), sizeof(RecInfo) * n_recs, cudaMemcpyHostToDevice, st));
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_cpre, cpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_uboff, ub_off.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_ntp, nth.data(), 4 * n_recs, cudaMemcpyHostToDevice, st));
+        pb.ri = d_ri;
+        pb.n_recs = n_recs;
+        pb.cpre = d_cpre;
+        pb.n_items = cpre[n_recs];
+        pb.nt = d_ntp;
+        pb.thr = d_thr;
+        pb.ub_off = d_uboff;
+        pb.blo = d_blo;
+        pb.bhi = d_bhi;
+        pb.nb = nb;
+        pb.hi_max = hi_max;
+        pb.ub = ub;
+        FEM_TRY(pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, mean_window(recs, hi_max), last_time(recs)));
+        S.kernel_launches++;
+    } else {
+        for (int r = 0; r < n_recs; ++r) {
+            const int words = (int)((nth[r] * (uint32_t)nb + 31) / 32);
+            int threads = std::min(256, (int)(48 * 1024 / (4 * words)) / 32 * 32);
+            threads = std::max(threads, 32);
+            if (recs[r]->n > 0 && (prev.h_off[r + 1] - prev.h_off[r]) >= 2) {
+                const int64_t blocks = std::min<int64_t>((recs[r]->n + threads - 1) / threads, 8 * ctx->n_sm);
+                k_pair_ub<<<(unsigned)blocks, threads, (size_t)threads * words * 4, st>>>(
+                    recs[r]->d_type, recs[r]->d_time, recs[r]->n, nth[r], d_blo, d_bhi, nb, hi_max, words,
+                    ub + ub_off[r]);
+                S.kernel_launches++;
+            }
+        }
     }
     const uint32_t **d_ubp;
     uint32_t *d_nt;
@@ -599,8 +657,6 @@ int MineGroup::gen_level2() {
     FEM_TRY(tmp.get(&d_ptmp, C / 1024 + 2));
     FEM_TRY(tmp.get(&d_ptot, 2));
     FEM_TRY(pcand->get(&d_kept, C));
-    std::vector<uint32_t> nth(n_recs);
-    for (int r = 0; r < n_recs; ++r) nth[r] = recs[r]->n_types;
     FEM_CUDA_TRY(cudaMemcpyAsync(d_ubp, ubp.data(), sizeof(void *) * n_recs, cudaMemcpyHostToDevice, st));
     FEM_CUDA_TRY(cudaMemcpyAsync(d_nt, nth.data(), 4 * n_recs, cudaMemcpyHostToDevice, st));
     k_prune2_flags<<<(unsigned)((C + B - 1) / B), B, 0, st>>>(d_order, C, cand.types, cand.lo, cand.hi, cand.rec, d_ubp,

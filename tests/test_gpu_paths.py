@@ -55,3 +55,55 @@ def test_few_episodes_over_a_long_recording(fb, ctx, mid, wide, device):
     assert np.array_equal(got, want), np.nonzero(got != want)[0][:5]
     assert want.max() > 0
     st.free()
+
+
+def pair_bounds(ty, tm, n_types, bins):
+    """ub[a, b, k]: b-events with an a-event inside bin k before them."""
+    ub = np.zeros((n_types, n_types, len(bins)), np.int64)
+    per = [tm[ty == a].astype(np.int64) for a in range(n_types)]
+    for a in range(n_types):
+        for b in range(n_types):
+            for k, (lo, hi) in enumerate(bins):
+                first = np.searchsorted(per[a], per[b] - hi, side="left")
+                last = np.searchsorted(per[a], per[b] - lo, side="left")
+                ub[a, b, k] = int((last > first).sum())
+    return ub
+
+
+PAIR_BINS = {
+    "one": [(0, 7)],
+    "gaps": [(3, 9), (20, 21)],
+    "overlap": [(0, 12), (5, 30), (29, 31)],
+    "eight": [(4 * k, 4 * k + 4) for k in range(8)],
+    "wide": [(0, 70000), (70000, 2**31 - 1)],
+}
+
+
+@pytest.mark.parametrize("host_path", [False, True])
+@pytest.mark.parametrize("bins", sorted(PAIR_BINS))
+@pytest.mark.parametrize("n,n_types,t_max", [(40, 16, 30), (3000, 17, 9000), (2600, 40, 700), (5000, 16, 2**31 - 2)])
+def test_pair_bound_drops_what_its_definition_drops(fb, ctx, n, n_types, t_max, bins, host_path):
+    """Level 2: the candidates that the pair bound drops are those whose
+    number of (second, first inside the bin) events is at or below the
+    threshold, for windows of 0.1 to 100 events, ties, gaps between bins,
+    overlapping bins and a window that reaches the last possible time."""
+    ty, tm = synth.tiny_random_stream(31, n, n_types, t_max)
+    bl = PAIR_BINS[bins]
+    thr = max(1, n // (4 * n_types))
+    ub = pair_bounds(ty, tm, n_types, bl)
+    freq = np.bincount(ty, minlength=n_types)
+    pairs = (freq[:, None] > thr) & (freq[None, :] > thr) & ~np.eye(n_types, dtype=bool)
+    want = int((pairs[:, :, None] & (ub <= thr)).sum())
+    kept = int((pairs[:, :, None] & (ub > thr)).sum())
+    st = ctx.load_stream(ty, tm, n_types)
+    ctx.set_tuning(level_graph=-1 if host_path else 0)
+    try:
+        res = ctx.mine_levelwise([st], bl, [thr], 2)
+    finally:
+        ctx.reset_tuning()
+    if res.stats()["graph_tails"] == 1 and kept == 0:
+        want = 0  # a graph's statistics end before a level that counts nothing
+    assert res.stats()["candidates_pruned"] == want
+    assert res.stats()["candidates_counted"] == kept
+    res.free()
+    st.free()
