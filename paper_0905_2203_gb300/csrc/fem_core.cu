@@ -99,11 +99,29 @@ void pool_release(fem_ctx *ctx) {
     ctx->cached_bytes = 0;
 }
 
+// Gives the entry lists back to the driver unless the call in progress works
+// with them.
+static bool track_give_back(fem_ctx *ctx) {
+    if (ctx->track_held || !ctx->track.p) return false;
+    cudaStreamSynchronize(ctx->stream);
+    std::lock_guard<std::mutex> g(ctx->pool_mu);
+    auto it = ctx->live.find(ctx->track.p);
+    if (it != ctx->live.end()) {
+        ctx->used -= it->second;
+        ctx->live.erase(it);
+    }
+    cudaFree(ctx->track.p);
+    ctx->track = DevBuf{};
+    return true;
+}
+
 int dev_alloc(fem_ctx *ctx, void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~size_t(255);
-    if (ctx->used.load() + bytes > ctx->budget) return FEM_ERR_NOMEM;
+    if (ctx->used.load() + bytes > ctx->budget &&
+        (!track_give_back(ctx) || ctx->used.load() + bytes > ctx->budget))
+        return FEM_ERR_NOMEM;
     {
         std::lock_guard<std::mutex> g(ctx->pool_mu);
         auto it = ctx->cached.lower_bound(bytes);
@@ -122,6 +140,10 @@ int dev_alloc(fem_ctx *ctx, void **p, size_t bytes) {
         cudaGetLastError();
         pool_release(ctx);
         e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation && track_give_back(ctx)) {
+            cudaGetLastError();
+            e = cudaMalloc(p, bytes);
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -171,6 +193,20 @@ int scratch(fem_ctx *ctx, int slot, size_t bytes, void **p) {
     if (st != FEM_OK) return st;
     b.cap = want;
     *p = b.p;
+    return FEM_OK;
+}
+
+int track_lists(fem_ctx *ctx, size_t bytes, void **p) {
+    if (!ctx->track.p || ctx->track.cap < bytes) {
+        ctx->track_held = false;
+        track_give_back(ctx);
+        void *q = nullptr;
+        FEM_TRY(dev_alloc(ctx, &q, bytes));
+        std::lock_guard<std::mutex> g(ctx->pool_mu);
+        ctx->track = DevBuf{q, ctx->live[q]};
+    }
+    ctx->track_held = true;
+    *p = ctx->track.p;
     return FEM_OK;
 }
 
@@ -571,6 +607,7 @@ int fem::load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t
     if (n > 0 && (!types || !times)) return FEM_ERR_INVAL;
     if (n > (int64_t)INT32_MAX * 4) return FEM_ERR_INVAL;
     *out = nullptr;
+    track_release(ctx);
     cudaSetDevice(ctx->device);
     fem_stream *s = new (std::nothrow) fem_stream();
     if (!s) return FEM_ERR_NOMEM;

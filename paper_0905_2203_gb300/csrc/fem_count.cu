@@ -1824,6 +1824,7 @@ constexpr int64_t kPltMinEvents = 1 << 20;
 static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int force_segments) {
     fem_ctx *ctx = cc.ctx;
     const int n_recs = (int)cc.recs.size();
+    track_release(ctx);
     // Local tracking, one warp per (episode, segment), one launch for every
     // multi-node episode: the default (kernel 0) and kernel 7; the last
     // fallback round and the explicit kernel choices 1-3 keep the
@@ -1847,7 +1848,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     int64_t track_cap = 1;
     if (track) {
         for (auto *r : cc.recs) track_cap = std::max(track_cap, r->max_list);
-        const size_t free_b = ctx->budget > ctx->used.load() ? ctx->budget - ctx->used.load() : 0;
+        const size_t free_b = track_room(ctx);
         track_nblocks = track_blocks(ctx->n_sm);
         while (track_nblocks > 1 && track_buf_bytes(track_nblocks, track_cap) > free_b / 4)
             track_nblocks = track_nblocks > ctx->n_sm ? track_nblocks - ctx->n_sm : track_nblocks / 2;
@@ -2124,7 +2125,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             const int64_t n_items = limit > 0 ? std::min(limit, pl.records) : pl.records;
             blocks = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kTrackWarps - 1) / kTrackWarps));
             void *pb = nullptr;
-            FEM_TRY(scratch(ctx, kSlotTrack, track_buf_bytes(blocks, cap) + 256, &pb));
+            FEM_TRY(track_lists(ctx, track_buf_bytes(blocks, cap), &pb));
             TrackArgs ta{};
             ta.rinfo = d_ri;
             ta.n_recs = n_recs;
@@ -2176,7 +2177,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             ta.relaxed = cc.mode == 2;
             ta.skip = nullptr;
             ta.queue = reinterpret_cast<unsigned long long *>(mb + o_q);
-            ta.buf = reinterpret_cast<int32_t *>(static_cast<char *>(pb) + 256);
+            ta.buf = static_cast<int32_t *>(pb);
             ta.cap = cap;
             ta.rec = rec_base;
             ta.counts = limit > 0 ? nullptr : cc.counts;  // unsegmented episodes: counts written directly

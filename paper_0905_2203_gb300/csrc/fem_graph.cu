@@ -663,7 +663,7 @@ struct GraphTail {
     bool track = false;
     int track_nblocks = 0;
     int64_t track_cap = 0;                 // longest per-type list of any recording
-    int32_t *tbuf = nullptr;
+    int32_t *tbuf = nullptr;               // the context's entry lists when the graph was captured
     int64_t *tqueue = nullptr;
     int32_t *tg_gidx = nullptr, *tg_gstart = nullptr, *tg_gfirst = nullptr, *tg_stmp = nullptr;
     int32_t *tg_gmax = nullptr;            // per recording: the level's largest prefix group
@@ -778,7 +778,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     if (g->track) {
         g->track_nblocks = track_blocks(ctx->n_sm);
         for (auto *s : g->recs) g->track_cap = std::max(g->track_cap, s->max_list);
-        const size_t fb = ctx->budget > ctx->used.load() ? ctx->budget - ctx->used.load() : 0;
+        const size_t fb = track_room(ctx);
         while (g->track_nblocks > ctx->n_sm && track_buf_bytes(g->track_nblocks, g->track_cap) > fb / 4)
             g->track_nblocks -= ctx->n_sm;
         if (track_buf_bytes(g->track_nblocks, g->track_cap) > fb / 4) return FEM_ERR_NOMEM;
@@ -826,7 +826,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     }
     g->cap2 = cap2;
     const int64_t tot1 = ntpre[n_recs];
-    const size_t free_b = ctx->budget > ctx->used.load() ? ctx->budget - ctx->used.load() : 0;
+    const size_t free_b = track_room(ctx);
     // local tracking cuts grouped levels finer (records per candidate and
     // segment): room for four segments per candidate where the budget has it
     if (g->track && (size_t)(g->target + 4 * cap) * kRecWords * 4 <= free_b / 4) g->cap_threads = g->target + 4 * cap;
@@ -857,7 +857,9 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     FEM_TRY(g->get(&rec, (size_t)g->cap_threads * kRecWords));
     FEM_TRY(g->get(&g->d_maxP, 1));
     if (g->track) {
-        FEM_TRY(g->get(&g->tbuf, track_buf_bytes(g->track_nblocks, g->track_cap) / sizeof(int32_t)));
+        void *tb = nullptr;
+        FEM_TRY(track_lists(ctx, track_buf_bytes(g->track_nblocks, g->track_cap), &tb));
+        g->tbuf = static_cast<int32_t *>(tb);
         FEM_TRY(g->get(&g->tqueue, 1));
         FEM_TRY(g->get(&g->tg_gidx, cap + 2));
         FEM_TRY(g->get(&g->tg_gstart, cap + 2));
@@ -1319,9 +1321,14 @@ static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
     while (cap < want && cap < (1 << 24)) cap <<= 1;
     if (cap < want) return FEM_OK;
     GraphTail *g = nullptr;
+    track_release(ctx);
     auto it = ctx->graphs.find(key);
-    if (it != ctx->graphs.end() && it->second->cap >= cap) {
+    if (it != ctx->graphs.end() && it->second->cap >= cap &&
+        (!it->second->track ||
+         (it->second->tbuf == ctx->track.p &&
+          ctx->track.cap >= track_buf_bytes(it->second->track_nblocks, it->second->track_cap)))) {
         g = it->second;
+        ctx->track_held = g->track;
     } else {
         if (it != ctx->graphs.end()) {
             delete it->second;

@@ -184,6 +184,8 @@ struct fem_ctx {
     fem_tuning tuning{};
     fem_stats last{};
     std::map<int, fem::DevBuf> scratch;  // slot -> buffer (grown on demand)
+    fem::DevBuf track;                   // per-warp entry lists of the local-tracking kernel (track_lists)
+    bool track_held = false;             // the call in progress works with them
     std::map<std::string, fem::TuneVal> tune;  // autotuner cache
     std::map<std::string, fem::GraphTail *> graphs;  // captured mining graphs
     std::map<std::string, int64_t> graph_cap;        // candidate capacity a graph key needed last time
@@ -259,6 +261,19 @@ int dev_alloc(fem_ctx *ctx, void **p, size_t bytes);
 void dev_free(fem_ctx *ctx, void *p, size_t bytes);
 // Scratch slot of at least `bytes` (contents undefined).
 int scratch(fem_ctx *ctx, int slot, size_t bytes, void **p);
+// The context's per-warp entry lists, at least `bytes`: one buffer for every
+// counting launch and mining graph of the context (their work is ordered on
+// its stream; each launch writes what it reads).  Grown exactly; a call that
+// begins lets go of it (track_release), and an allocation that finds no room
+// then takes it back.  A captured graph remembers the pointer and is captured
+// again when the buffer has moved.
+int track_lists(fem_ctx *ctx, size_t bytes, void **p);
+inline void track_release(fem_ctx *ctx) { ctx->track_held = false; }
+// Budget left for those lists: what is free and what they hold.
+inline size_t track_room(const fem_ctx *ctx) {
+    const size_t used = ctx->used.load() - ctx->track.cap;
+    return ctx->budget > used ? ctx->budget - used : 0;
+}
 // Reads and clears the device status word (synchronises the stream).
 int sync_status(fem_ctx *ctx);
 // Copy helpers honouring host/device pointers.
@@ -450,7 +465,7 @@ enum Slot : int {
     kSlotCandOffs = 1, kSlotCandTypes, kSlotCandLo, kSlotCandHi, kSlotCandRec,
     kSlotPrep, kSlotPerm, kSlotBucket, kSlotRecords, kSlotSeg, kSlotCounts,
     kSlotFallback, kSlotRings, kSlotDensTab, kSlotScanTmp, kSlotMisc, kSlotRecTab, kSlotDensArgs,
-    kSlotTrack, kSlotTrackGrp,
+    kSlotTrackGrp,
     kSlotMine0 = 64,
 };
 
