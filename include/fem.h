@@ -143,12 +143,14 @@ typedef struct {
                              kernel first waits (with the default limit) for
                              its copies in flight, so the context stays
                              usable */
-    int track_last;       /* last node of the warp-per-item local tracking
-                             kernel: 0 = per (episode, segment), driven by
-                             node N-1's events or, when they outnumber node
-                             N-2's entries more than twice, by those entries
-                             (one lookup in the stream's per-type time index
-                             per entry, for the first end it can serve);
+    int track_last;       /* node steps of the warp-per-item local tracking
+                             kernel, from the second node to the last: 0 =
+                             per step, driven by the node's events or, when
+                             they outnumber the previous node's entries more
+                             than twice, by those entries (lookups in the
+                             stream's per-type time index for the events
+                             each entry serves: all of them for an inner
+                             node, the first one for the last node);
                              1 = always by events; 2 = always by entries */
 } fem_tuning;
 

@@ -265,6 +265,72 @@ __device__ __forceinline__ void last_by_index(const int32_t *__restrict__ tl, in
     __syncwarp();
 }
 
+// An inner node step driven by node k-1's entries, for entry lists shorter
+// than the node's event list: entry i's events are those in
+// (T_i + lo, min(T_i + hi, T_{i+1} + lo)], all valid with latest start L_i, and
+// the intervals of successive entries follow one another, so the lanes' events
+// in lane order are the node's entries in time order.  One lookup in the time
+// index finds an interval's first event, as in last_by_index; most intervals
+// hold none or one (compacted by ballot), the others are counted and placed
+// by a scan.
+//
+// Entries thin out node by node (60 types at 20 Hz with bursts, 5 ms edges:
+// 23%, 11%, 6.5% of a type's events), so from the third node on the events
+// are several times the entries: 200k episodes of 2-8 nodes over 4M events
+// 174 -> 131 ms.
+template <bool HASL>
+__device__ __forceinline__ int inner_by_index(const int32_t *__restrict__ tl, int cb, int ce,
+                                              const int32_t *__restrict__ row, int shift, uint32_t tbase,
+                                              int64_t ncell, Entries<HASL> p, int m, int32_t lo_e, int32_t hi_e,
+                                              int2 *__restrict__ out, int lane) {
+    const uint32_t lo = (uint32_t)lo_e, hi = (uint32_t)hi_e;
+    int wc = 0;  // entries written
+    int2 next = lane < m ? p.get(lane) : make_int2(-1, 0);
+    for (int base = 0; base < m; base += 32) {
+        const int i = base + lane;
+        const int2 E = next;
+        // the next 32 entries; the first of them ends this chunk's last interval
+        next = i + 32 < m ? p.get(i + 32) : make_int2(-1, 0);
+        const uint32_t T = (uint32_t)E.x, q = T + lo + 1u;
+        uint32_t Tn = __shfl_down_sync(kFull, T, 1);
+        const uint32_t T_after = __shfl_sync(kFull, (uint32_t)next.x, 0);
+        if (lane == 31) Tn = T_after;
+        uint32_t end = T + hi;
+        if (i + 1 < m) end = min(end, Tn + lo);
+        const uint64_t c = q > tbase ? (uint64_t)((q - tbase) >> shift) : 0;
+        int pos = i < m ? row[c < (uint64_t)ncell ? c : (uint64_t)ncell] : ce;
+        if (pos < cb) pos = cb;
+        uint32_t x = pos < ce ? (uint32_t)tl[pos] : 0xFFFFFFFFu;
+        while (x < q) {
+            ++pos;
+            x = pos < ce ? (uint32_t)tl[pos] : 0xFFFFFFFFu;
+        }
+        const bool ok = i < m && x <= end;
+        const bool two = ok && pos + 1 < ce && (uint32_t)tl[pos + 1] <= end;
+        const unsigned bm = __ballot_sync(kFull, ok);
+        if (!__any_sync(kFull, two)) {
+            if (ok) out[wc + __popc(bm & ((1u << lane) - 1u))] = make_int2((int32_t)x, E.y);
+            wc += __popc(bm);
+        } else {
+            int n = ok ? 1 : 0;
+            if (two) {
+                n = 2;
+                while (pos + n < ce && (uint32_t)tl[pos + n] <= end) ++n;
+            }
+            int at = n;  // inclusive scan over the lanes
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int y = __shfl_up_sync(kFull, at, d);
+                if (lane >= d) at += y;
+            }
+            for (int k = 0; k < n; ++k) out[wc + at - n + k] = make_int2(tl[pos + k], E.y);
+            wc += __shfl_sync(kFull, at, 31);
+        }
+    }
+    __syncwarp();
+    return wc;
+}
+
 __device__ __forceinline__ void machine_init(Machine<2, 0> &st, int N) {
     st.N = N;
     st.ncls = 0;
@@ -374,6 +440,14 @@ __global__ void __launch_bounds__(kTrackWarps * 32, kTrackMaxBlocksPerSm) k_coun
                 e = (seg_e < ri.n) ? warp_lower_bound(ttime, b, b1, Tend, lane) : b1;
             }
         };
+        // whether a node with n_ev events is stepped by node k-1's m entries:
+        // the entry steps' scattered lookups cost about two streamed events
+        // (the same 200k episodes: 143 ms with the line at 1, 131 at 2, 130 at
+        // 3; 48 recordings with groups of 3-node episodes are fastest at 1-2)
+        auto by_entries = [&](int m, int n_ev) {
+            return ri.tidx &&
+                   (a.last_mode == 2 || (a.last_mode == 0 && (int64_t)m * kTrackEntryRatio < (int64_t)n_ev));
+        };
         // shared prefix: node 0 (its type's times), then nodes 1..N-2
         // (entry lists in the warp's buffer)
         Entries<false> p0{nullptr};
@@ -390,7 +464,17 @@ __global__ void __launch_bounds__(kTrackWarps * 32, kTrackMaxBlocksPerSm) k_coun
                 range(a.ctypes[o0 + k], cb, ce);
                 int2 *out = (k & 1) ? b1 : b0;
                 const int32_t lo_k = a.relaxed ? 0 : a.clo[eo0 + k - 1], hi_k = a.chi[eo0 + k - 1];
-                if (k == 1)
+                if (by_entries(m, (int)(ce - cb))) {
+                    const uint32_t E = a.ctypes[o0 + k];
+                    const int64_t t0 = toff[E];
+                    const int32_t *row = ri.tidx + (int64_t)E * (ri.tcells + 1);
+                    if (k == 1)
+                        m = inner_by_index(ttime + t0, (int)(cb - t0), (int)(ce - t0), row, ri.tshift,
+                                           (uint32_t)ri.tbase, ri.tcells, p0, m, lo_k, hi_k, out, lane);
+                    else
+                        m = inner_by_index(ttime + t0, (int)(cb - t0), (int)(ce - t0), row, ri.tshift,
+                                           (uint32_t)ri.tbase, ri.tcells, pe, m, lo_k, hi_k, out, lane);
+                } else if (k == 1)
                     m = node_step<false>(ttime + cb, (int)(ce - cb), p0, m, lo_k, hi_k, out, st, 0, lane);
                 else
                     m = node_step<false>(ttime + cb, (int)(ce - cb), pe, m, lo_k, hi_k, out, st, 0, lane);
@@ -412,11 +496,8 @@ __global__ void __launch_bounds__(kTrackWarps * 32, kTrackMaxBlocksPerSm) k_coun
                 range(a.ctypes[oc + N - 1], cb, ce);
                 const int n_ev = (int)(ce - cb);
                 const int32_t lo_l = a.relaxed ? 0 : a.clo[ec + N - 2], hi_l = a.chi[ec + N - 2];
-                // entries well short of the events: search per entry
-                const bool by_entries = ri.tidx && (a.last_mode == 2 || (a.last_mode == 0 &&
-                                                                         (int64_t)m * kTrackEntryRatio < (int64_t)n_ev));
                 const int32_t *evl = ttime + cb;
-                if (by_entries) {
+                if (by_entries(m, n_ev)) {
                     const uint32_t E = a.ctypes[oc + N - 1];
                     const int64_t t0 = toff[E];
                     const int32_t *row = ri.tidx + (int64_t)E * (ri.tcells + 1);
