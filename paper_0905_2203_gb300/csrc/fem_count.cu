@@ -1820,6 +1820,76 @@ static int count_grid_wide(CountCall &cc, std::vector<int32_t> &work, int varian
 constexpr int64_t kPltMaxCands = 256;
 constexpr int64_t kPltMinEvents = 1 << 20;
 
+// Large candidate sets in which few episodes share all but their last node
+// (a random or hand-made set, not a level-wise join): the slots are sorted by
+// recording, first node, second node and first edge, so that one item tracks
+// the common two-node prefix once for all of its episodes.  That prefix is the
+// longest step (every event of two types; later nodes run over the few
+// entries left): 200k episodes of 2-8 nodes, 60 types, 4M events, 14 episodes
+// a group.  The sort (three or four partition passes) and its two host reads
+// cost 0.4 ms: for sets of at least kPairMinSlots episodes and kPairMinWork
+// relevant events (about 2.5 ms of counting).
+constexpr int64_t kPairMinSlots = 1 << 14;
+constexpr double kPairMinWork = 1e9;
+constexpr double kPairMinAvg = 2.0;   // episodes per group that repay the order ...
+constexpr double kPairMaxJoin = 3.0;  // ... unless groups of all but the last node are this large
+
+static int group_pairs(CountCall &cc, int32_t *d_perm, int64_t ns, bool *use, double *avg) {
+    fem_ctx *ctx = cc.ctx;
+    cudaStream_t st = ctx->stream;
+    const int n_recs = (int)cc.recs.size();
+    int nt = 1;
+    for (auto *r : cc.recs) nt = std::max(nt, (int)r->n_types);
+    const int n_keys[4] = {kPairEdgeKeys, nt, nt, n_recs};
+    if (n_recs > 8192) return FEM_OK;
+    const int64_t nblk = (ns + kPartBlock - 1) / kPartBlock;
+    const int64_t tab_n = (int64_t)std::max({kPairEdgeKeys, nt, n_recs}) * nblk;
+    TmpDev tmp(ctx);
+    int32_t *key, *perm[2], *blk, *stmp, *total;
+    if (tmp.get(&key, ns + 2) != FEM_OK || tmp.get(&perm[0], ns) != FEM_OK || tmp.get(&perm[1], ns) != FEM_OK ||
+        tmp.get(&blk, tab_n) != FEM_OK || tmp.get(&stmp, std::max(tab_n, ns + 2) / kScanBlock + 2) != FEM_OK ||
+        tmp.get(&total, 1) != FEM_OK)
+        return FEM_OK;  // no room: the order stays
+    TrackGroupIn gi{};
+    gi.slot2cand = d_perm;
+    gi.n_slots_cap = ns;
+    gi.offs = cc.offs;
+    gi.ctypes = cc.types;
+    gi.clo = cc.lo;
+    gi.chi = cc.hi;
+    gi.cand_rec = cc.cand_rec;
+    auto groups = [&](bool pair, double *a) -> int {
+        gi.pair = pair;
+        gi.gidx = key;
+        FEM_TRY(track_group_flags(st, ctx->n_sm, gi));
+        FEM_TRY(scan_exclusive(st, key, ns + 1, stmp, total, &cc.stats.kernel_launches));
+        int32_t g = 0;
+        FEM_CUDA_TRY(cudaMemcpyAsync(&g, total, 4, cudaMemcpyDeviceToHost, st));
+        FEM_CUDA_TRY(cudaStreamSynchronize(st));
+        *a = (double)ns / std::max(g, 1);
+        return FEM_OK;
+    };
+    double join = 1.0;
+    FEM_TRY(groups(false, &join));
+    if (join >= kPairMaxJoin) return FEM_OK;
+    for (int w = 0; w < (n_recs > 1 ? 4 : 3); ++w) {
+        track_pair_keys(st, ctx->n_sm, gi, w, key);
+        k_part_count<<<(unsigned)nblk, 256, n_keys[w] * 4, st>>>(key, ns, n_keys[w], nblk, blk);
+        FEM_TRY(scan_exclusive(st, blk, (int64_t)n_keys[w] * nblk, stmp, nullptr, &cc.stats.kernel_launches));
+        k_part_scatter<<<(unsigned)nblk, 32, n_keys[w] * 4, st>>>(key, ns, n_keys[w], nblk, blk, gi.slot2cand,
+                                                                  perm[w & 1], nullptr);
+        gi.slot2cand = perm[w & 1];
+    }
+    FEM_CUDA_TRY(cudaGetLastError());
+    double pair = 1.0;
+    FEM_TRY(groups(true, &pair));
+    if (pair < kPairMinAvg) return FEM_OK;
+    FEM_CUDA_TRY(cudaMemcpyAsync(d_perm, gi.slot2cand, 4 * ns, cudaMemcpyDeviceToDevice, st));
+    *use = true;
+    *avg = pair;
+    return FEM_OK;
+}
+
 // Builds the per-recording RecInfo table and the density table.
 static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int force_segments) {
     fem_ctx *ctx = cc.ctx;
@@ -1981,6 +2051,14 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             cc.stats.counted_episode_events += (double)(key_off[k + 1] - key_off[k]) * (double)cc.recs[k % n_recs]->n;
     cc.stats.relevant_events += (double)relv;
 
+    // --- groups by the first two nodes for large sets
+    bool pair_groups = false;
+    double pair_avg = 1.0;  // episodes per group
+    if (track && ctx->tuning.kernel == 0 && force_segments == 0 && bmax[kBuckets] >= 3 &&
+        key_off[n_recs] >= kPairMinSlots && (double)relv >= kPairMinWork &&
+        track_buf_bytes(track_nblocks, track_cap, true) <= track_room(ctx) / 4)
+        FEM_TRY(group_pairs(cc, d_perm, key_off[n_recs], &pair_groups, &pair_avg));
+
     // --- launches per bucket
     const int T_def = ctx->tuning.tile_events > 0 ? ctx->tuning.tile_events : 1024;
     struct Plan {
@@ -2028,6 +2106,9 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
                 work += (double)c * (double)cc.recs[r]->n;
             }
             seg_len = std::max(1.0, work / desired) / seg_mult;
+            // an item is a whole group: four items' worth of segments per
+            // group keep the launch's tail short
+            if (pl.track && pair_groups) seg_len /= kTrackPairCut * pair_avg;
         } else {
             const size_t sm = tiled_smem_rt(pl.nclass, K, pl.R, T);
             const int occ = occupancy_tiled(pl.nclass, K, pl.R, sm);
@@ -2125,7 +2206,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             const int64_t n_items = limit > 0 ? std::min(limit, pl.records) : pl.records;
             blocks = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kTrackWarps - 1) / kTrackWarps));
             void *pb = nullptr;
-            FEM_TRY(track_lists(ctx, track_buf_bytes(blocks, cap), &pb));
+            FEM_TRY(track_lists(ctx, track_buf_bytes(blocks, cap, pair_groups), &pb));
             TrackArgs ta{};
             ta.rinfo = d_ri;
             ta.n_recs = n_recs;
@@ -2165,6 +2246,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
                 gi.gstart = i32 + (ns + 2);
                 gi.gfirst = i32 + 2 * (ns + 2);
                 gi.scan_tmp = i32 + 2 * (ns + 2) + n_recs;
+                gi.pair = pair_groups;
                 const bool grouped = ctx->tuning.kernel != 7;
                 FEM_TRY(track_groups(ctx->stream, ctx->n_sm, gi, grouped, &ta));
                 cc.stats.kernel_launches += grouped ? 4 : 1;

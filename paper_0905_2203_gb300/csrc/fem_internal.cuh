@@ -82,6 +82,12 @@ struct RecInfo {
 constexpr int kTrackWarps = 8;           // warps per block
 constexpr int kTrackMaxBlocksPerSm = 6;  // resident blocks per SM the grid asks for (40 registers)
 constexpr int kTrackGroupMax = 64;       // episodes per prefix group (a new group every 64 slots)
+// Groups of a common two-node prefix: episodes per group and segments per
+// group (this times its episodes).  200k episodes over 4M events, (16, 12):
+// (8, 4) 122 ms, (16, 4) 148, (8, 12) 96, (16, 12) 99, (32, 12) 101,
+// (16, 40) 97: a group of frequent chains outlasts the launch when cut coarsely.
+constexpr int kTrackPairMax = 16;
+constexpr double kTrackPairCut = 12.0;
 constexpr int kTrackMinSeg = 8192;       // shortest segment (events) of a local-tracking item
 constexpr int kTrackEntryRatio = 2;      // last node by entries when events > this x entries
 constexpr int kTrackEntrySlots = 2;      // entries per lane of the entry-driven last node step
@@ -99,7 +105,7 @@ struct TrackArgs {
     int relaxed;                 // every lower bound taken as 0 (upper bound)
     const uint8_t *skip;         // if set, candidates c with skip[c] != 0 are not counted
     unsigned long long *queue;   // work counter (zeroed by launch_track)
-    int32_t *buf;                // per warp 4 * cap words (entry lists, ping-pong)
+    int32_t *buf;                // per warp 4 * cap words (two entry lists), 6 * cap with `pair`
     int64_t cap;                 // at least the longest per-type list of every recording
     int32_t *rec;                // records, kRecWords each
     uint32_t *counts;            // if set: episodes of unsegmented recordings (P = 1) write their
@@ -113,7 +119,8 @@ struct TrackArgs {
     const int32_t *gfirst;
     const int64_t *ibase;
     const int32_t *rorder;
-    int last_mode;               // last node: 0 by the shorter side, 1 by events, 2 by entries
+    int last_mode;               // node steps: 0 by the shorter side, 1 by events, 2 by entries
+    int pair;                    // groups share their first two nodes (else all but the last)
 };
 // Inputs of track_groups: the slots (slot2cand, live count on the device or
 // n_slots_cap), the candidate CSR, per-candidate recordings, the launch's
@@ -136,6 +143,7 @@ struct TrackGroupIn {
     int64_t *ibase, *n_items;
     int32_t *gmax;               // if set: per recording, the largest group (track_group_starts)
     bool starts_ready;           // gidx / gstart already written by track_group_starts
+    bool pair;                   // groups by the first two nodes and their edge
 };
 
 // Results of the levels of level-wise mining run in a captured graph.
@@ -455,9 +463,15 @@ inline double mean_window(const std::vector<fem_stream *> &recs, int64_t hi) {
 // Prefix groups of the slots (flags, scan, first slot of each group, and,
 // if in.gmax is set, each recording's largest group) without the item
 // numbering, which depends on the segmentation.
+int track_group_flags(cudaStream_t st, int n_sm, const TrackGroupIn &in);
 int track_group_starts(cudaStream_t st, int n_sm, const TrackGroupIn &in);
 int track_groups(cudaStream_t st, int n_sm, const TrackGroupIn &in, bool grouped, TrackArgs *a);
-size_t track_buf_bytes(int blocks, int64_t cap);
+// Sort keys that bring slots with the same first two nodes together (least
+// significant first: which = 0 the edge, 1 the second node, 2 the first, 3 the
+// recording).
+constexpr int kPairEdgeKeys = 256;
+void track_pair_keys(cudaStream_t st, int n_sm, const TrackGroupIn &in, int which, int32_t *key);
+size_t track_buf_bytes(int blocks, int64_t cap, bool pair = false);
 int launch_track(cudaStream_t st, int blocks, const TrackArgs &a);
 
 // Scratch slot ids.

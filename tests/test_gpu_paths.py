@@ -107,3 +107,61 @@ def test_pair_bound_drops_what_its_definition_drops(fb, ctx, n, n_types, t_max, 
     assert res.stats()["candidates_counted"] == kept
     res.free()
     st.free()
+
+
+@pytest.mark.parametrize("recs", [1, 3])
+@pytest.mark.parametrize("size_lo,size_hi", [(1, 5), (3, 3), (2, 16)])
+def test_large_sets_share_their_first_two_nodes(fb, ctx, size_lo, size_hi, recs):
+    """Sets large enough to be sorted by their first two nodes (2^14 episodes,
+    1e9 relevant events), of mixed sizes, over one and several recordings:
+    counts in input order.  Ten types and two bins make groups far longer than
+    one item holds."""
+    n_types, n_cand = 10, 21_000
+    r = synth.Rng(5, size_hi)
+    streams = [synth.tiny_random_stream(40 + i, 160_000 - 40_000 * i, n_types, 1_300_000) for i in range(recs)]
+    sizes = r.integers(size_lo, size_hi, n_cand)
+    offs = np.zeros(n_cand + 1, np.int64)
+    offs[1:] = np.cumsum(sizes)
+    ct = r.integers(0, n_types - 1, int(offs[-1])).astype(np.uint16)
+    pick = r.integers(0, 1, int(offs[-1]) - n_cand)
+    lo, hi = np.array([0, 9], np.int32)[pick], np.array([30, 55], np.int32)[pick]
+    rec = r.integers(0, recs - 1, n_cand).astype(np.uint32)
+    st = [ctx.load_stream(ty, tm, n_types) for ty, tm in streams]
+    got = ctx.count_batch(st, fb.Cands(offs, ct, lo, hi), rec).astype(np.int64)
+    for i, (ty, tm) in enumerate(streams):
+        which = np.nonzero(rec == i)[0]
+        so = np.zeros(len(which) + 1, np.int64)
+        so[1:] = np.cumsum(sizes[which])
+        nodes = np.concatenate([np.arange(offs[c], offs[c + 1]) for c in which])
+        edges = np.concatenate([np.arange(offs[c] - c, offs[c + 1] - c - 1) for c in which])
+        want = oracle_counts(ty, tm, so, ct[nodes], lo[edges], hi[edges])
+        assert np.array_equal(got[which], want), np.nonzero(got[which] != want)[0][:5]
+    assert got.max() > 0
+    for s in st:
+        s.free()
+
+
+@pytest.mark.parametrize("t_max", [2_000, 40_000, 900_000])
+@pytest.mark.parametrize("n", [31, 33, 64, 1000, 30_000])
+def test_inner_nodes_by_entries(fb, ctx, n, t_max):
+    """Inner nodes stepped by entries (forced), from 0.2 to 100 events of a
+    type inside an edge, with chunks of entries that end a warp's 32."""
+    n_types = 4
+    ty, tm = synth.tiny_random_stream(60, n, n_types, t_max)
+    r = synth.Rng(61, n)
+    n_cand = 200
+    sizes = r.integers(3, 6, n_cand)
+    offs = np.zeros(n_cand + 1, np.int64)
+    offs[1:] = np.cumsum(sizes)
+    ct = r.integers(0, n_types - 1, int(offs[-1])).astype(np.uint16)
+    lo = r.integers(0, 40, int(offs[-1]) - n_cand).astype(np.int32)
+    hi = (lo + 1 + r.integers(0, 60, lo.size)).astype(np.int32)
+    want = oracle_counts(ty, tm, offs, ct, lo, hi)
+    st = ctx.load_stream(ty, tm, n_types)
+    ctx.set_tuning(track_last=2)
+    try:
+        got = ctx.count_episodes(st, fb.Cands(offs, ct, lo, hi)).astype(np.int64)
+    finally:
+        ctx.reset_tuning()
+    assert np.array_equal(got, want), np.nonzero(got != want)[0][:5]
+    st.free()
