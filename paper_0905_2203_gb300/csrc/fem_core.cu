@@ -240,19 +240,29 @@ int copy_out(fem_ctx *ctx, void *dst, const void *src_dev, size_t bytes, int dst
 }
 
 // ---------------------------------------------------------------------------
-// Stream validation (Definition 1 plus the library's input rules): type in
-// range, time >= 0, times non-decreasing, no repeated (type, time).  A
-// repeated pair must sit inside one run of equal times, so each event looks
-// back only while the time is unchanged.
-__global__ void k_validate(const uint16_t *__restrict__ ty, const int32_t *__restrict__ tm, int64_t n,
-                           uint32_t n_types, int *err) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// Stream validation (Definition 1 plus the library's input rules) and level 1
+// in one pass: type in range, time >= 0, times non-decreasing, no repeated
+// (type, time); a repeated pair must sit inside one run of equal times, so
+// each event looks back only while the time is unchanged.  Level 1 (a 1-node
+// episode's count is its frequency): per-type histogram, privatised in shared
+// memory when the alphabet fits; out-of-range types are skipped (the host has
+// not read the validation result yet).
+__global__ void k_load_scan(const uint16_t *__restrict__ ty, const int32_t *__restrict__ tm, int64_t n,
+                            uint32_t n_types, int *err, uint32_t *__restrict__ freq) {
+    extern __shared__ uint32_t h[];
+    const bool priv = n_types <= 12288;
+    if (priv)
+        for (uint32_t a = threadIdx.x; a < n_types; a += blockDim.x) h[a] = 0;
+    __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int e = 0;
-    for (; i < n; i += stride) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint16_t a = ty[i];
         const int32_t t = tm[i];
-        if (a >= n_types) e |= 1;
+        if (a >= n_types)
+            e |= 1;
+        else
+            atomicAdd(priv ? &h[a] : &freq[a], 1u);
         if (t < 0 || t == INT32_MAX) e |= 2;
         if (i > 0) {
             const int32_t tp = tm[i - 1];
@@ -265,31 +275,29 @@ __global__ void k_validate(const uint16_t *__restrict__ ty, const int32_t *__res
         }
     }
     if (e) atomicOr(err, e);
-}
-
-// Level 1 (a 1-node episode's count is its frequency): per-type histogram,
-// privatised in shared memory when the alphabet fits.  It runs before the
-// host has read the validation result, so out-of-range types are skipped.
-__global__ void k_histogram(const uint16_t *__restrict__ ty, int64_t n, uint32_t n_types,
-                            uint32_t *__restrict__ freq) {
-    extern __shared__ uint32_t h[];
-    const bool priv = n_types <= 12288;
-    if (priv)
-        for (uint32_t a = threadIdx.x; a < n_types; a += blockDim.x) h[a] = 0;
-    __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint16_t a = ty[i];
-        if (a >= n_types) continue;
-        if (priv)
-            atomicAdd(&h[a], 1u);
-        else
-            atomicAdd(&freq[a], 1u);
-    }
     __syncthreads();
     if (priv)
         for (uint32_t a = threadIdx.x; a < n_types; a += blockDim.x)
             if (h[a]) atomicAdd(&freq[a], h[a]);
+}
+
+// What the host needs to know of a loaded stream, in one read: the validation
+// result, the first and last time, the largest frequency (one block).
+__global__ void k_load_info(const int32_t *__restrict__ tm, int64_t n, const uint32_t *__restrict__ freq,
+                            uint32_t n_types, const int *err, int *info) {
+    __shared__ uint32_t s_max;
+    if (threadIdx.x == 0) s_max = 0;
+    __syncthreads();
+    uint32_t m = 0;
+    for (uint32_t a = threadIdx.x; a < n_types; a += blockDim.x) m = max(m, freq[a]);
+    atomicMax(&s_max, m);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        info[0] = *err;
+        info[1] = n > 0 ? tm[0] : 0;
+        info[2] = n > 0 ? tm[n - 1] : 0;
+        info[3] = (int)s_max;
+    }
 }
 
 __global__ void k_fill_pad(uint16_t *ty, int32_t *tm, int64_t from, int64_t to) {
@@ -508,16 +516,16 @@ extern "C" int fem_ctx_create(int device, size_t hbm_budget_bytes, void *cuda_st
         ctx->own_stream = true;
     }
     void *p = nullptr;
-    int st = dev_alloc(ctx, &p, sizeof(int) * 4);
+    int st = dev_alloc(ctx, &p, sizeof(int) * kStatusWords);
     if (st != FEM_OK) {
         if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
         return st;
     }
     ctx->d_status = static_cast<int *>(p);
-    cudaMemsetAsync(ctx->d_status, 0, sizeof(int) * 4, ctx->stream);
-    if (cudaMallocHost(&ctx->h_status, sizeof(int) * 4) != cudaSuccess) {
-        dev_free(ctx, ctx->d_status, sizeof(int) * 4);
+    cudaMemsetAsync(ctx->d_status, 0, sizeof(int) * kStatusWords, ctx->stream);
+    if (cudaMallocHost(&ctx->h_status, sizeof(int) * kStatusWords) != cudaSuccess) {
+        dev_free(ctx, ctx->d_status, sizeof(int) * kStatusWords);
         if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
         return FEM_ERR_CUDA;
@@ -538,7 +546,7 @@ extern "C" void fem_ctx_destroy(fem_ctx *ctx) {
     ctx->pinned = nullptr;
     for (auto &kv : ctx->scratch) dev_free(ctx, kv.second.p, kv.second.cap);
     ctx->scratch.clear();
-    dev_free(ctx, ctx->d_status, sizeof(int) * 4);
+    dev_free(ctx, ctx->d_status, sizeof(int) * kStatusWords);
     pool_release(ctx);
     for (auto &kv : ctx->live) cudaFree(kv.first);
     ctx->live.clear();
@@ -640,24 +648,21 @@ int fem::load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t
     cudaMemsetAsync(ctx->d_status + 1, 0, sizeof(int), ctx->stream);
     if (n > 0) {
         const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, ctx->n_sm * 8));
-        k_validate<<<blocks, 256, 0, ctx->stream>>>(s->d_type, s->d_time, n, n_types, ctx->d_status + 1);
         const size_t hs = n_types <= 12288 ? n_types * sizeof(uint32_t) : 0;
-        k_histogram<<<blocks, 256, hs, ctx->stream>>>(s->d_type, n, n_types, s->d_freq);
+        k_load_scan<<<blocks, 256, hs, ctx->stream>>>(s->d_type, s->d_time, n, n_types, ctx->d_status + 1, s->d_freq);
     }
+    int *const info = ctx->h_status + kStatusInfo;
+    k_load_info<<<1, 256, 0, ctx->stream>>>(s->d_time, n, s->d_freq, n_types, ctx->d_status + 1,
+                                            ctx->d_status + kStatusInfo);
     if (cudaGetLastError() != cudaSuccess) return fail(FEM_ERR_CUDA);
-    if (cudaMemcpyAsync(ctx->h_status + 1, ctx->d_status + 1, sizeof(int), cudaMemcpyDeviceToHost,
-                        ctx->stream) != cudaSuccess ||
+    if (cudaMemcpyAsync(info, ctx->d_status + kStatusInfo, 4 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) !=
+            cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
         return fail(FEM_ERR_CUDA);
-    const int e = ctx->h_status[1];
-    if (n > 0 && e == 0) {
-        int32_t tt[2] = {0, 0};
-        if (cudaMemcpy(&tt[0], s->d_time, 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-            cudaMemcpy(&tt[1], s->d_time + n - 1, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-            return fail(FEM_ERR_CUDA);
-        s->t_first = tt[0];
-        s->t_last = tt[1];
-    }
+    const int e = info[0];
+    s->t_first = info[1];
+    s->t_last = info[2];
+    s->max_list = (int64_t)(uint32_t)info[3];
     if (e & 1) return fail(FEM_ERR_INVAL);
     if (e & 2) return fail(FEM_ERR_RANGE);
     if (e & 4) return fail(FEM_ERR_UNSORTED);

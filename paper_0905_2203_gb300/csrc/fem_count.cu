@@ -819,11 +819,17 @@ __global__ void k_prep(PrepArgs a) {
 // Stable partition by key: blocks of kPartBlock elements.  k_part_count
 // writes blk[k * nblk + b] = elements of block b with key k; after an
 // exclusive scan of that key-major table, blk[k * nblk + b] is where block b's
-// first key-k element goes, and k_part_scatter (one warp per block, walking
-// its elements in order) assigns stable positions.
+// first key-k element goes, and k_part_scatter assigns stable positions: each
+// of the block's warps takes a contiguous part, counts its keys, starts after
+// the warps before it and walks its elements 32 at a time (equal keys of a
+// step ranked by a match).  One warp per block walked all 4096 alone, a chain
+// of 128 steps: the lists of 1M events took 86 us and a gather of 8 us, those
+// of 20M events 243 and 117 us; now 20 and 289 us, times written directly.
 constexpr int kPartBlock = 4096;
+constexpr int kPartWarps = 8;
 
-__global__ void k_part_count(const int32_t *__restrict__ key, int64_t n, int n_keys, int64_t nblk,
+template <typename K>
+__global__ void k_part_count(const K *__restrict__ key, int64_t n, int n_keys, int64_t nblk,
                              int32_t *__restrict__ blk) {
     extern __shared__ int32_t cnt[];
     for (int k = threadIdx.x; k < n_keys; k += blockDim.x) cnt[k] = 0;
@@ -835,30 +841,75 @@ __global__ void k_part_count(const int32_t *__restrict__ key, int64_t n, int n_k
     for (int k = threadIdx.x; k < n_keys; k += blockDim.x) blk[(int64_t)k * nblk + blockIdx.x] = cnt[k];
 }
 
-__global__ void k_part_scatter(const int32_t *__restrict__ key, int64_t n, int n_keys, int64_t nblk,
-                               const int32_t *__restrict__ blk, const int32_t *__restrict__ subset,
-                               int32_t *__restrict__ out, int32_t *__restrict__ out_key) {
-    extern __shared__ int32_t run[];
-    const int lane = threadIdx.x;
-    for (int k = lane; k < n_keys; k += 32) run[k] = blk[(int64_t)k * nblk + blockIdx.x];
-    __syncwarp();
-    const int64_t b0 = blockIdx.x * (int64_t)kPartBlock;
-    const int64_t b1 = (n < b0 + kPartBlock) ? n : b0 + kPartBlock;
+// Element i goes to position pos: out[pos] = subset[i] (or i), out_key[pos] =
+// its key, out_tm[pos] = tm[i], each where asked for.
+struct PartOut {
+    const int32_t *subset;
+    int32_t *out, *out_key;
+    const int32_t *tm;
+    int32_t *out_tm;
+};
+
+template <typename K>
+__global__ void __launch_bounds__(kPartWarps * 32)
+    k_part_scatter(const K *__restrict__ key, int64_t n, int n_keys, int64_t nblk, const int32_t *__restrict__ blk,
+                   PartOut o) {
+    extern __shared__ int32_t s_run[];  // per warp: next position of every key
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int32_t *run = s_run + w * n_keys;
+    const int per = kPartBlock / nw;
+    const int64_t b0 = blockIdx.x * (int64_t)kPartBlock + w * per;
+    const int64_t b1 = min(n, b0 + per);
+    if (nw > 1) {
+        for (int k = threadIdx.x; k < nw * n_keys; k += blockDim.x) s_run[k] = 0;
+        __syncthreads();
+        for (int64_t i = b0 + lane; i < b1; i += 32) atomicAdd(&run[key[i]], 1);
+        __syncthreads();
+    }
+    for (int k = threadIdx.x; k < n_keys; k += blockDim.x) {
+        int32_t at = blk[(int64_t)k * nblk + blockIdx.x];
+        for (int v = 0; v < nw; ++v) {
+            const int32_t c = nw > 1 ? s_run[v * n_keys + k] : 0;
+            s_run[v * n_keys + k] = at;
+            at += c;
+        }
+    }
+    __syncthreads();
+    int next = b0 + lane < b1 ? (int)key[b0 + lane] : -1;
     for (int64_t base = b0; base < b1; base += 32) {
         const int64_t i = base + lane;
-        const int k = i < b1 ? key[i] : -1;
+        const int k = next;
+        next = i + 32 < b1 ? (int)key[i + 32] : -1;
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, k);
         const int rank = __popc(peers & ((1u << lane) - 1));
         int32_t pos = 0;
         if (k >= 0) pos = run[k] + rank;
         __syncwarp();
         if (k >= 0) {
-            out[pos] = subset ? subset[i] : (int32_t)i;
-            if (out_key) out_key[pos] = k;
+            if (o.out) o.out[pos] = o.subset ? o.subset[i] : (int32_t)i;
+            if (o.out_key) o.out_key[pos] = k;
+            if (o.out_tm) o.out_tm[pos] = o.tm[i];
             if (rank == 0) run[k] += __popc(peers);
         }
         __syncwarp();
     }
+}
+
+// Both passes: blk holds n_keys x blocks counters, tmp the scan's block sums.
+template <typename K>
+int partition(cudaStream_t st, const K *key, int64_t n, int n_keys, int32_t *blk, int32_t *tmp, const PartOut &o,
+              int64_t *launches) {
+    const int64_t nblk = (n + kPartBlock - 1) / kPartBlock;
+    if (nblk == 0) return FEM_OK;
+    // as many warps per block as their key tables fit 48 KB
+    const int room = 48 * 1024 / (4 * n_keys);
+    const int nw = room >= 8 ? 8 : room >= 4 ? 4 : room >= 2 ? 2 : 1;
+    k_part_count<K><<<(unsigned)nblk, 256, n_keys * 4, st>>>(key, n, n_keys, nblk, blk);
+    FEM_TRY(scan_exclusive(st, blk, (int64_t)n_keys * nblk, tmp, nullptr, launches));
+    k_part_scatter<K><<<(unsigned)nblk, nw * 32, nw * n_keys * 4, st>>>(key, n, n_keys, nblk, blk, o);
+    FEM_CUDA_TRY(cudaGetLastError());
+    if (launches) *launches += 2;
+    return FEM_OK;
 }
 
 __global__ void k_gather_keyoff(const int32_t *__restrict__ blk, int n_keys, int64_t nblk,
@@ -1511,97 +1562,63 @@ __global__ void k_group_stats(const int32_t *__restrict__ perm, const int32_t *_
     }
 }
 
-// Per-type event lists of a stream: a stable partition of the event indices
-// by type, then the times gathered in that order.
-__global__ void k_widen_types(const uint16_t *__restrict__ ty, int64_t n, int32_t *__restrict__ key) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        key[i] = ty[i];
-}
-
-__global__ void k_gather_ttime(const int32_t *__restrict__ perm, const int32_t *__restrict__ tm, int64_t n,
-                               int32_t *__restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = tm[perm[i]];
-}
-
-__global__ void k_toff(const int32_t *__restrict__ keyoff, int n_types, int64_t n, int64_t *__restrict__ toff) {
+// Per-type event lists of a stream: a stable partition of the event times
+// (and, where asked for, indices) by type.
+__global__ void k_toff(const int32_t *__restrict__ blk, int64_t nblk, int n_types, int64_t n,
+                       int64_t *__restrict__ toff) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a < n_types) toff[a] = keyoff[a];
+    if (a < n_types) toff[a] = blk[(int64_t)a * nblk];
     if (a == n_types) toff[a] = n;
 }
 
 // The lists and (with pos) their stream positions: what is there already is
-// kept.  The positions are the partition's permutation; without pos it is
-// released with the other temporaries.
+// kept.  Nothing waits for the GPU: the temporaries go back to the context's
+// cache, whose blocks are reused in stream order, and the longest list is the
+// largest frequency, known since the load.
 int stream_bytype(fem_ctx *ctx, fem_stream *s, bool pos) {
     if (s->d_ttime && (!pos || s->d_tpos)) return FEM_OK;
     if (s->n_types > 8192 || s->n > INT32_MAX / 2) return FEM_ERR_INVAL;
     const int64_t n = s->n;
     const bool lists = !s->d_ttime;
     const size_t toff_b = sizeof(int64_t) * (s->n_types + 1), list_b = sizeof(int32_t) * std::max<int64_t>(n, 1);
-    void *p1 = nullptr, *p2 = nullptr, *p3 = nullptr;
-    auto drop = [&](int code) {
-        dev_free(ctx, p1, toff_b);
-        dev_free(ctx, p2, list_b);
-        dev_free(ctx, p3, list_b);
-        return code;
-    };
+    const int n_keys = (int)s->n_types;
+    const int64_t nblk = (n + kPartBlock - 1) / kPartBlock;
+    const size_t tab_b = sizeof(int32_t) * (size_t)std::max<int64_t>(n_keys * nblk, 1);
+    const size_t tmp_b = sizeof(int32_t) * (size_t)((n_keys * nblk) / kScanBlock + 2);
+    void *p1 = nullptr, *p2 = nullptr, *p3 = nullptr, *p4 = nullptr, *p5 = nullptr;
     int st = FEM_OK;
     if (lists) st = dev_alloc(ctx, &p1, toff_b);
     if (st == FEM_OK && lists) st = dev_alloc(ctx, &p2, list_b);
     if (st == FEM_OK && pos) st = dev_alloc(ctx, &p3, list_b);
-    if (st != FEM_OK) return drop(st);
+    if (st == FEM_OK) st = dev_alloc(ctx, &p4, tab_b);
+    if (st == FEM_OK) st = dev_alloc(ctx, &p5, tmp_b);
     int64_t *toff = static_cast<int64_t *>(p1);
-    int32_t *ttime = static_cast<int32_t *>(p2);
-    const int n_keys = (int)s->n_types;
-    const int64_t nblk = std::max<int64_t>(1, (n + kPartBlock - 1) / kPartBlock);
-    const int64_t tab_n = (int64_t)n_keys * nblk;
-    TmpDev tmp(ctx);
-    int32_t *key, *perm = static_cast<int32_t *>(p3), *blk, *stmp, *koff;
-    st = tmp.get(&key, std::max<int64_t>(n, 1));
-    if (st == FEM_OK && !pos) st = tmp.get(&perm, std::max<int64_t>(n, 1));
-    if (st == FEM_OK) st = tmp.get(&blk, tab_n);
-    if (st == FEM_OK) st = tmp.get(&stmp, tab_n / kScanBlock + 2);
-    if (st == FEM_OK) st = tmp.get(&koff, n_keys + 1);
-    if (st != FEM_OK) return drop(st);
+    int32_t *blk = static_cast<int32_t *>(p4);
     cudaStream_t cs = ctx->stream;
-    auto build = [&]() -> int {
-        if (n > 0) {
-            const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, 8 * ctx->n_sm);
-            k_widen_types<<<g, 256, 0, cs>>>(s->d_type, n, key);
-            k_part_count<<<(unsigned)nblk, 256, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk);
-            FEM_TRY(scan_exclusive(cs, blk, tab_n, stmp, nullptr, nullptr));
-            k_part_scatter<<<(unsigned)nblk, 32, n_keys * 4, cs>>>(key, n, n_keys, nblk, blk, nullptr, perm, nullptr);
-            if (lists) {
-                k_gather_keyoff<<<(n_keys + 255) / 256, 256, 0, cs>>>(blk, n_keys, nblk, koff);
-                k_gather_ttime<<<g, 256, 0, cs>>>(perm, s->d_time, n, ttime);
-                k_toff<<<(n_keys + 1 + 255) / 256, 256, 0, cs>>>(koff, n_keys, n, toff);
-            }
-        } else if (lists) {
-            FEM_CUDA_TRY(cudaMemsetAsync(toff, 0, toff_b, cs));
-        }
-        FEM_CUDA_TRY(cudaGetLastError());
-        if (!lists) return FEM_OK;
-        // longest per-type list (sizes the per-warp buffers of local tracking)
-        std::vector<int64_t> toff_h(s->n_types + 1, 0);
-        FEM_CUDA_TRY(cudaMemcpyAsync(toff_h.data(), toff, toff_b, cudaMemcpyDeviceToHost, cs));
-        FEM_CUDA_TRY(cudaStreamSynchronize(cs));
-        s->max_list = 0;
-        for (uint32_t a = 0; a < s->n_types; ++a) s->max_list = std::max(s->max_list, toff_h[a + 1] - toff_h[a]);
-        return FEM_OK;
-    };
-    st = build();
+    if (st == FEM_OK && n > 0) {
+        PartOut o{nullptr, static_cast<int32_t *>(p3), nullptr, s->d_time, static_cast<int32_t *>(p2)};
+        st = partition(cs, s->d_type, n, n_keys, blk, static_cast<int32_t *>(p5), o, nullptr);
+        if (st == FEM_OK && lists)
+            k_toff<<<(n_keys + 1 + 255) / 256, 256, 0, cs>>>(blk, nblk, n_keys, n, toff);
+    } else if (st == FEM_OK && lists && cudaMemsetAsync(toff, 0, toff_b, cs) != cudaSuccess) {
+        st = FEM_ERR_CUDA;
+    }
+    if (st == FEM_OK && cudaGetLastError() != cudaSuccess) st = FEM_ERR_CUDA;
+    dev_free(ctx, p4, tab_b);
+    dev_free(ctx, p5, tmp_b);
     if (st != FEM_OK) {
-        cudaStreamSynchronize(cs);
-        return drop(st);
+        dev_free(ctx, p1, toff_b);
+        dev_free(ctx, p2, list_b);
+        dev_free(ctx, p3, list_b);
+        return st;
     }
     if (lists) {
         s->d_toff = toff;
-        s->d_ttime = ttime;
+        s->d_ttime = static_cast<int32_t *>(p2);
         s->bytes += toff_b + sizeof(int32_t) * n;
     }
     if (pos) {
-        s->d_tpos = perm;
+        s->d_tpos = static_cast<int32_t *>(p3);
         s->bytes += sizeof(int32_t) * n;
     }
     return FEM_OK;
@@ -1874,10 +1891,8 @@ static int group_pairs(CountCall &cc, int32_t *d_perm, int64_t ns, bool *use, do
     if (join >= kPairMaxJoin) return FEM_OK;
     for (int w = 0; w < (n_recs > 1 ? 4 : 3); ++w) {
         track_pair_keys(st, ctx->n_sm, gi, w, key);
-        k_part_count<<<(unsigned)nblk, 256, n_keys[w] * 4, st>>>(key, ns, n_keys[w], nblk, blk);
-        FEM_TRY(scan_exclusive(st, blk, (int64_t)n_keys[w] * nblk, stmp, nullptr, &cc.stats.kernel_launches));
-        k_part_scatter<<<(unsigned)nblk, 32, n_keys[w] * 4, st>>>(key, ns, n_keys[w], nblk, blk, gi.slot2cand,
-                                                                  perm[w & 1], nullptr);
+        FEM_TRY(partition(st, key, ns, n_keys[w], blk, stmp,
+                          PartOut{gi.slot2cand, perm[w & 1], nullptr, nullptr, nullptr}, &cc.stats.kernel_launches));
         gi.slot2cand = perm[w & 1];
     }
     FEM_CUDA_TRY(cudaGetLastError());
@@ -2023,16 +2038,14 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     pa.status = ctx->d_status;
     if (n_work > 0) {
         k_prep<<<(unsigned)nprep, pb, 0, ctx->stream>>>(pa);
-        k_part_count<<<(unsigned)nblk, 256, n_keys * 4, ctx->stream>>>(d_key, n_work, n_keys, nblk, d_blk);
-        FEM_TRY(scan_exclusive(ctx->stream, d_blk, tab_n, d_scan_tmp, nullptr, &cc.stats.kernel_launches));
-        k_part_scatter<<<(unsigned)nblk, 32, n_keys * 4, ctx->stream>>>(d_key, n_work, n_keys, nblk, d_blk,
-                                                                        subset, d_perm, d_slotkey);
+        FEM_TRY(partition(ctx->stream, d_key, n_work, n_keys, d_blk, d_scan_tmp,
+                          PartOut{subset, d_perm, d_slotkey, nullptr, nullptr}, &cc.stats.kernel_launches));
         k_gather_keyoff<<<(n_keys + 255) / 256, 256, 0, ctx->stream>>>(d_blk, n_keys, nblk, d_keyoff);
         unsigned long long *units = reinterpret_cast<unsigned long long *>(mb + o_units);
         k_group_stats<<<(unsigned)((n_work + 127) / 128), 128, 0, ctx->stream>>>(
             d_perm, d_slotkey, n_work, n_recs, cc.offs, cc.types, reinterpret_cast<const RecInfo *>(mb + o_ri), units,
             units + kBuckets);
-        cc.stats.kernel_launches += 5;
+        cc.stats.kernel_launches += 3;
         FEM_CUDA_TRY(cudaGetLastError());
     }
     std::vector<int32_t> key_off(n_keys + 1, 0);

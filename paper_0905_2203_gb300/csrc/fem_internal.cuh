@@ -32,6 +32,10 @@ constexpr uint32_t kDensUnknown = 0xFFFFFFFFu;
 // Device status bits (ctx->d_status).
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusInval = 2;
+// Status words of a context: [0] the bits above, [1] a load's validation
+// result, [kStatusInfo ..] a load's summary (k_load_info).
+constexpr int kStatusWords = 8;
+constexpr int kStatusInfo = 4;
 
 // Record meta bits.
 constexpr int kMetaRingOverflow = 1 << 8;
@@ -234,7 +238,7 @@ struct fem_stream {
     int64_t *d_toff = nullptr;    // per-type event lists (built on first use): offsets [n_types + 1]
     int32_t *d_ttime = nullptr;   // times grouped by type, ascending within a type [n]
     int32_t *d_tpos = nullptr;    // stream position of every list entry [n] (built on request)
-    int64_t max_list = 0;         // longest per-type list (set with the lists)
+    int64_t max_list = 0;         // longest per-type list (the largest frequency)
     // Per-type time index (built on first use, after the lists): cells of
     // 2^tshift ticks from t_first; d_tidx[a * (tcells + 1) + c] is the
     // position in type a's list of its first event at or after
