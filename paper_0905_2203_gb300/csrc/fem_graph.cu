@@ -33,6 +33,8 @@ namespace {
 
 constexpr int kRingCap = 32;      // largest shared-memory ring in the graph path
 constexpr int kMaxPerRec = 4096;  // finest segmentation of a recording
+constexpr int64_t kMaxCap = 1 << 24;  // largest candidate capacity of a level
+constexpr int kManyRecs = 8;              // recordings of a call whose graph is sized for them all
 constexpr int64_t kFusedCap = 16384;  // largest level capacity for the single-block join / threshold
 
 // Counters per level: [0] candidates counted C, [1] frequent F, [2] flags,
@@ -1301,11 +1303,14 @@ struct Level2In {
 }  // namespace
 
 // Runs levels first..max_size through the cached (or newly captured) graph.
-static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const std::vector<int32_t> &blo,
-                     const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr,
-                     const std::vector<int32_t> &lo_vals, int max_size, int first, bool prepass, int64_t cap_min,
-                     const Level2In *in2, TailResult *out, bool *used) {
+// *grow: a level had more candidates than the graph's capacity and nothing
+// else went wrong; the next call captures a larger one.
+static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const std::vector<int32_t> &blo,
+                          const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr,
+                          const std::vector<int32_t> &lo_vals, int max_size, int first, bool prepass, int64_t cap_min,
+                          const Level2In *in2, TailResult *out, bool *used, bool *grow) {
     *used = false;
+    *grow = false;
     const int n_recs = (int)recs.size();
     for (auto *s : recs)
         if (s->n_types > 8192 || s->n > INT32_MAX / 2) return FEM_OK;
@@ -1318,12 +1323,22 @@ static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
     int64_t cap = 4096;
     auto hint = ctx->graph_cap.find(key);
     const int64_t want = std::max<int64_t>(cap_min, hint != ctx->graph_cap.end() ? hint->second : 0);
-    while (cap < want && cap < (1 << 24)) cap <<= 1;
+    while (cap < want && cap < kMaxCap) cap <<= 1;
     if (cap < want) return FEM_OK;
+    // Several recordings: a quarter of all ordered pairs x bins to begin with
+    // (within 2^20; about 800 bytes a candidate), so that level 2 seldom
+    // overflows and the deepest level needs one larger capture at most; one
+    // recording starts at 4096, where the single-block kernels do its levels.
+    const int64_t cap_need = cap;
+    if (n_recs >= kManyRecs) {
+        int64_t pairs = 0;
+        for (auto *s : recs) pairs += (int64_t)s->n_types * (s->n_types - 1) * (int64_t)blo.size();
+        while (cap < pairs / 4 && cap < (1 << 20)) cap <<= 1;
+    }
     GraphTail *g = nullptr;
     track_release(ctx);
     auto it = ctx->graphs.find(key);
-    if (it != ctx->graphs.end() && it->second->cap >= cap &&
+    if (it != ctx->graphs.end() && it->second->cap >= cap_need &&
         (!it->second->track ||
          (it->second->tbuf == ctx->track.p &&
           ctx->track.cap >= track_buf_bytes(it->second->track_nblocks, it->second->track_cap)))) {
@@ -1335,19 +1350,25 @@ static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
             ctx->graphs.erase(it);
         }
         if (ctx->graphs.size() >= 4) graph_cache_clear(ctx);
-        std::unique_ptr<GraphTail> ng(new GraphTail());
-        ng->ctx = ctx;
-        ng->key = key;
-        ng->recs = recs;
-        ng->n_recs = n_recs;
-        ng->max_size = max_size;
-        ng->first = first;
-        ng->prepass = prepass;
-        ng->jb_on = jb_on;
-        ng->coarse = coarse;
-        ng->coarse_min = 0;
-        ng->cap = cap;
-        const int st = build_graph(ng.get(), blo, bhi, thr, lo_vals);
+        int st = FEM_OK;
+        std::unique_ptr<GraphTail> ng;
+        for (;;) {
+            ng.reset(new GraphTail());
+            ng->ctx = ctx;
+            ng->key = key;
+            ng->recs = recs;
+            ng->n_recs = n_recs;
+            ng->max_size = max_size;
+            ng->first = first;
+            ng->prepass = prepass;
+            ng->jb_on = jb_on;
+            ng->coarse = coarse;
+            ng->coarse_min = 0;
+            ng->cap = cap;
+            st = build_graph(ng.get(), blo, bhi, thr, lo_vals);
+            if (st != FEM_ERR_NOMEM || cap == cap_need) break;
+            cap = cap_need;  // no room for the guess
+        }
         if (st == FEM_ERR_NOMEM || st == FEM_ERR_INVAL) return FEM_OK;  // not applicable: host path
         if (st != FEM_OK) return st;
         g = ng.release();
@@ -1384,17 +1405,20 @@ static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
     const int64_t *coff = reinterpret_cast<const int64_t *>(ho + g->lay.o_coff);
     const int64_t *coff2 = reinterpret_cast<const int64_t *>(ho + g->lay.o_coff2);
     const unsigned long long *rel = reinterpret_cast<const unsigned long long *>(ho + g->lay.o_rel);
-    bool flagged = false;
+    bool flagged = false, other = false;
     int64_t need = 0;
     for (int N = std::max(first, 2); N <= max_size; ++N) {
         const int32_t *c = &ctr[(size_t)N * kCtr];
         if (c[2] != 0 || c[3] != 0) flagged = true;
+        if ((c[2] & ~(kFlagCap | kFlagFreq)) != 0 || c[3] != 0) other = true;
         if (c[2] & kFlagCap) need = std::max<int64_t>(need, (int64_t)c[5] + 1);
         if (c[2] & kFlagFreq) need = std::max<int64_t>(need, 2 * g->cap);
     }
     if (flagged) {
-        // redo on the host path; a capacity overflow grows the next capture
+        // a capacity overflow grows the next capture, for several recordings
+        // at once; anything else is redone on the host path
         if (need > 0) ctx->graph_cap[key] = std::max<int64_t>(need, 2 * g->cap);
+        *grow = !other && need > 0 && need <= kMaxCap && n_recs >= kManyRecs;
         return FEM_OK;
     }
     float gms = 0.f;
@@ -1448,6 +1472,22 @@ static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
         if ((N >= 2 && c[0] == 0) || Fn == 0) break;
     }
     *used = true;
+    return FEM_OK;
+}
+
+// Captures and runs until every level's candidates fit (several recordings):
+// another capture costs less than the host-driven path, and each overflow at
+// least doubles the capacity.
+static int run_graph(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const std::vector<int32_t> &blo,
+                     const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr,
+                     const std::vector<int32_t> &lo_vals, int max_size, int first, bool prepass, int64_t cap_min,
+                     const Level2In *in2, TailResult *out, bool *used) {
+    for (int i = 0; i < 12; ++i) {
+        bool grow = false;
+        FEM_TRY(run_graph_once(ctx, recs, blo, bhi, thr, lo_vals, max_size, first, prepass, cap_min, in2, out, used,
+                               &grow));
+        if (!grow) break;
+    }
     return FEM_OK;
 }
 

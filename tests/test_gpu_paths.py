@@ -165,3 +165,32 @@ def test_inner_nodes_by_entries(fb, ctx, n, t_max):
         ctx.reset_tuning()
     assert np.array_equal(got, want), np.nonzero(got != want)[0][:5]
     st.free()
+
+
+def test_many_recordings_capture_again_when_a_level_overflows(fb, ctx):
+    """Eight recordings in which every ordered pair survives level 2, four
+    times what the first capture holds: the call captures a larger graph and
+    finishes in it, with the host-driven path's results."""
+    n_types, bins = 32, [(0, 50), (50, 100), (100, 150), (150, 200)]
+    st = [ctx.load_stream(*synth.tiny_random_stream(0xCB0 + i, 40_000 + 1000 * i, n_types, 400_000), n_types)
+          for i in range(8)]
+    thr = [100] * 8
+
+    def run():
+        res = ctx.mine_levelwise(st, bins, thr, 2)
+        out = [res.level(r, N) for r in range(8) for N in (1, 2)]
+        stats = res.stats()
+        res.free()
+        return out, stats
+
+    a, sa = run()
+    ctx.set_tuning(level_graph=-1)
+    try:
+        h, _ = run()
+    finally:
+        ctx.reset_tuning()
+    assert a == h
+    assert sum(len(c) for _, c in h[1::2]) > 8 * n_types * (n_types - 1)
+    assert sa["graph_tails"] == 1
+    for s in st:
+        s.free()
