@@ -610,9 +610,10 @@ extern "C" int fem_ctx_memory(const fem_ctx *ctx, size_t *used, size_t *budget) 
 // ---------------------------------------------------------------------------
 // C ABI: streams.
 int fem::load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t *times, int64_t n,
-                              uint32_t n_types, int ptr_is_device, fem_stream **out) {
+                              uint32_t n_types, int ptr_is_device, fem_stream **out, const LoadHead *head) {
     if (!ctx || !out || n < 0 || n_types < 1 || n_types > 65536) return FEM_ERR_INVAL;
     if (n > 0 && (!types || !times)) return FEM_ERR_INVAL;
+    if (head) n += head->n;
     if (n > (int64_t)INT32_MAX * 4) return FEM_ERR_INVAL;
     *out = nullptr;
     track_release(ctx);
@@ -640,8 +641,12 @@ int fem::load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t
     s->d_time = static_cast<int32_t *>(p2);
     s->d_freq = static_cast<uint32_t *>(p3);
     s->bytes = (sizeof(uint16_t) + sizeof(int32_t)) * cap + sizeof(uint32_t) * n_types;
-    if (copy_in(ctx, s->d_type, types, sizeof(uint16_t) * n, ptr_is_device) != FEM_OK ||
-        copy_in(ctx, s->d_time, times, sizeof(int32_t) * n, ptr_is_device) != FEM_OK)
+    const int64_t nh = head ? head->n : 0;
+    if (nh > 0 && (copy_in(ctx, s->d_type, head->types, sizeof(uint16_t) * nh, 1) != FEM_OK ||
+                   copy_in(ctx, s->d_time, head->times, sizeof(int32_t) * nh, 1) != FEM_OK))
+        return fail(FEM_ERR_CUDA);
+    if (copy_in(ctx, s->d_type + nh, types, sizeof(uint16_t) * (n - nh), ptr_is_device) != FEM_OK ||
+        copy_in(ctx, s->d_time + nh, times, sizeof(int32_t) * (n - nh), ptr_is_device) != FEM_OK)
         return fail(FEM_ERR_CUDA);
     k_fill_pad<<<64, 256, 0, ctx->stream>>>(s->d_type, s->d_time, n, cap);
     cudaMemsetAsync(s->d_freq, 0, sizeof(uint32_t) * n_types, ctx->stream);

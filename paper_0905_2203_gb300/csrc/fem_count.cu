@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kStitchWarps * 32)
              const int32_t *__restrict__ slot2cand, const uint32_t *__restrict__ cand_rec, int slot_begin,
              int n_slots, uint32_t *__restrict__ counts, int32_t *fb_list, int *fb_count,
              const int32_t *d_n_slots = nullptr, int max_P = INT32_MAX, const uint8_t *skip = nullptr,
-             const int *d_maxP = nullptr, int direct_p1 = 0) {
+             const int *d_maxP = nullptr, int direct_p1 = 0, int32_t *entry = nullptr) {
     const int lane = threadIdx.x & 31;
     // direct_p1: the counting kernel wrote the counts of unsegmented
     // episodes itself (no records); nothing to do when no recording is cut
@@ -524,7 +524,8 @@ __global__ void __launch_bounds__(kStitchWarps * 32)
         warp_compose(f, lane);
         const bool any_bad = __shfl_sync(0xFFFFFFFFu, (int)f.bad, 0) != 0;
         const bool any_ovf = __shfl_sync(0xFFFFFFFFu, (int)f.ovf, 0) != 0;
-        int32_t x = INT32_MIN;  // before the first occurrence
+        // before the first occurrence, or (appended events) the last end kept
+        int32_t x = entry ? entry[cand] : INT32_MIN;
         uint32_t total = 0;
         if (!any_bad && !any_ovf)
             lanemap_apply(f, x, total);  // lane 0's map of the whole episode
@@ -534,6 +535,9 @@ __global__ void __launch_bounds__(kStitchWarps * 32)
             if (any_bad) {
                 const int q = atomicAdd(fb_count, 1);
                 fb_list[q] = cand;
+            } else if (entry) {
+                counts[cand] += total;
+                entry[cand] = x;
             } else {
                 counts[cand] = total;
             }
@@ -1006,12 +1010,13 @@ int scan_exclusive(cudaStream_t st, int32_t *data, int64_t m, int32_t *tmp, int3
 // recording cut into 130 segments.
 constexpr int kSegThreads = 256;
 
+// `base` is added to every boundary (a part of a recording that starts there).
 __global__ void __launch_bounds__(kSegThreads) k_segments(const int32_t *__restrict__ tm, int64_t n, int P,
-                                                          int64_t *__restrict__ seg) {
+                                                          int64_t *__restrict__ seg, int64_t base = 0) {
     __shared__ unsigned long long s_best[kSegThreads / 32];
     const int p = blockIdx.x;
     if (p == 0 || p == P) {
-        if (threadIdx.x == 0) seg[p] = p == 0 ? 0 : n;
+        if (threadIdx.x == 0) seg[p] = base + (p == 0 ? 0 : n);
         return;
     }
     const int64_t nom = (int64_t)((__int128)n * p / P);
@@ -1039,7 +1044,7 @@ __global__ void __launch_bounds__(kSegThreads) k_segments(const int32_t *__restr
     int64_t b = best ? hi + 1 - (int64_t)(uint32_t)best : nom;
     if ((best >> 32) == 0)
         while (b < n && b > 0 && tm[b] == tm[b - 1]) ++b;
-    seg[p] = b;
+    seg[p] = base + b;
 }
 
 int stream_segments(fem_ctx *ctx, fem_stream *s, int P, const int64_t **seg) {
@@ -2831,6 +2836,107 @@ static int count_entry(fem_ctx *ctx, const fem_stream *const *recs, int n_recs, 
     cc.stats.count_kernel_ms = cc.count_ms;
     cc.stats.total_ms = (now_s() - t0) * 1e3;
     ctx->last = cc.stats;
+    return FEM_OK;
+}
+
+// Appended events: 1-node episodes (cand[n_slots ..]) gain their type's new
+// events; the relevant events of all are summed up for the statistics.
+__global__ void k_append_n1(const int32_t *__restrict__ cand, int n_slots, int n, const int64_t *__restrict__ offs,
+                            const uint16_t *__restrict__ types, const uint32_t *__restrict__ freq,
+                            const int32_t *__restrict__ tail_cnt, uint32_t *__restrict__ counts,
+                            unsigned long long *relevant) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long rel = 0;
+    if (i < n) {
+        const int c = cand[i];
+        const int64_t o = offs[c], e = offs[c + 1];
+        for (int64_t k = o; k < e; ++k) rel += freq[types[k]];
+        if (i >= n_slots) counts[c] += freq[types[o]] - (uint32_t)tail_cnt[types[o]];
+    }
+    for (int d = 16; d > 0; d >>= 1) rel += __shfl_down_sync(0xFFFFFFFFu, rel, d);
+    if ((threadIdx.x & 31) == 0 && rel) atomicAdd(relevant, rel);
+}
+
+int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCount &c, fem_stats *stats, bool *used) {
+    *used = false;
+    cudaStream_t st = ctx->stream;
+    track_release(ctx);
+    const int64_t m = fs->n, n_new = m - n_tail;
+    // events of one type in the longest span (see few_by_segments)
+    const double span = std::max(1.0, (double)fs->t_last - (double)fs->t_first);
+    const double in_span = std::min((double)m, (double)m * (double)c.sumhi / span);
+    const int64_t want = std::max<int64_t>(1, (int64_t)((double)n_new / std::max((double)kTrackMinSeg, 8.0 * in_span)));
+    const bool wide = in_span / (double)fs->n_types > kFewMaxPerSpan;
+    if (n_new >= kPltMinEvents && c.n_slots <= kPltMaxCands && (wide || (double)want < kFewMinSegments)) return FEM_OK;
+    const int sb = stream_tindex(ctx, fs);
+    if (sb == FEM_ERR_NOMEM) return FEM_OK;
+    FEM_TRY(sb);
+    // about four items per resident warp; at most kStitchSplit segments, so
+    // that one warp composes an episode's records
+    const int full = track_blocks(ctx->n_sm);
+    int P = (int)std::min<int64_t>(want, kStitchSplit);
+    P = (int)std::max<int64_t>(1, std::min<int64_t>(P, (int64_t)4 * full * kTrackWarps / std::max(c.n_slots, 1) + 1));
+    if (wide) P = 1;  // (the first segment's entry value is known: one class, nothing to run out of)
+    const int64_t items = (int64_t)c.n_slots * P;
+    int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(full, (items + kTrackWarps - 1) / kTrackWarps));
+    const size_t free_b = track_room(ctx);
+    while (blocks > 1 && track_buf_bytes(blocks, fs->max_list) > free_b / 4) blocks = (blocks + 1) / 2;
+    if (track_buf_bytes(blocks, fs->max_list) + (size_t)items * kRecWords * 4 > free_b / 2) return FEM_OK;
+    void *pb = nullptr, *pr = nullptr, *pt = nullptr;
+    // table: [queue][RecInfo][segment starts]
+    if (track_lists(ctx, track_buf_bytes(blocks, fs->max_list), &pb) != FEM_OK ||
+        scratch(ctx, kSlotRecords, (size_t)std::max<int64_t>(items, 1) * kRecWords * 4, &pr) != FEM_OK ||
+        scratch(ctx, kSlotRecTab, 512 + sizeof(int64_t) * (kStitchSplit + 1), &pt) != FEM_OK)
+        return FEM_OK;
+    FEM_CUDA_TRY(cudaMemsetAsync(c.fb_count, 0, sizeof(int), st));
+    FEM_CUDA_TRY(cudaMemsetAsync(c.relevant, 0, 8, st));
+    cudaEventRecord(ctx->ev0, st);
+    if (c.n_slots > 0) {
+        char *tab = static_cast<char *>(pt);
+        int64_t *seg = reinterpret_cast<int64_t *>(tab + 512);
+        RecInfo ri{};
+        ri.type = fs->d_type;
+        ri.time = fs->d_time;
+        ri.n = m;
+        ri.seg = seg;
+        ri.P = P;
+        ri.freq = fs->d_freq;
+        recinfo_lists(ri, fs);
+        RecInfo *d_ri = reinterpret_cast<RecInfo *>(tab + 256);
+        static_assert(sizeof(RecInfo) <= 256, "RecInfo fits its place in the table");
+        FEM_CUDA_TRY(cudaMemcpyAsync(d_ri, &ri, sizeof(ri), cudaMemcpyHostToDevice, st));
+        k_segments<<<P + 1, kSegThreads, 0, st>>>(fs->d_time + n_tail, n_new, P, seg, n_tail);
+        TrackArgs ta{};
+        ta.rinfo = d_ri;
+        ta.n_recs = 1;
+        ta.n_items = items;
+        ta.offs = c.offs;
+        ta.ctypes = c.types;
+        ta.clo = c.lo;
+        ta.chi = c.hi;
+        ta.slot2cand = c.slots;
+        ta.queue = reinterpret_cast<unsigned long long *>(tab);
+        ta.buf = static_cast<int32_t *>(pb);
+        ta.cap = std::max<int64_t>(fs->max_list, 1);
+        ta.rec = static_cast<int32_t *>(pr);
+        ta.last_mode = ctx->tuning.track_last;
+        ta.prev = c.prev;
+        ta.tail_cnt = c.tail_cnt;
+        FEM_TRY(launch_track(st, blocks, ta));
+        k_stitch<<<(c.n_slots + kStitchWarps - 1) / kStitchWarps, kStitchWarps * 32, 0, st>>>(
+            ta.rec, d_ri, c.slots, nullptr, 0, c.n_slots, c.counts, c.fb_list, c.fb_count, nullptr, INT32_MAX, nullptr,
+            nullptr, 0, c.prev);
+    }
+    cudaEventRecord(ctx->ev1, st);
+    const int nc = c.n_slots + c.n_singles;
+    k_append_n1<<<(nc + 255) / 256, 256, 0, st>>>(c.slots, c.n_slots, nc, c.offs, c.types, fs->d_freq, c.tail_cnt,
+                                                  c.counts, c.relevant);
+    FEM_CUDA_TRY(cudaGetLastError());
+    stats->kernel_launches += 5;
+    stats->sparse_launches += 1;
+    stats->candidates_counted += nc;
+    stats->counted_episode_events += (double)nc * (double)m;
+    *used = true;
     return FEM_OK;
 }
 

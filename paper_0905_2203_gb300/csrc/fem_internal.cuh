@@ -125,6 +125,11 @@ struct TrackArgs {
     const int32_t *rorder;
     int last_mode;               // node steps: 0 by the shorter side, 1 by events, 2 by entries
     int pair;                    // groups share their first two nodes (else all but the last)
+    // Appended events (null elsewhere): per candidate the last end kept
+    // before the first segment, and per type the recording's leading events
+    // whose ends were offered before.
+    const int32_t *prev;
+    const int32_t *tail_cnt;
 };
 // Inputs of track_groups: the slots (slot2cand, live count on the device or
 // n_slots_cap), the candidate CSR, per-candidate recordings, the launch's
@@ -384,6 +389,26 @@ int count_plt(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const int64_t
               bool relaxed, uint32_t *d_counts, fem_stats *stats, float *kernel_ms, int variant,
               const PltSession *sess = nullptr);
 
+// Counting continued over appended events by the warp-per-item kernel: the
+// recording fs is a retained tail of n_tail events followed by the new ones.
+struct AppendCount {
+    const int64_t *offs;         // candidates (device CSR)
+    const uint16_t *types;
+    const int32_t *lo, *hi;
+    const int32_t *slots;        // the multi-node ones [n_slots], then the
+    int n_slots, n_singles;      // 1-node ones [n_singles]
+    int64_t sumhi;               // largest sum of an episode's upper bounds
+    const int32_t *tail_cnt;     // tail events per type
+    uint32_t *counts;            // added to
+    int32_t *prev;               // last kept ends, updated
+    int32_t *fb_list;            // candidates that ran out of entry classes: neither is changed
+    int *fb_count;               // (zeroed here)
+    unsigned long long *relevant;  // relevant events of all candidates (zeroed here)
+};
+// *used = false (nothing launched): the spans hold too many events of a type
+// to cut the recording, or the lists have no room.  Does not wait.
+int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCount &c, fem_stats *stats, bool *used);
+
 // Persistent grid of the local-tracking kernel on this device (blocks), the
 // bytes of its per-warp buffers, and its launch (queue reset + kernel).
 int track_blocks(int n_sm);
@@ -542,8 +567,14 @@ void graph_cache_clear(fem_ctx *ctx);
 void graph_cache_forget(fem_ctx *ctx, const fem_stream *s);
 // Stream load without taking the context lock (caller holds it or owns the
 // context exclusively).
+// Events in two parts: np device-resident ones, then n.
+struct LoadHead {
+    const uint16_t *types;
+    const int32_t *times;
+    int64_t n;
+};
 int load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t *times, int64_t n, uint32_t n_types,
-                         int ptr_is_device, fem_stream **out);
+                         int ptr_is_device, fem_stream **out, const LoadHead *head = nullptr);
 void stream_free_unlocked(fem_stream *s);
 // Exclusive scan of m int32 in place; tmp holds ceil(m / 1024) entries.
 int scan_exclusive(cudaStream_t st, int32_t *data, int64_t m, int32_t *tmp, int32_t *total, int64_t *launches);

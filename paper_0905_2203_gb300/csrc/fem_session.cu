@@ -7,12 +7,17 @@
 // it kept last.  So a session keeps, per episode, the count and the time of
 // the last kept end, plus the tail of the stream that a new end can still
 // reach back to: the events at or after t_last - max sum(hi).  An append
-// counts, by node-by-node local tracking (fem_plt.cu), the tail followed by
-// the new events, takes only the ends among the new events, and starts
-// the greedy from the stored last end.  Ends inside the tail cannot be kept
+// counts the tail followed by the new events by local tracking, one warp per
+// (episode, segment of the new events) (fem_track.cu; grid-wide, fem_plt.cu,
+// where spans are too wide to cut), takes only the ends among the new events,
+// and starts the greedy from the stored last end.  The tail's counts per type
+// stay on the device, so an append waits for the GPU twice, for the
+// validation and for the new tail's length: ten appends of 100k events with
+// 256 episodes take 2.0 ms, 9.0 with grid-wide tracking throughout.  Ends inside the tail cannot be kept
 // again: their latest start is at most the stored last end (each was either
 // kept, moving the last end to its own time, or refused for that reason).
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -31,26 +36,33 @@ struct fem_session {
     uint16_t *d_tail_type = nullptr; // retained tail
     int32_t *d_tail_time = nullptr;
     int64_t n_tail = 0, tail_cap = 0;
-    std::vector<int64_t> tail_cnt;   // tail events per type
+    int32_t *d_tail_cnt = nullptr;   // tail events per type: two sets, `cur` in use,
+    int cur = 0;                     // the other written by an append
+    int32_t *d_info = nullptr;       // the next tail's start, overflowed candidates, relevant events (64 bits)
+    int32_t *d_fb = nullptr;         // candidates that overflowed [n_cand]
+    int32_t *d_slots = nullptr;      // multi-node candidates, then 1-node ones [n_cand]
+    int n_slots = 0;                 // multi-node candidates
     int64_t seen = 0;                // events appended so far
 };
 
 namespace fem {
 namespace {
 
-// First index with time >= cut (one thread).
-__global__ void k_lower_bound(const int32_t *__restrict__ tm, int64_t n, int64_t cut, int64_t *out) {
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)tm[mid] < cut) lo = mid + 1; else hi = mid;
-    }
-    *out = lo;
-}
-
-__global__ void k_type_hist(const uint16_t *__restrict__ ty, int64_t n, unsigned long long *__restrict__ h) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&h[ty[i]], 1ull);
+// The tail that later occurrences can reach back into: info[0] = its first
+// event (time >= cut), tail_cnt[a] = its events of type a (one block).
+__global__ void k_session_tail(const int32_t *__restrict__ tm, int64_t n, int64_t cut,
+                               const int64_t *__restrict__ toff, const int32_t *__restrict__ ttime, uint32_t n_types,
+                               int32_t *__restrict__ tail_cnt, int32_t *__restrict__ info) {
+    auto first = [cut](const int32_t *v, int64_t lo, int64_t hi) {
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int64_t)v[mid] < cut) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    if (threadIdx.x == 0) info[0] = (int32_t)first(tm, 0, n);
+    for (uint32_t a = threadIdx.x; a < n_types; a += blockDim.x)
+        tail_cnt[a] = (int32_t)(toff[a + 1] - first(ttime, toff[a], toff[a + 1]));
 }
 
 void session_free_buffers(fem_session *s) {
@@ -62,6 +74,10 @@ void session_free_buffers(fem_session *s) {
     dev_free(ctx, s->d_hi, 4 * ne);
     dev_free(ctx, s->d_counts, 4 * std::max<int64_t>(s->n_cand, 1));
     dev_free(ctx, s->d_prev, 4 * std::max<int64_t>(s->n_cand, 1));
+    dev_free(ctx, s->d_tail_cnt, 8 * (size_t)s->n_types);
+    dev_free(ctx, s->d_info, 16);
+    dev_free(ctx, s->d_fb, 4 * std::max<int64_t>(s->n_cand, 1));
+    dev_free(ctx, s->d_slots, 4 * std::max<int64_t>(s->n_cand, 1));
     if (s->tail_cap) {
         dev_free(ctx, s->d_tail_type, 2 * s->tail_cap);
         dev_free(ctx, s->d_tail_time, 4 * s->tail_cap);
@@ -125,15 +141,22 @@ extern "C" int fem_session_create(fem_ctx *ctx, const fem_cands *c, uint32_t n_t
     s->n_cand = n;
     s->n_nodes = n_nodes;
     s->span_max = span_max;
-    s->tail_cnt.assign(n_types, 0);
+    std::vector<int32_t> slots;
+    for (int64_t i = 0; i < n; ++i)
+        if (offs[i + 1] - offs[i] > 1) slots.push_back((int32_t)i);
+    s->n_slots = (int)slots.size();
+    for (int64_t i = 0; i < n; ++i)
+        if (offs[i + 1] - offs[i] == 1) slots.push_back((int32_t)i);
     const int64_t ne = std::max<int64_t>(n_edges, 1), nc = std::max<int64_t>(n, 1);
-    void *p[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    const size_t sz[6] = {size_t(8 * (n + 1)), size_t(2 * std::max<int64_t>(n_nodes, 1)), size_t(4 * ne),
-                          size_t(4 * ne), size_t(4 * nc), size_t(4 * nc)};
+    constexpr int kBufs = 10;
+    void *p[kBufs] = {};
+    const size_t sz[kBufs] = {size_t(8 * (n + 1)), size_t(2 * std::max<int64_t>(n_nodes, 1)), size_t(4 * ne),
+                              size_t(4 * ne), size_t(4 * nc), size_t(4 * nc), size_t(8) * n_types, 16,
+                              size_t(4 * nc), size_t(4 * nc)};
     int st = FEM_OK;
-    for (int i = 0; i < 6 && st == FEM_OK; ++i) st = dev_alloc(ctx, &p[i], sz[i]);
+    for (int i = 0; i < kBufs && st == FEM_OK; ++i) st = dev_alloc(ctx, &p[i], sz[i]);
     if (st != FEM_OK) {
-        for (int i = 0; i < 6; ++i)
+        for (int i = 0; i < kBufs; ++i)
             if (p[i]) dev_free(ctx, p[i], sz[i]);
         delete s;
         return st;
@@ -144,13 +167,20 @@ extern "C" int fem_session_create(fem_ctx *ctx, const fem_cands *c, uint32_t n_t
     s->d_hi = static_cast<int32_t *>(p[3]);
     s->d_counts = static_cast<uint32_t *>(p[4]);
     s->d_prev = static_cast<int32_t *>(p[5]);
+    s->d_tail_cnt = static_cast<int32_t *>(p[6]);
+    s->d_info = static_cast<int32_t *>(p[7]);
+    s->d_fb = static_cast<int32_t *>(p[8]);
+    s->d_slots = static_cast<int32_t *>(p[9]);
     std::vector<int32_t> prev(nc, INT32_MIN);
     st = copy_in(ctx, s->d_offs, offs.data(), 8 * (n + 1), 0);
     if (st == FEM_OK && n_nodes > 0) st = copy_in(ctx, s->d_types, ty.data(), 2 * n_nodes, 0);
     if (st == FEM_OK && n_edges > 0) st = copy_in(ctx, s->d_lo, lo.data(), 4 * n_edges, 0);
     if (st == FEM_OK && n_edges > 0) st = copy_in(ctx, s->d_hi, hi.data(), 4 * n_edges, 0);
     if (st == FEM_OK) st = copy_in(ctx, s->d_prev, prev.data(), 4 * nc, 0);
-    if (st == FEM_OK && cudaMemsetAsync(s->d_counts, 0, 4 * nc, ctx->stream) != cudaSuccess) st = FEM_ERR_CUDA;
+    if (st == FEM_OK && n > 0) st = copy_in(ctx, s->d_slots, slots.data(), 4 * n, 0);
+    if (st == FEM_OK && (cudaMemsetAsync(s->d_counts, 0, 4 * nc, ctx->stream) != cudaSuccess ||
+                         cudaMemsetAsync(s->d_tail_cnt, 0, 8 * (size_t)n_types, ctx->stream) != cudaSuccess))
+        st = FEM_ERR_CUDA;
     if (st == FEM_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess) st = FEM_ERR_CUDA;
     if (st != FEM_OK) {
         session_free_buffers(s);
@@ -175,87 +205,99 @@ extern "C" int fem_session_append(fem_session *s, const uint16_t *types, const i
     // tail followed by the new events, validated as one recording (order and
     // repeated (type, time) pairs across the join included)
     fem_stream *fs = nullptr;
-    {
-        TmpDev tmp(ctx);
-        uint16_t *bt;
-        int32_t *bm;
-        FEM_TRY(tmp.get(&bt, m));
-        FEM_TRY(tmp.get(&bm, m));
-        if (s->n_tail > 0) {
-            FEM_CUDA_TRY(cudaMemcpyAsync(bt, s->d_tail_type, 2 * s->n_tail, cudaMemcpyDeviceToDevice, st));
-            FEM_CUDA_TRY(cudaMemcpyAsync(bm, s->d_tail_time, 4 * s->n_tail, cudaMemcpyDeviceToDevice, st));
-        }
-        FEM_TRY(copy_in(ctx, bt + s->n_tail, types, 2 * n, ptr_is_device));
-        FEM_TRY(copy_in(ctx, bm + s->n_tail, times, 4 * n, ptr_is_device));
-        FEM_TRY(load_stream_unlocked(ctx, bt, bm, m, s->n_types, 1, &fs));
-    }
+    const LoadHead head{s->d_tail_type, s->d_tail_time, s->n_tail};
+    FEM_TRY(load_stream_unlocked(ctx, types, times, n, s->n_types, ptr_is_device, &fs, &head));
     fem_stats stats{};
     float ms = 0.f;
-    int rc = FEM_OK;
-    if (s->n_cand > 0) {
-        std::vector<int32_t> work(s->n_cand);
-        for (int64_t i = 0; i < s->n_cand; ++i) work[i] = (int32_t)i;
-        PltSession ps{&s->tail_cnt, s->d_prev};
-        std::vector<fem_stream *> recs{fs};
-        rc = count_plt(ctx, recs, s->d_offs, s->d_types, s->d_lo, s->d_hi, nullptr, work, false, s->d_counts, &stats,
-                       &ms, 0, &ps);
+    bool used = false;
+    const int32_t *tail_cnt = s->d_tail_cnt + (size_t)s->cur * s->n_types;
+    int32_t *tail_next = s->d_tail_cnt + (size_t)(1 - s->cur) * s->n_types;
+    int rc = stream_bytype(ctx, fs);
+    if (rc == FEM_OK && s->n_cand > 0) {
+        AppendCount ac{};
+        ac.offs = s->d_offs;
+        ac.types = s->d_types;
+        ac.lo = s->d_lo;
+        ac.hi = s->d_hi;
+        ac.slots = s->d_slots;
+        ac.n_slots = s->n_slots;
+        ac.n_singles = (int)s->n_cand - s->n_slots;
+        ac.sumhi = s->span_max;
+        ac.tail_cnt = tail_cnt;
+        ac.counts = s->d_counts;
+        ac.prev = s->d_prev;
+        ac.fb_list = s->d_fb;
+        ac.fb_count = s->d_info + 1;
+        ac.relevant = reinterpret_cast<unsigned long long *>(s->d_info + 2);
+        rc = count_appended(ctx, fs, s->n_tail, ac, &stats, &used);
     }
     // the new tail: events at or after t_last - max sum(hi)
-    int64_t cut_idx = 0;
-    std::vector<unsigned long long> h(s->n_types, 0);
+    int32_t info[4] = {};
     if (rc == FEM_OK) {
-        TmpDev tmp(ctx);
-        int64_t *d_idx;
-        unsigned long long *d_h;
-        rc = tmp.get(&d_idx, 1);
-        if (rc == FEM_OK) rc = tmp.get(&d_h, s->n_types);
+        k_session_tail<<<1, 256, 0, st>>>(fs->d_time, m, (int64_t)fs->t_last - s->span_max, fs->d_toff, fs->d_ttime,
+                                          s->n_types, tail_next, s->d_info);
+        if (cudaGetLastError() != cudaSuccess ||
+            cudaMemcpyAsync(info, s->d_info, sizeof info, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            rc = FEM_ERR_CUDA;
+    }
+    // grid-wide tracking for the candidates that ran out of entry classes, or
+    // for all
+    std::vector<int32_t> work;
+    if (rc == FEM_OK && used) {
+        unsigned long long rel = 0;
+        std::memcpy(&rel, info + 2, 8);
+        stats.relevant_events += (double)rel;
+        if (cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1) != cudaSuccess) cudaGetLastError();
+        work.resize(info[1]);
+        stats.fallback_recounts += info[1];
+        stats.candidates_counted -= info[1];
+        if (info[1] > 0) rc = copy_out(ctx, work.data(), s->d_fb, 4 * (size_t)info[1], 0);
+    } else if (rc == FEM_OK) {
+        work.resize(s->n_cand);
+        for (int64_t i = 0; i < s->n_cand; ++i) work[i] = (int32_t)i;
+    }
+    if (rc == FEM_OK && !work.empty()) {
+        std::vector<int32_t> tc(s->n_types, 0);
+        rc = copy_out(ctx, tc.data(), tail_cnt, 4 * (size_t)s->n_types, 0);
+        if (rc == FEM_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = FEM_ERR_CUDA;
+        const std::vector<int64_t> tail(tc.begin(), tc.end());
+        const PltSession ps{&tail, s->d_prev};
+        if (rc == FEM_OK)
+            rc = count_plt(ctx, {fs}, s->d_offs, s->d_types, s->d_lo, s->d_hi, nullptr, work, false, s->d_counts,
+                           &stats, &ms, 0, &ps);
+    }
+    const int64_t cut_idx = info[0], nt = m - cut_idx;
+    if (rc == FEM_OK && nt > s->tail_cap) {
+        const int64_t cap = std::max<int64_t>(nt, 2 * s->tail_cap);
+        void *p1 = nullptr, *p2 = nullptr;
+        rc = dev_alloc(ctx, &p1, 2 * cap);
         if (rc == FEM_OK) {
-            k_lower_bound<<<1, 1, 0, st>>>(fs->d_time, m, (int64_t)fs->t_last - s->span_max, d_idx);
-            if (cudaMemcpyAsync(&cut_idx, d_idx, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess)
-                rc = FEM_ERR_CUDA;
-        }
-        const int64_t nt = m - cut_idx;
-        if (rc == FEM_OK && nt > s->tail_cap) {
-            const int64_t cap = std::max<int64_t>(nt, 2 * s->tail_cap);
-            void *p1 = nullptr, *p2 = nullptr;
-            rc = dev_alloc(ctx, &p1, 2 * cap);
-            if (rc == FEM_OK) {
-                rc = dev_alloc(ctx, &p2, 4 * cap);
-                if (rc != FEM_OK) dev_free(ctx, p1, 2 * cap);
-            }
-            if (rc == FEM_OK) {
-                cudaStreamSynchronize(st);
-                if (s->tail_cap) {
-                    dev_free(ctx, s->d_tail_type, 2 * s->tail_cap);
-                    dev_free(ctx, s->d_tail_time, 4 * s->tail_cap);
-                }
-                s->d_tail_type = static_cast<uint16_t *>(p1);
-                s->d_tail_time = static_cast<int32_t *>(p2);
-                s->tail_cap = cap;
-            }
+            rc = dev_alloc(ctx, &p2, 4 * cap);
+            if (rc != FEM_OK) dev_free(ctx, p1, 2 * cap);
         }
         if (rc == FEM_OK) {
-            cudaMemsetAsync(d_h, 0, 8 * s->n_types, st);
-            cudaMemcpyAsync(s->d_tail_type, fs->d_type + cut_idx, 2 * nt, cudaMemcpyDeviceToDevice, st);
-            cudaMemcpyAsync(s->d_tail_time, fs->d_time + cut_idx, 4 * nt, cudaMemcpyDeviceToDevice, st);
-            if (nt > 0) {
-                const unsigned gsz = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nt + 255) / 256, 4 * ctx->n_sm));
-                k_type_hist<<<gsz, 256, 0, st>>>(s->d_tail_type, nt, d_h);
+            if (s->tail_cap) {
+                dev_free(ctx, s->d_tail_type, 2 * s->tail_cap);
+                dev_free(ctx, s->d_tail_time, 4 * s->tail_cap);
             }
-            if (cudaGetLastError() != cudaSuccess ||
-                cudaMemcpyAsync(h.data(), d_h, 8 * s->n_types, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess)
-                rc = FEM_ERR_CUDA;
-            else
-                s->n_tail = nt;
+            s->d_tail_type = static_cast<uint16_t *>(p1);
+            s->d_tail_time = static_cast<int32_t *>(p2);
+            s->tail_cap = cap;
         }
+    }
+    if (rc == FEM_OK) {
+        if (cudaMemcpyAsync(s->d_tail_type, fs->d_type + cut_idx, 2 * nt, cudaMemcpyDeviceToDevice, st) !=
+                cudaSuccess ||
+            cudaMemcpyAsync(s->d_tail_time, fs->d_time + cut_idx, 4 * nt, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            rc = FEM_ERR_CUDA;
+        s->n_tail = nt;
+        s->cur = 1 - s->cur;
     }
     stream_free_unlocked(fs);
     // A failure after counting leaves the session unusable for exact counts:
     // the caller gets the error and should recreate it.
     if (rc != FEM_OK) return rc;
-    for (uint32_t a = 0; a < s->n_types; ++a) s->tail_cnt[a] = (int64_t)h[a];
     s->seen += n;
     stats.kernel_launches += 2;
     stats.count_kernel_ms = ms;

@@ -85,6 +85,15 @@ struct Classes {
         open = 1;
         flags = 0;
     }
+    // The entry value is known: one class that holds for every value.
+    __device__ __forceinline__ void init_known(int32_t x) {
+        init();
+        thr = INT32_MAX;
+        prev = x;
+        ncls = 1;
+        live = 1u;
+        open = 0;
+    }
     // An end at t with latest start L (both uniform).
     __device__ __forceinline__ void end(int32_t t, int32_t L, int32_t Tp, int lane) {
         if (((live >> lane) & 1u) && L > prev) {
@@ -568,10 +577,16 @@ __global__ void __launch_bounds__(kTrackWarps * 32, kTrackMaxBlocksPerSm) k_coun
                     if (k == depth) m_pre = m;
                 }
             }
-            st.init();
+            const bool known = a.prev && p == 0;
+            if (known) st.init_known(a.prev[c]); else st.init();
             if (m > 0) {
                 int cb = 0, ce = 0;
                 range(a.ctypes[oc + N - 1], cb, ce);
+                // appended events: the retained tail's ends were offered before
+                if (known) {
+                    const uint32_t E = a.ctypes[oc + N - 1];
+                    cb = min(ce, max(cb, (int)ri.toff[E] + a.tail_cnt[E]));
+                }
                 const int n_ev = ce - cb;
                 const int32_t lo_l = a.relaxed ? 0 : a.clo[ec + N - 2], hi_l = a.chi[ec + N - 2];
                 if (by_entries(m, n_ev)) {

@@ -194,3 +194,37 @@ def test_many_recordings_capture_again_when_a_level_overflows(fb, ctx):
     assert sa["graph_tails"] == 1
     for s in st:
         s.free()
+
+
+@pytest.mark.parametrize("chunk", [1, 700, 40_000])
+@pytest.mark.parametrize("wide", [1, 12, 200])
+def test_session_counts_by_segments_and_grid_wide(fb, ctx, wide, chunk):
+    """Appends counted in segments (edges of up to 20 ticks; with 40,000-event
+    chunks several segments), with episodes that run out of entry classes
+    (240), and grid-wide or unsegmented (4000): after every append that is
+    checked the counts are the oracle's on the prefix."""
+    n_types = 6
+    ty, tm = synth.tiny_random_stream(77, 90_000 if chunk > 1 else 2_000, n_types, 600_000 if chunk > 1 else 9_000)
+    r = synth.Rng(78, wide)
+    n_cand = 150
+    sizes = r.integers(1, 5, n_cand)
+    offs = np.zeros(n_cand + 1, np.int64)
+    offs[1:] = np.cumsum(sizes)
+    ct = r.integers(0, n_types - 1, int(offs[-1])).astype(np.uint16)
+    lo = (r.integers(0, 9, int(offs[-1]) - n_cand) * wide).astype(np.int32)
+    hi = (lo + wide * r.integers(1, 11, lo.size)).astype(np.int32)
+    sess = ctx.session(fb.Cands(offs, ct, lo, hi), n_types)
+    cuts = [0, 300, 301] + list(range(301 + chunk, min(len(ty), 301 + 40 * chunk), chunk)) + [len(ty)]
+    try:
+        for i, (a, b) in enumerate(zip(cuts[:-1], cuts[1:])):
+            sess.append(ty[a:b], tm[a:b])
+            if i < 4 or b == len(ty):
+                want = oracle_counts(ty[:b], tm[:b], offs, ct, lo, hi)
+                got = sess.counts().astype(np.int64)
+                assert np.array_equal(got, want), (b, np.nonzero(got != want)[0][:5])
+        assert want.max() > 0
+        # relevant events of the last append: its recording's, tail included
+        seen, _ = sess.info()
+        assert seen == len(ty) and ctx.last_stats()["relevant_events"] > 0
+    finally:
+        sess.close()
