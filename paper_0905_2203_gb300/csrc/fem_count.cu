@@ -29,7 +29,6 @@
 #include <algorithm>
 #include <cstring>
 #include <numeric>
-#include <set>
 #include <vector>
 
 #include "fem_internal.cuh"
@@ -1824,7 +1823,9 @@ struct CountCall {
     const int32_t *hi = nullptr;
     const uint32_t *cand_rec = nullptr;  // null = all recording 0
     uint32_t *counts = nullptr;          // device, n_cand
-    std::vector<int32_t> lo_vals;        // distinct lo values (host)
+    std::vector<int32_t> lo_vals;        // distinct lo values (host), see need_lo_vals
+    bool lo_known = false;               // lo_vals is set
+    int64_t n_edges = 0;                 // entries of lo
     int mode = 0;                        // 0 exact, 1 plain, 2 relaxed
     double seg_div = 1.0;                // fallback rounds divide the segment count
     bool force_tiled = false;            // last fallback round: tiled kernel, one segment
@@ -1835,7 +1836,21 @@ struct CountCall {
 };
 
 static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int force_segments);
+// The distinct lower bounds size the per-episode kernels' rings; local
+// tracking does without (collecting those of 200k episodes took 8 ms).
+static int need_lo_vals(CountCall &cc) {
+    if (cc.lo_known) return FEM_OK;
+    std::vector<int32_t> lo(cc.n_edges);
+    if (cc.n_edges > 0) FEM_TRY(copy_out(cc.ctx, lo.data(), cc.lo, 4 * cc.n_edges, 0));
+    FEM_CUDA_TRY(cudaStreamSynchronize(cc.ctx->stream));
+    std::sort(lo.begin(), lo.end());
+    lo.erase(std::unique(lo.begin(), lo.end()), lo.end());
+    cc.lo_vals = lo;
+    cc.lo_known = true;
+    return FEM_OK;
+}
 static int count_grid_wide(CountCall &cc, std::vector<int32_t> &work, int variant);
+static int recount_overflowed(CountCall &cc, std::vector<int32_t> &hsub);
 
 // Automatic grid-wide local tracking (fem_plt.cu): at most this many episodes
 // over a recording of at least this many events (see run_count).
@@ -1957,6 +1972,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     }
     const int n_keys = kBuckets * n_recs;
     // --- density tables and per-recording tables
+    if (!track) FEM_TRY(need_lo_vals(cc));
     std::vector<int32_t> lov = cc.lo_vals;
     if (cc.mode == 2) lov = {0};
     if (lov.empty()) lov = {0};
@@ -2623,39 +2639,45 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     }
     cc.stats.candidates_counted += n_work - fbc;
     if (fbc > 0) {
-        // Exact recount of the episodes whose machines ran out of entry
-        // classes at some segment boundary.
-        cc.stats.fallback_recounts += fbc;
         void *p_sub = nullptr;
         FEM_TRY(scratch(ctx, kSlotScanTmp, sizeof(int32_t) * fbc, &p_sub));
         FEM_CUDA_TRY(cudaMemcpyAsync(p_sub, fb_list, sizeof(int32_t) * fbc, cudaMemcpyDeviceToDevice, ctx->stream));
-        // the sub-call reuses the scratch slots, so keep its subset elsewhere
         std::vector<int32_t> hsub(fbc);
         FEM_CUDA_TRY(cudaMemcpyAsync(hsub.data(), p_sub, sizeof(int32_t) * fbc, cudaMemcpyDeviceToHost, ctx->stream));
         FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-        if (cc.plt_ok) return count_grid_wide(cc, hsub, 0);
-        void *p_keep = nullptr;
-        FEM_TRY(dev_alloc(ctx, &p_keep, sizeof(int32_t) * fbc));
-        cudaMemcpyAsync(p_keep, hsub.data(), sizeof(int32_t) * fbc, cudaMemcpyHostToDevice, ctx->stream);
-        // Each round divides the segment count by 8 (fewer boundaries, so
-        // fewer entry classes); after a few rounds a single segment remains,
-        // which never needs more than one class.
-        // The last round runs the tiled kernel on one segment, where neither
-        // entry classes nor rings (sized from the stream's densities) can
-        // overflow.
-        const double saved = cc.seg_div;
-        const bool saved_ft = cc.force_tiled;
-        cc.seg_div *= 8.0;
-        const bool last = cc.seg_div >= 4096.0;
-        if (last) cc.force_tiled = true;
-        const int st = count_core(cc, static_cast<int32_t *>(p_keep), fbc, last ? 1 : 0);
-        cc.seg_div = saved;
-        cc.force_tiled = saved_ft;
-        cudaStreamSynchronize(ctx->stream);
-        dev_free(ctx, p_keep, sizeof(int32_t) * fbc);
-        return st;
+        return recount_overflowed(cc, hsub);
     }
     return FEM_OK;
+}
+
+// Exact recount of the episodes whose machines ran out of entry classes at
+// some segment boundary.
+static int recount_overflowed(CountCall &cc, std::vector<int32_t> &hsub) {
+    fem_ctx *ctx = cc.ctx;
+    const int fbc = (int)hsub.size();
+    cc.stats.fallback_recounts += fbc;
+    if (cc.plt_ok) return count_grid_wide(cc, hsub, 0);
+    // the sub-call reuses the scratch slots, so keep its subset elsewhere
+    void *p_keep = nullptr;
+    FEM_TRY(dev_alloc(ctx, &p_keep, sizeof(int32_t) * fbc));
+    cudaMemcpyAsync(p_keep, hsub.data(), sizeof(int32_t) * fbc, cudaMemcpyHostToDevice, ctx->stream);
+    // Each round divides the segment count by 8 (fewer boundaries, so
+    // fewer entry classes); after a few rounds a single segment remains,
+    // which never needs more than one class.
+    // The last round runs the tiled kernel on one segment, where neither
+    // entry classes nor rings (sized from the stream's densities) can
+    // overflow.
+    const double saved = cc.seg_div;
+    const bool saved_ft = cc.force_tiled;
+    cc.seg_div *= 8.0;
+    const bool last = cc.seg_div >= 4096.0;
+    if (last) cc.force_tiled = true;
+    const int st = count_core(cc, static_cast<int32_t *>(p_keep), fbc, last ? 1 : 0);
+    cc.seg_div = saved;
+    cc.force_tiled = saved_ft;
+    cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, p_keep, sizeof(int32_t) * fbc);
+    return st;
 }
 
 // Counts the candidates `work` by grid-wide local tracking (fem_plt.cu).
@@ -2724,8 +2746,7 @@ static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int fo
     return count_core(cc, subset, n_sub, force_segments);
 }
 
-// Copies (or aliases) the candidate CSR to the device and collects the
-// distinct lower bounds.
+// Copies (or aliases) the candidate CSR to the device.
 static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, const uint32_t *rec_id,
                             int n_recs) {
     const int64_t n = c->n_cand;
@@ -2748,19 +2769,15 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
     }
     if (n_nodes < n || n_nodes > (int64_t)n * FEM_MAX_NODES) return FEM_ERR_INVAL;
     const int64_t n_edges = n_nodes - n;
-    std::vector<int32_t> lo_h;
+    cc.n_edges = n_edges;
     if (c->ptr_is_device) {
         cc.offs = c->offs;
         cc.types = c->types;
         cc.lo = c->lo;
         cc.hi = c->hi;
-        lo_h.resize(n_edges);
-        if (n_edges > 0) {
-            FEM_CUDA_TRY(cudaMemcpyAsync(lo_h.data(), c->lo, 4 * n_edges, cudaMemcpyDeviceToHost, ctx->stream));
-            if (few) {
-                hi_h.resize(n_edges);
-                FEM_CUDA_TRY(cudaMemcpyAsync(hi_h.data(), c->hi, 4 * n_edges, cudaMemcpyDeviceToHost, ctx->stream));
-            }
+        if (few && n_edges > 0) {
+            hi_h.resize(n_edges);
+            FEM_CUDA_TRY(cudaMemcpyAsync(hi_h.data(), c->hi, 4 * n_edges, cudaMemcpyDeviceToHost, ctx->stream));
             FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
         }
         if (rec_id) cc.cand_rec = rec_id;
@@ -2778,7 +2795,6 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
         cc.types = static_cast<uint16_t *>(p2);
         cc.lo = static_cast<int32_t *>(p3);
         cc.hi = static_cast<int32_t *>(p4);
-        lo_h.assign(c->lo, c->lo + n_edges);
         if (rec_id) {
             for (int64_t i = 0; i < n; ++i)
                 if (rec_id[i] >= (uint32_t)n_recs) return FEM_ERR_INVAL;
@@ -2788,8 +2804,6 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
             cc.cand_rec = static_cast<uint32_t *>(p5);
         }
     }
-    std::set<int32_t> los(lo_h.begin(), lo_h.end());
-    cc.lo_vals.assign(los.begin(), los.end());
     if (few) {
         const int64_t *o = c->ptr_is_device ? offs_h.data() : c->offs;
         const int32_t *h = c->ptr_is_device ? hi_h.data() : c->hi;
@@ -2801,6 +2815,250 @@ static int stage_candidates(fem_ctx *ctx, const fem_cands *c, CountCall &cc, con
             cc.sumhi = std::max(cc.sumhi, sum);
         }
     }
+    return FEM_OK;
+}
+
+// ---------------------------------------------------------------------------
+// One recording, candidates in host memory, no launch overridden: the usual
+// call.  Preparation, counting and statistics of the general driver (twelve
+// launches, a dozen small copies, two host reads) take 140 us whatever the
+// work; here the candidates and the recording's table go up in one copy, one
+// kernel checks them and marks the prefix groups, one block numbers the items,
+// and the counts come back with the statistics in one copy and one wait.
+// A malformed candidate leaves no items and no slots (status word).
+struct QuickInfo {
+    int status, fb_count;
+    unsigned long long relevant;
+    int64_t n_items;
+    unsigned long long queue;
+    int64_t ibase[2];
+    int32_t gfirst, n_live;
+};
+static_assert(sizeof(QuickInfo) <= 64, "QuickInfo fits its place");
+
+// Larger sets may be worth sorting (group_pairs) and take the general driver.
+constexpr int64_t kQuickMaxCands = kPairMinSlots - 1;
+
+// Checks candidate i, adds up its relevant events, makes it slot i and marks
+// the start of a prefix group (see k_track_group_flags).
+__global__ void k_quick_prep(int n, const int64_t *__restrict__ offs, const uint16_t *__restrict__ ctypes,
+                             const int32_t *__restrict__ clo, const int32_t *__restrict__ chi, uint32_t n_types,
+                             const uint32_t *__restrict__ freq, int32_t *__restrict__ slot2cand,
+                             int32_t *__restrict__ flag, QuickInfo *info) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long rel = 0;
+    if (i < n) {
+        const int64_t o = offs[i];
+        const int N = (int)(offs[i + 1] - o);
+        bool bad = false;
+        for (int k = 0; k < N; ++k) {
+            const uint32_t a = ctypes[o + k];
+            if (a >= n_types) {
+                bad = true;
+                break;
+            }
+            rel += freq[a];
+            if (k < N - 1) bad = bad || clo[o - i + k] < 0 || clo[o - i + k] >= chi[o - i + k];
+        }
+        if (bad) atomicOr(&info->status, kStatusInval);
+        bool f = i % kTrackGroupMax == 0;
+        if (!f) {
+            const int64_t b = offs[i - 1];
+            f = (int)(o - b) != N || N < 3;
+            for (int k = 0; k < N - 1 && !f; ++k) f = ctypes[o + k] != ctypes[b + k];
+            for (int k = 0; k < N - 2 && !f; ++k)
+                f = clo[o - i + k] != clo[b - i + 1 + k] || chi[o - i + k] != chi[b - i + 1 + k];
+        }
+        flag[i] = f ? 1 : 0;
+        slot2cand[i] = i;
+    }
+    for (int d = 16; d > 0; d >>= 1) rel += __shfl_down_sync(0xFFFFFFFFu, rel, d);
+    if ((threadIdx.x & 31) == 0 && rel) atomicAdd(&info->relevant, rel);
+}
+
+// One block: the groups' first slots and the item count.
+__global__ void __launch_bounds__(1024) k_quick_groups(int n, const int32_t *__restrict__ flag, int P,
+                                                       int32_t *__restrict__ gstart, QuickInfo *info) {
+    __shared__ int32_t wsum[32];
+    __shared__ int32_t s_total;
+    const int per = (n + 1023) / 1024;
+    const int i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
+    int32_t c = 0;
+    for (int i = i0; i < i1; ++i) c += flag[i];
+    const int32_t incl = block_incl_scan(c, wsum);
+    if (threadIdx.x == 1023) s_total = incl;
+    int32_t g = incl - c;
+    for (int i = i0; i < i1; ++i)
+        if (flag[i]) gstart[g++] = i;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const bool ok = info->status == 0;
+        gstart[s_total] = n;
+        info->gfirst = 0;
+        info->ibase[0] = 0;
+        info->ibase[1] = info->n_items = ok ? (int64_t)s_total * P : 0;
+        info->n_live = ok ? n : 0;
+    }
+}
+
+__global__ void k_quick_n1(int n, const int64_t *__restrict__ offs, const uint16_t *__restrict__ ctypes,
+                           const uint32_t *__restrict__ freq, uint32_t *__restrict__ counts, const QuickInfo *info) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n && info->status == 0 && offs[i + 1] - offs[i] == 1) counts[i] = freq[ctypes[offs[i]]];
+}
+
+// *used = false (nothing launched): the general driver counts.
+static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t *counts, int out_is_device, int mode,
+                       CountCall &cc, bool *used) {
+    *used = false;
+    const fem_tuning &tu = ctx->tuning;
+    const int64_t n = c->n_cand;
+    if (c->ptr_is_device || mode == 1 || n > kQuickMaxCands || tu.kernel != 0 || tu.segments != 0 ||
+        tu.lanes_per_cta != 0 || tu.tile_events != 0 || tu.autotune != 0 || !ctx->tune.empty() ||
+        s->n_types > 8192 || s->n > INT32_MAX / 2 || c->offs[0] != 0)
+        return FEM_OK;
+    int64_t n_slots = 0;
+    for (int64_t i = 0; i < n; ++i) {
+        const int64_t N = c->offs[i + 1] - c->offs[i];
+        if (N < 1 || N > FEM_MAX_NODES) return FEM_OK;
+        int64_t sum = 0;
+        for (int64_t e = c->offs[i] - i; e < c->offs[i + 1] - i - 1; ++e) sum += c->hi[e];
+        cc.sumhi = std::max(cc.sumhi, sum);
+        n_slots += N > 1;
+    }
+    cc.plt_ok = n <= kPltMaxCands && s->n >= kPltMinEvents;
+    if (cc.plt_ok && !few_by_segments(cc)) return FEM_OK;
+    track_release(ctx);
+    const int sb = stream_tindex(ctx, s);
+    if (sb == FEM_ERR_NOMEM) return FEM_OK;
+    FEM_TRY(sb);
+    // segments: about four items per resident warp, none shorter than
+    // kTrackMinSeg events or 8 halos (the general driver's rule)
+    const int full = track_blocks(ctx->n_sm);
+    const double desired = 4.0 * full * kTrackWarps;
+    const double seg_len = std::max(1.0, (double)n_slots * (double)s->n / desired);
+    const double span = std::max(1.0, (double)s->t_last - (double)s->t_first);
+    const double halo_ev = (double)s->n * (double)std::max<int64_t>(cc.sumhi, 0) / span;
+    const double min_seg = std::max((double)kTrackMinSeg, 8.0 * halo_ev);
+    const int P = std::min(512, (int)std::max(1.0, std::min((double)s->n / seg_len, (double)s->n / min_seg)));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(full, (n * P + kTrackWarps - 1) / kTrackWarps));
+    const size_t free_b = track_room(ctx);
+    if (track_buf_bytes(blocks, s->max_list) > free_b / 4 || (size_t)(n * P) * kRecWords * 4 > free_b / 4)
+        return FEM_OK;
+    const int64_t nn = c->offs[n], ne = nn - n;
+    // one block: [RecInfo][offs][lo][hi][types][QuickInfo] up, then
+    // [QuickInfo][counts] down, then what stays on the device
+    size_t off = 0;
+    auto carve = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 63) & ~size_t(63);
+        return o;
+    };
+    const size_t o_ri = carve(sizeof(RecInfo)), o_of = carve(8 * (n + 1)), o_lo = carve(4 * ne), o_hi = carve(4 * ne),
+                 o_ty = carve(2 * nn), o_in = carve(64), o_ct = carve(4 * n), o_s2c = carve(4 * n),
+                 o_fl = carve(4 * n), o_gs = carve(4 * (n + 1)), o_fb = carve(4 * n);
+    const size_t up = o_in + 64, down = 64 + 4 * (size_t)n;
+    void *pd = nullptr, *pb = nullptr, *pr = nullptr;
+    if (scratch(ctx, kSlotQuick, off, &pd) != FEM_OK ||
+        track_lists(ctx, track_buf_bytes(blocks, s->max_list), &pb) != FEM_OK ||
+        scratch(ctx, kSlotRecords, (size_t)(n * P) * kRecWords * 4, &pr) != FEM_OK)
+        return FEM_OK;
+    if (ctx->stage_bytes < std::max(up, down)) {
+        if (ctx->stage) cudaFreeHost(ctx->stage);
+        ctx->stage = nullptr;
+        ctx->stage_bytes = 0;
+        const size_t want = std::max<size_t>(std::max(up, down) * 2, 64 << 10);
+        if (cudaMallocHost(&ctx->stage, want) != cudaSuccess) {
+            cudaGetLastError();
+            return FEM_OK;
+        }
+        ctx->stage_bytes = want;
+    }
+    const int64_t *seg = nullptr;
+    FEM_TRY(stream_segments(ctx, s, P, &seg));
+    *used = true;
+    cudaStream_t st = ctx->stream;
+    char *d = static_cast<char *>(pd), *h = static_cast<char *>(ctx->stage);
+    RecInfo ri{s->d_type, s->d_time, s->n, seg, P, 0, 0, s->d_freq};
+    recinfo_lists(ri, s);
+    std::memcpy(h + o_ri, &ri, sizeof ri);
+    std::memcpy(h + o_of, c->offs, 8 * (n + 1));
+    std::memcpy(h + o_lo, c->lo, 4 * ne);
+    std::memcpy(h + o_hi, c->hi, 4 * ne);
+    std::memcpy(h + o_ty, c->types, 2 * nn);
+    std::memset(h + o_in, 0, 64);
+    FEM_CUDA_TRY(cudaMemcpyAsync(d, h, up, cudaMemcpyHostToDevice, st));
+    QuickInfo *info = reinterpret_cast<QuickInfo *>(d + o_in);
+    cc.offs = reinterpret_cast<int64_t *>(d + o_of);
+    cc.types = reinterpret_cast<uint16_t *>(d + o_ty);
+    cc.lo = reinterpret_cast<int32_t *>(d + o_lo);
+    cc.hi = reinterpret_cast<int32_t *>(d + o_hi);
+    cc.counts = reinterpret_cast<uint32_t *>(d + o_ct);
+    int32_t *s2c = reinterpret_cast<int32_t *>(d + o_s2c), *fl = reinterpret_cast<int32_t *>(d + o_fl);
+    int32_t *fb = reinterpret_cast<int32_t *>(d + o_fb);
+    const unsigned g = (unsigned)((n + 127) / 128);
+    k_quick_prep<<<g, 128, 0, st>>>((int)n, cc.offs, cc.types, cc.lo, cc.hi, s->n_types, s->d_freq, s2c, fl, info);
+    k_quick_groups<<<1, 1024, 0, st>>>((int)n, fl, P, reinterpret_cast<int32_t *>(d + o_gs), info);
+    cudaEventRecord(ctx->ev0, st);
+    TrackArgs ta{};
+    ta.rinfo = reinterpret_cast<RecInfo *>(d + o_ri);
+    ta.n_recs = 1;
+    ta.d_n_items = &info->n_items;
+    ta.offs = cc.offs;
+    ta.ctypes = cc.types;
+    ta.clo = cc.lo;
+    ta.chi = cc.hi;
+    ta.slot2cand = s2c;
+    ta.relaxed = mode == 2;
+    ta.queue = &info->queue;
+    ta.buf = static_cast<int32_t *>(pb);
+    ta.cap = std::max<int64_t>(s->max_list, 1);
+    ta.rec = static_cast<int32_t *>(pr);
+    ta.counts = cc.counts;
+    ta.gstart = reinterpret_cast<int32_t *>(d + o_gs);
+    ta.gfirst = &info->gfirst;
+    ta.ibase = info->ibase;
+    ta.last_mode = tu.track_last;
+    FEM_TRY(launch_track(st, blocks, ta, false));
+    if (P > 1) {
+        k_stitch<<<(unsigned)((n + kStitchWarps - 1) / kStitchWarps), kStitchWarps * 32, 0, st>>>(
+            ta.rec, ta.rinfo, s2c, nullptr, 0, (int)n, cc.counts, fb, &info->fb_count, &info->n_live, kStitchSplit);
+        cc.stats.kernel_launches += 1;
+    }
+    if (P > kStitchSplit) {
+        k_stitch_block<<<(unsigned)std::min<int64_t>(n, (int64_t)ctx->n_sm * 4), kStitchBlock, 0, st>>>(
+            ta.rec, ta.rinfo, s2c, nullptr, 0, (int)n, cc.counts, fb, &info->fb_count, &info->n_live, kStitchSplit);
+        cc.stats.kernel_launches += 1;
+    }
+    cudaEventRecord(ctx->ev1, st);
+    if (n_slots < n) {
+        k_quick_n1<<<g, 128, 0, st>>>((int)n, cc.offs, cc.types, s->d_freq, cc.counts, info);
+        cc.stats.kernel_launches += 1;
+    }
+    FEM_CUDA_TRY(cudaGetLastError());
+    FEM_CUDA_TRY(cudaMemcpyAsync(h, d + o_in, out_is_device ? 64 : down, cudaMemcpyDeviceToHost, st));
+    FEM_CUDA_TRY(cudaStreamSynchronize(st));
+    QuickInfo hi;
+    std::memcpy(&hi, h, sizeof hi);
+    if (hi.status) return FEM_ERR_INVAL;
+    cc.stats.kernel_launches += 3;
+    cc.stats.sparse_launches += 1;
+    cc.stats.counted_episode_events += (double)n * (double)s->n;
+    cc.stats.relevant_events += (double)hi.relevant;
+    cc.stats.candidates_counted += n - hi.fb_count;
+    if (cudaEventElapsedTime(&cc.count_ms, ctx->ev0, ctx->ev1) != cudaSuccess) cudaGetLastError();
+    if (hi.fb_count > 0) {
+        std::vector<int32_t> hsub(hi.fb_count);
+        FEM_TRY(copy_out(ctx, hsub.data(), fb, sizeof(int32_t) * hsub.size(), 0));
+        FEM_CUDA_TRY(cudaStreamSynchronize(st));
+        cc.n_edges = ne;
+        FEM_TRY(recount_overflowed(cc, hsub));
+    } else if (!out_is_device) {
+        std::memcpy(counts, h + 64, 4 * (size_t)n);
+        return FEM_OK;
+    }
+    FEM_TRY(copy_out(ctx, counts, cc.counts, 4 * n, out_is_device));
+    FEM_CUDA_TRY(cudaStreamSynchronize(st));
     return FEM_OK;
 }
 
@@ -2825,6 +3083,18 @@ static int count_entry(fem_ctx *ctx, const fem_stream *const *recs, int n_recs, 
         return FEM_OK;
     }
     if (!c->types || !c->lo || !c->hi) return FEM_ERR_INVAL;
+    auto finish = [&]() {
+        cc.stats.episode_events = cc.stats.counted_episode_events;
+        cc.stats.count_kernel_ms = cc.count_ms;
+        cc.stats.total_ms = (now_s() - t0) * 1e3;
+        ctx->last = cc.stats;
+        return FEM_OK;
+    };
+    if (n_recs == 1) {
+        bool used = false;
+        FEM_TRY(count_quick(ctx, cc.recs[0], c, counts, out_is_device, mode, cc, &used));
+        if (used) return finish();
+    }
     FEM_TRY(stage_candidates(ctx, c, cc, n_recs > 1 ? rec_id : nullptr, n_recs));
     void *pc = nullptr;
     FEM_TRY(scratch(ctx, kSlotCounts, 4 * c->n_cand, &pc));
@@ -2832,11 +3102,7 @@ static int count_entry(fem_ctx *ctx, const fem_stream *const *recs, int n_recs, 
     FEM_TRY(run_count(cc, nullptr, c->n_cand, 0));
     FEM_TRY(copy_out(ctx, counts, cc.counts, 4 * c->n_cand, out_is_device));
     FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    cc.stats.episode_events = cc.stats.counted_episode_events;
-    cc.stats.count_kernel_ms = cc.count_ms;
-    cc.stats.total_ms = (now_s() - t0) * 1e3;
-    ctx->last = cc.stats;
-    return FEM_OK;
+    return finish();
 }
 
 // Appended events: 1-node episodes (cand[n_slots ..]) gain their type's new
@@ -2958,6 +3224,7 @@ int count_device(fem_ctx *ctx, const std::vector<fem_stream *> &recs, int64_t n_
     cc.cand_rec = cand_rec;
     cc.counts = counts;
     cc.lo_vals = lo_vals;
+    cc.lo_known = true;
     cc.sumhi = sumhi;
     // `order` (optional) lists every candidate once, in the order the
     // counting kernels should hold them (lane neighbours share types).

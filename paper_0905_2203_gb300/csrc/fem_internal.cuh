@@ -216,6 +216,8 @@ struct fem_ctx {
     std::multimap<size_t, void *> cached;
     size_t cached_bytes = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    void *stage = nullptr;        // pinned staging of small counting calls
+    size_t stage_bytes = 0;
     void *pinned = nullptr;       // mapped host buffer of a destroyed mining graph, for the next one
     size_t pinned_bytes = 0;
 };
@@ -501,14 +503,15 @@ int track_groups(cudaStream_t st, int n_sm, const TrackGroupIn &in, bool grouped
 constexpr int kPairEdgeKeys = 256;
 void track_pair_keys(cudaStream_t st, int n_sm, const TrackGroupIn &in, int which, int32_t *key);
 size_t track_buf_bytes(int blocks, int64_t cap, bool pair = false);
-int launch_track(cudaStream_t st, int blocks, const TrackArgs &a);
+// (reset: zero the work counter first; else it is zero already)
+int launch_track(cudaStream_t st, int blocks, const TrackArgs &a, bool reset = true);
 
 // Scratch slot ids.
 enum Slot : int {
     kSlotCandOffs = 1, kSlotCandTypes, kSlotCandLo, kSlotCandHi, kSlotCandRec,
     kSlotPrep, kSlotPerm, kSlotBucket, kSlotRecords, kSlotSeg, kSlotCounts,
     kSlotFallback, kSlotRings, kSlotDensTab, kSlotScanTmp, kSlotMisc, kSlotRecTab, kSlotDensArgs,
-    kSlotTrackGrp,
+    kSlotTrackGrp, kSlotQuick,
     kSlotMine0 = 64,
 };
 

@@ -771,9 +771,9 @@ size_t track_buf_bytes(int blocks, int64_t cap, bool pair) {
     return (size_t)blocks * kTrackWarps * (pair ? 6 : 4) * (size_t)std::max<int64_t>(cap, 1) * sizeof(int32_t);
 }
 
-int launch_track(cudaStream_t st, int blocks, const TrackArgs &a) {
+int launch_track(cudaStream_t st, int blocks, const TrackArgs &a, bool reset) {
     if (blocks < 1) return FEM_OK;
-    if (cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), st) != cudaSuccess) return FEM_ERR_CUDA;
+    if (reset && cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), st) != cudaSuccess) return FEM_ERR_CUDA;
     k_count_track<<<(unsigned)blocks, kTrackWarps * 32, 0, st>>>(a);
     FEM_CUDA_TRY(cudaGetLastError());
     return FEM_OK;

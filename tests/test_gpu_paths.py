@@ -228,3 +228,49 @@ def test_session_counts_by_segments_and_grid_wide(fb, ctx, wide, chunk):
         assert seen == len(ty) and ctx.last_stats()["relevant_events"] > 0
     finally:
         sess.close()
+
+
+@pytest.mark.parametrize("n_cand", [1, 33, 1025, 16_383, 16_384])
+def test_one_recording_from_host_memory(fb, ctx, n_cand):
+    """The short way of a host call (up to 16,383 episodes) and the general
+    one: sizes 1-16, prefixes shared by runs longer than a group, one and many
+    segments, counts to the host and to the device, the relaxed bound, and a
+    malformed episode at the end refused with the counts untouched."""
+    import torch
+    n_types = 20
+    r = synth.Rng(91, n_cand)
+    sizes = np.repeat(r.integers(1, 16, (n_cand + 99) // 100), 100)[:n_cand]
+    offs = np.zeros(n_cand + 1, np.int64)
+    offs[1:] = np.cumsum(sizes)
+    ct = r.integers(0, n_types - 1, int(offs[-1])).astype(np.uint16)
+    lo = r.integers(0, 3, int(offs[-1]) - n_cand).astype(np.int32) * 10
+    hi = lo + 25
+    for c in range(1, n_cand):  # runs of 100 share all but their last node and edge
+        if c % 100 and sizes[c] > 1:
+            n = int(sizes[c])
+            o, b = int(offs[c]), int(offs[c - 1])
+            ct[o:o + n - 1] = ct[b:b + n - 1]
+            lo[o - c:o - c + n - 2] = lo[b - c + 1:b - c + 1 + n - 2]
+    hi = lo + 25
+    for n_ev, t_max in ((3000, 9000), (60_000, 900_000)):
+        ty, tm = synth.tiny_random_stream(92, n_ev, n_types, t_max)
+        st = ctx.load_stream(ty, tm, n_types)
+        want = oracle_counts(ty, tm, offs, ct, lo, hi)
+        cands = fb.Cands(offs, ct, lo, hi)
+        assert np.array_equal(ctx.count_episodes(st, cands).astype(np.int64), want)
+        out = torch.zeros(n_cand, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        ctx.count_episodes(st, cands, out)
+        assert np.array_equal(out.cpu().numpy().astype(np.int64), want)
+        assert np.array_equal(ctx.upper_bound(st, cands).astype(np.int64),
+                              oracle_counts(ty, tm, offs, ct, np.zeros_like(lo), hi))
+        freq = np.bincount(ty, minlength=n_types)
+        ctx.count_episodes(st, cands)
+        assert ctx.last_stats()["relevant_events"] == freq[ct].sum()
+        bad = ct.copy()
+        bad[-1] = n_types
+        keep = np.full(n_cand, 7, np.uint32)
+        with pytest.raises(fb.FemError) as e:
+            ctx.count_episodes(st, fb.Cands(offs, bad, lo, hi), keep)
+        assert e.value.status == fb.FEM_ERR_INVAL and (keep == 7).all()
+        st.free()
