@@ -1743,7 +1743,7 @@ int launch_count_dev(cudaStream_t st, int nmax, int nodes, int R, const RecInfo 
 int launch_stitch_dev(cudaStream_t st, int nsm, const RecInfo *rinfo, const int32_t *slot2cand,
                       const uint32_t *cand_rec, const int32_t *rec, const int32_t *d_n_slots, int64_t cap_slots,
                       uint32_t *counts, int32_t *fb_list, int *fb_count, const uint8_t *skip, const int *d_maxP,
-                      int direct_p1) {
+                      int direct_p1, int p_limit) {
     // the live segment counts are only known on the device: both stitch
     // kernels run, each taking the episodes on its side of kStitchSplit
     const int64_t gst = std::min<int64_t>((cap_slots + kStitchWarps - 1) / kStitchWarps, (int64_t)std::max(1, nsm) * 8);
@@ -1752,9 +1752,10 @@ int launch_stitch_dev(cudaStream_t st, int nsm, const RecInfo *rinfo, const int3
         k_stitch<<<(unsigned)gst, kStitchWarps * 32, 0, st>>>(rec, rinfo, slot2cand, cand_rec, 0, (int)cap_slots,
                                                             counts, fb_list, fb_count, d_n_slots, kStitchSplit, skip,
                                                             d_maxP, direct_p1);
-        k_stitch_block<<<(unsigned)gsb, kStitchBlock, 0, st>>>(rec, rinfo, slot2cand, cand_rec, 0, (int)cap_slots,
-                                                               counts, fb_list, fb_count, d_n_slots, kStitchSplit,
-                                                               skip, d_maxP);
+        if (p_limit > kStitchSplit)
+            k_stitch_block<<<(unsigned)gsb, kStitchBlock, 0, st>>>(rec, rinfo, slot2cand, cand_rec, 0, (int)cap_slots,
+                                                                   counts, fb_list, fb_count, d_n_slots, kStitchSplit,
+                                                                   skip, d_maxP);
     }
     FEM_CUDA_TRY(cudaGetLastError());
     return FEM_OK;

@@ -382,17 +382,13 @@ __global__ void k_g_levelinfo(const uint32_t *crec, const int32_t *ctr, int N, i
 // Level N = M + 1 in one block: zero the level's counters, check every
 // (alpha, beta) pair of frequent (N-1)-episodes of the same recording for the
 // join (pairs numbered alpha-major, each thread a contiguous run of them),
-// scan, write the candidates in that order, then index and segment the level
-// (for levels whose capacity keeps one block fast; at most kFusedRecs
-// recordings).
+// scan, write the candidates in that order (for levels whose capacity keeps
+// one block fast; at most kFusedRecs recordings).  Returns their number.
 constexpr int kFusedRecs = 1024;
 
-__global__ void __launch_bounds__(1024, 1)
-    k_g_join_fused(const uint16_t *ft, const int32_t *fl, const int32_t *fh, const uint32_t *frec,
-                   const int64_t *foff, const int32_t *ctr_prev, int M, int64_t cap, uint16_t *ct, int32_t *cl,
-                   int32_t *ch, uint32_t *crec, int32_t *ctr, unsigned long long *rel, int64_t *offs, int32_t *iota,
-                   int n_recs, int64_t *coff, RecInfo *ri, int64_t *nthreads, const int32_t *pfine, int32_t *sstep,
-                   int64_t target, int *maxP) {
+__device__ int64_t join_block(const uint16_t *ft, const int32_t *fl, const int32_t *fh, const int64_t *foff, int M,
+                              int64_t cap, uint16_t *ct, int32_t *cl, int32_t *ch, uint32_t *crec, int32_t *ctr,
+                              unsigned long long *rel, int n_recs) {
     __shared__ int64_t s_pp[kFusedRecs + 1];  // pair offsets per recording
     const int N = M + 1;
     {
@@ -442,18 +438,193 @@ __global__ void __launch_bounds__(1024, 1)
         ctr[5] = (int32_t)(total < INT32_MAX ? total : INT32_MAX);
         *rel = 0ull;
     }
-    level_index(C, N, cap, offs, iota, threadIdx.x, blockDim.x);
     __syncthreads();  // crec complete
+    return C;
+}
+
+// The join and the level's index and segmentation (per-episode kernels).
+__global__ void __launch_bounds__(1024, 1)
+    k_g_join_fused(const uint16_t *ft, const int32_t *fl, const int32_t *fh, const int64_t *foff, int M, int64_t cap,
+                   uint16_t *ct, int32_t *cl, int32_t *ch, uint32_t *crec, int32_t *ctr, unsigned long long *rel,
+                   int64_t *offs, int32_t *iota, int n_recs, int64_t *coff, RecInfo *ri, int64_t *nthreads,
+                   const int32_t *pfine, int32_t *sstep, int64_t target, int *maxP) {
+    const int64_t C = join_block(ft, fl, fh, foff, M, cap, ct, cl, ch, crec, ctr, rel, n_recs);
+    level_index(C, M + 1, cap, offs, iota, threadIdx.x, blockDim.x);
     level_info(crec, C, n_recs, coff, ri, nthreads, pfine, sstep, target, maxP);
 }
 
-// The level's threshold in one block: flags, scan, write of the frequent
+// Everything between a level's frequent set and its count launch in one block,
+// for local tracking and levels that one block keeps fast: the join (N >= 3;
+// level 2's candidates are there already), the CSR index, the prefix groups
+// (N >= 3), the segmentation by the largest of them, the segment starts, the
+// item numbering and the work counter.  As eleven launches these took longer
+// than the counting they prepare: a level of a mid-size recording has some
+// twenty candidates (mining 1.07M events, 128 types, six levels: 700 -> 539
+// us; a 5k-event recording, four levels: 360 -> 291 us).
+struct SmallLevel {
+    int N;
+    const uint16_t *ft;              // level N - 1's frequent set (N >= 3)
+    const int32_t *fl, *fh;
+    const int64_t *foff;
+    int64_t cap;
+    uint16_t *ct;
+    int32_t *cl, *ch;
+    uint32_t *crec;
+    int32_t *ctr;
+    unsigned long long *rel;
+    int64_t *offs;
+    int32_t *iota;
+    int n_recs;
+    int64_t *coff;
+    RecInfo *ri;
+    int64_t *nthreads;
+    const int32_t *pfine;
+    int32_t *sstep;
+    int64_t target, cap_threads;
+    int *maxP;
+    const int64_t *segf;             // finest segment starts, and the level's
+    int64_t *segl;
+    const int32_t *rorder;           // item order of the recordings
+    int32_t *gidx, *gstart, *gfirst, *gmax;
+    int64_t *ibase, *n_items;
+    unsigned long long *queue;
+};
+
+__global__ void __launch_bounds__(1024, 1) k_g_level_small(SmallLevel a) {
+    const int N = a.N, n_recs = a.n_recs;
+    const int64_t C = N >= 3 ? join_block(a.ft, a.fl, a.fh, a.foff, N - 1, a.cap, a.ct, a.cl, a.ch, a.crec, a.ctr,
+                                          a.rel, n_recs)
+                             : (int64_t)a.ctr[0];
+    level_index(C, N, a.cap, a.offs, a.iota, threadIdx.x, blockDim.x);
+    if (N >= 3) {
+        // groups: as k_track_group_flags / k_track_group_starts
+        for (int r = threadIdx.x; r < n_recs; r += blockDim.x) a.gmax[r] = 0;
+        const int64_t per = (C + blockDim.x - 1) / blockDim.x;
+        const int64_t i0 = min(C, (int64_t)threadIdx.x * per), i1 = min(C, i0 + per);
+        auto starts = [&](int64_t i) {
+            bool f = i % kTrackGroupMax == 0 || a.crec[i] != a.crec[i - 1];
+            for (int k = 0; k < N - 1 && !f; ++k) f = a.ct[i * N + k] != a.ct[(i - 1) * N + k];
+            for (int k = 0; k < N - 2 && !f; ++k)
+                f = a.cl[i * (N - 1) + k] != a.cl[(i - 1) * (N - 1) + k] ||
+                    a.ch[i * (N - 1) + k] != a.ch[(i - 1) * (N - 1) + k];
+            return f;
+        };
+        int64_t cnt = 0;
+        for (int64_t i = i0; i < i1; ++i) cnt += starts(i);
+        int64_t total = 0;
+        int64_t g = block_excl_scan(cnt, &total);
+        for (int64_t i = i0; i < i1; ++i) {
+            a.gidx[i] = (int32_t)g;  // groups before slot i
+            if (starts(i)) a.gstart[g++] = (int32_t)i;
+        }
+        if (threadIdx.x == 0) {
+            a.gidx[C] = (int32_t)total;
+            a.gstart[total] = (int32_t)C;
+        }
+        __syncthreads();
+        for (int64_t q = threadIdx.x; q < total; q += blockDim.x)
+            atomicMax(a.gmax + a.crec[a.gstart[q]], a.gstart[q + 1] - a.gstart[q]);
+        __syncthreads();
+    }
+    level_info(a.crec, C, n_recs, a.coff, a.ri, a.nthreads, a.pfine, a.sstep, a.target, a.maxP,
+               N >= 3 ? a.gmax : nullptr, a.cap_threads);
+    for (int r = 0; r < n_recs; ++r) {
+        const int P = a.ri[r].P, st = a.sstep[r], pf = a.pfine[r];
+        const int64_t *f = a.segf + (size_t)r * (kMaxPerRec + 1);
+        int64_t *o = a.segl + (size_t)r * (kMaxPerRec + 1);
+        for (int p = threadIdx.x; p <= P; p += blockDim.x) o[p] = f[min(p * st, pf)];
+    }
+    if (threadIdx.x == 0) {  // as k_track_group_recs
+        auto first = [&](int r) -> int64_t {
+            const int64_t sf = r < n_recs ? (int64_t)a.ri[r].slot_first : C;
+            const int64_t c = sf < C ? sf : C;
+            return N >= 3 ? (int64_t)a.gidx[c] : c;
+        };
+        int64_t base = 0;
+        for (int i = 0; i < n_recs; ++i) {
+            const int r = a.rorder[i];
+            const int64_t g0 = first(r), g1 = first(r + 1);
+            a.gfirst[r] = (int32_t)g0;
+            a.ibase[i] = base;
+            base += (g1 - g0) * a.ri[r].P;
+        }
+        a.ibase[n_recs] = base;
+        *a.n_items = base;
+        *a.queue = 0ull;
+    }
+}
+
+// Level 1 in one block (flags, scan, write, per-recording offsets), then level
+// 2's generated pairs per recording.
+__global__ void __launch_bounds__(1024, 1)
+    k_g_l1_small(const RecInfo *ri, const uint32_t *thr, const int64_t *ntpre, int n_recs, int64_t tot, uint16_t *ft,
+                 uint32_t *frec, uint32_t *fcnt, int64_t *foff, int32_t *ctr, unsigned long long *rel, int nb,
+                 int64_t cap2, int64_t *coff2) {
+    const int64_t per = (tot + blockDim.x - 1) / blockDim.x;
+    const int64_t i0 = min(tot, (int64_t)threadIdx.x * per), i1 = min(tot, i0 + per);
+    auto freq = [&](int64_t i, int *r) {
+        *r = seg_of(ntpre, n_recs, i);
+        return ri[*r].freq[i - ntpre[*r]];
+    };
+    int64_t cnt = 0;
+    int r = 0;
+    for (int64_t i = i0; i < i1; ++i) cnt += freq(i, &r) > thr[r];
+    int64_t total = 0;
+    int64_t o = block_excl_scan(cnt, &total);
+    for (int64_t i = i0; i < i1; ++i) {
+        const uint32_t f = freq(i, &r);
+        if (!(f > thr[r])) continue;
+        ft[o] = (uint16_t)(i - ntpre[r]);
+        frec[o] = (uint32_t)r;
+        fcnt[o] = f;
+        ++o;
+    }
+    // (levels 1 and 2 of the counters)
+    if (threadIdx.x < 2 * kCtr) ctr[threadIdx.x] = threadIdx.x == 0 ? (int32_t)tot : threadIdx.x == 1 ? (int32_t)total : 0;
+    if (threadIdx.x < 2) rel[threadIdx.x] = 0ull;
+    __syncthreads();  // frec, ctr complete
+    for (int q = threadIdx.x; q <= n_recs; q += blockDim.x) {
+        int64_t lo = 0, hi = total;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int)frec[mid] < q) lo = mid + 1; else hi = mid;
+        }
+        foff[q] = lo;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int64_t s = 0;
+        coff2[0] = 0;
+        for (int q = 0; q < n_recs; ++q) {
+            const int64_t F = foff[q + 1] - foff[q];
+            s += F >= 2 ? F * (F - 1) * nb : 0;
+            coff2[q + 1] = s;
+        }
+        ctr[kCtr + 4] = (int32_t)(s < INT32_MAX ? s : INT32_MAX);
+        if (s > cap2) ctr[kCtr + 2] |= kFlagGen;
+    }
+}
+
+// The level's threshold in one block (and, with rel, the sum of its relevant
+// events): flags, scan, write of the frequent
 // episodes in candidate order, then the per-recording offsets.
 __global__ void __launch_bounds__(1024, 1)
     k_g_thr_fused(const uint32_t *counts, const uint16_t *ct, const int32_t *cl, const int32_t *ch,
                   const uint32_t *crec, const uint32_t *thr, int N, int64_t cap, uint16_t *ft, int32_t *fl,
-                  int32_t *fh, uint32_t *frec, uint32_t *fcnt, int32_t *ctr, int n_recs, int64_t *foff) {
+                  int32_t *fh, uint32_t *frec, uint32_t *fcnt, int32_t *ctr, int n_recs, int64_t *foff,
+                  const RecInfo *ri, const uint8_t *skip, unsigned long long *rel) {
     const int64_t C = ctr[0];
+    if (rel) {
+        // the counted candidates' relevant events (see k_g_ringcheck)
+        unsigned long long acc = 0;
+        for (int64_t i = threadIdx.x; i < C; i += blockDim.x) {
+            if (skip && skip[i]) continue;
+            const uint32_t *fq = ri[crec[i]].freq;
+            for (int k = 0; k < N; ++k) acc += fq[ct[i * N + k]];
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0 && acc) atomicAdd(rel, acc);
+    }
     const int64_t per = (C + blockDim.x - 1) / blockDim.x;
     const int64_t i0 = min(C, (int64_t)threadIdx.x * per), i1 = min(C, i0 + per);
     int64_t cnt = 0;
@@ -1035,6 +1206,10 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     // levels whose candidate capacity keeps one block fast use the fused
     // single-block join and threshold kernels
     const bool fused = cap <= kFusedCap && n_recs <= kFusedRecs;
+    const bool small = fused && g->track;
+    const bool small1 = small && first == 1 && tot1 <= kFusedCap;
+    int pfine_max = 1;
+    for (int32_t p : pfine_h) pfine_max = std::max(pfine_max, p);
     for (int N = first; N <= L && cst == FEM_OK; ++N) {
         int32_t *cn = g->ctr + (size_t)N * kCtr;
         int64_t *coffN = g->coff + (size_t)N * (n_recs + 1);
@@ -1064,9 +1239,23 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
             return gi;
         };
         bool groups_ready = false;
-        if (!fuse_join) {
+        auto level_small = [&](const FLevel *pf) {
+            const SmallLevel sl{N, pf ? pf->types : nullptr, pf ? pf->lo : nullptr, pf ? pf->hi : nullptr,
+                                pf ? pf->foff : nullptr, cap, ct, cl, ch, crec, cn, g->rel + N, offs, iota, n_recs,
+                                coffN, d_ri, nthreads, g->pfine, g->sstep, g->target, g->cap_threads, g->d_maxP,
+                                g->segf, g->segl, g->rorder, g->tg_gidx, g->tg_gstart, g->tg_gfirst, g->tg_gmax,
+                                g->tg_ibase, g->tg_nitems, reinterpret_cast<unsigned long long *>(g->tqueue)};
+            k_g_level_small<<<1, 1024, 0, st>>>(sl);
+        };
+        if (!fuse_join && !(small1 && N <= 2)) {
             ok(cudaMemsetAsync(cn, 0, sizeof(int32_t) * kCtr, st));
             ok(cudaMemsetAsync(g->rel + N, 0, sizeof(unsigned long long), st));
+        }
+        if (N == 1 && small1) {
+            k_g_l1_small<<<1, 1024, 0, st>>>(d_ri, g->d_thr, d_ntpre, n_recs, tot1, nf.types, nf.rec, nf.counts,
+                                             nf.foff, cn, g->rel + 1, nb, cap2, g->coff2);
+            ok(cudaGetLastError());
+            continue;
         }
         if (N == 1) {
             k_g_l1_flags<<<gb1, 256, 0, st>>>(d_ri, g->d_thr, d_ntpre, n_recs, tot1, pos);
@@ -1080,7 +1269,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
         const int nmax = N <= 2 ? 2 : N <= 4 ? 4 : N <= 8 ? 8 : 16;
         if (N == 2) {
             const FLevel &f1 = g->F[1];
-            k_g_gen2_off<<<1, 32, 0, st>>>(f1.foff, n_recs, nb, cap2, g->coff2, cn);
+            if (!small1) k_g_gen2_off<<<1, 32, 0, st>>>(f1.foff, n_recs, nb, cap2, g->coff2, cn);
             k_g_gen2<<<gb2, 256, 0, st>>>(f1.types, f1.foff, g->coff2, n_recs, d_blo, d_bhi, nb, cap2, gt, glo, ghi,
                                           grec);
             if (g->prepass) {
@@ -1097,26 +1286,23 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
             if (cst == FEM_OK) cst = scan_exclusive(st, pos, cap2 + 1, scan_tmp, nullptr, nullptr);
             k_g_prune_write<<<gb2, 256, 0, st>>>(pos, gt, glo, ghi, grec, cap2, ubp, d_uboff, d_nt, d_blo, d_bhi, nb,
                                                  g->d_thr, cap, ct, cl, ch, crec, cn);
-            k_g_level_index<<<gb, 256, 0, st>>>(cn, N, cap, offs, iota);
-            k_g_levelinfo<<<1, 256, 0, st>>>(crec, cn, N, cap, offs, iota, n_recs, coffN, d_ri, nthreads, g->pfine,
-                                             g->sstep, g->target, g->d_maxP, nullptr, g->cap_threads);
+            if (small) {
+                level_small(nullptr);
+            } else {
+                k_g_level_index<<<gb, 256, 0, st>>>(cn, N, cap, offs, iota);
+                k_g_levelinfo<<<1, 256, 0, st>>>(crec, cn, N, cap, offs, iota, n_recs, coffN, d_ri, nthreads,
+                                                 g->pfine, g->sstep, g->target, g->d_maxP, nullptr, g->cap_threads);
+            }
         } else {
             const int M = N - 1;
             const FLevel &pf = g->F[M];
             int32_t *cp = g->ctr + (size_t)M * kCtr;  // previous level's counters
-            if (fuse_join) {
-                k_g_join_fused<<<1, 1024, 0, st>>>(pf.types, pf.lo, pf.hi, pf.rec, pf.foff, cp, M, cap, ct, cl, ch,
-                                                   crec, cn, g->rel + N, offs, iota, n_recs, coffN, d_ri, nthreads,
-                                                   g->pfine, g->sstep, g->target, g->d_maxP);
-                // local tracking: segment again, allowing for the largest
-                // prefix group
-                if (g->track && cst == FEM_OK) {
-                    cst = track_group_starts(st, ctx->n_sm, group_in());
-                    groups_ready = cst == FEM_OK;
-                    k_g_levelinfo<<<1, 256, 0, st>>>(crec, cn, N, cap, offs, iota, n_recs, coffN, d_ri, nthreads,
-                                                     g->pfine, g->sstep, g->target, g->d_maxP,
-                                                     groups_ready ? g->tg_gmax : nullptr, g->cap_threads);
-                }
+            if (small) {
+                level_small(&pf);
+            } else if (fuse_join) {
+                k_g_join_fused<<<1, 1024, 0, st>>>(pf.types, pf.lo, pf.hi, pf.foff, M, cap, ct, cl, ch, crec, cn,
+                                                   g->rel + N, offs, iota, n_recs, coffN, d_ri, nthreads, g->pfine,
+                                                   g->sstep, g->target, g->d_maxP);
             } else {
                 k_g_join_count<<<gb, 256, 0, st>>>(pf.types, pf.lo, pf.hi, pf.rec, pf.foff, cp, M, cap, pos);
                 if (cst == FEM_OK) cst = scan_exclusive(st, pos, cap + 1, scan_tmp, nullptr, nullptr);
@@ -1175,7 +1361,8 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
             cst = join_bound_level3(st, ctx->n_sm, ja);
         }
         const bool skipping = bounded || jbound;
-        k_g_ringcheck<<<gb, 256, 0, st>>>(ct, cl, crec, cn, N, need_dens ? d_dens : nullptr, d_lov,
+        if (!small)
+            k_g_ringcheck<<<gb, 256, 0, st>>>(ct, cl, crec, cn, N, need_dens ? d_dens : nullptr, d_lov,
                                           (int)lo_vals.size(), g->ring_cap, d_ri,
                                           cn, g->rel + N, n_recs, g->segf, g->pfine, g->sstep, g->segl,
                                           skipping ? g->skip : nullptr);
@@ -1201,13 +1388,21 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
             // items: recordings longest first; level 2 shares no prefix
             // work (one item per episode and segment), levels >= 3 group
             // episodes by their (N-1)-node prefix
-            TrackGroupIn gi = group_in();
-            gi.starts_ready = groups_ready;
-            cst = track_groups(st, ctx->n_sm, gi, N >= 3, &ta);
-            if (cst == FEM_OK) cst = launch_track(st, g->track_nblocks, ta);
+            if (small) {  // numbered by k_g_level_small
+                ta.gstart = N >= 3 ? g->tg_gstart : nullptr;
+                ta.gfirst = g->tg_gfirst;
+                ta.ibase = g->tg_ibase;
+                ta.rorder = g->rorder;
+                ta.d_n_items = g->tg_nitems;
+            } else {
+                TrackGroupIn gi = group_in();
+                gi.starts_ready = groups_ready;
+                cst = track_groups(st, ctx->n_sm, gi, N >= 3, &ta);
+            }
+            if (cst == FEM_OK) cst = launch_track(st, g->track_nblocks, ta, !small);
             if (cst == FEM_OK)
                 cst = launch_stitch_dev(st, ctx->n_sm, d_ri, iota, crec, rec, cn, cap, counts, fb_list, cn + 3,
-                                        skipping ? g->skip : nullptr, g->d_maxP, 1);
+                                        skipping ? g->skip : nullptr, g->d_maxP, 1, pfine_max);
         } else if (cst == FEM_OK) {
             cst = launch_count_dev(st, nmax, N, g->ring_cap, d_ri, n_recs, nthreads, g->cap_threads, offs, ct, cl, ch,
                                    iota, crec, rec, cn, cap, counts, fb_list, cn + 3, d_dens, d_lov,
@@ -1216,7 +1411,8 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
         ok(cudaEventRecordWithFlags(g->ev[2 * N + 1], st, cudaEventRecordExternal));
         if (fused) {
             k_g_thr_fused<<<1, 1024, 0, st>>>(counts, ct, cl, ch, crec, g->d_thr, N, cap, nf.types, nf.lo, nf.hi,
-                                              nf.rec, nf.counts, cn, n_recs, nf.foff);
+                                              nf.rec, nf.counts, cn, n_recs, nf.foff, d_ri,
+                                              skipping ? g->skip : nullptr, small ? g->rel + N : nullptr);
         } else {
             k_g_thr_flags<<<gb, 256, 0, st>>>(counts, crec, g->d_thr, cn, cap, pos);
             if (cst == FEM_OK) cst = scan_exclusive(st, pos, cap + 1, scan_tmp, nullptr, nullptr);

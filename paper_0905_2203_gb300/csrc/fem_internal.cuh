@@ -547,11 +547,12 @@ size_t sparse_smem_bytes(int nmax, int R);
 // Both stitch kernels over the live slots (count on the device) of a launch
 // whose records follow rinfo (per recording: slot_first, recbase, P).
 // d_maxP (optional): the largest segment count of any recording (device);
-// direct_p1: the counting kernel wrote the counts of unsegmented episodes.
+// direct_p1: the counting kernel wrote the counts of unsegmented episodes;
+// p_limit: no recording is ever cut into more segments.
 int launch_stitch_dev(cudaStream_t st, int nsm, const RecInfo *rinfo, const int32_t *slot2cand,
                       const uint32_t *cand_rec, const int32_t *rec, const int32_t *d_n_slots, int64_t cap_slots,
                       uint32_t *counts, int32_t *fb_list, int *fb_count, const uint8_t *skip, const int *d_maxP,
-                      int direct_p1);
+                      int direct_p1, int p_limit = INT32_MAX);
 // Segment boundaries (P + 1 entries) of a stream cut into P segments at time changes.
 int launch_segments(cudaStream_t st, const int32_t *time, int64_t n, int P, int64_t *seg);
 // Levels 1..max_size in one captured graph (streams resident; no host step
