@@ -421,6 +421,7 @@ int track_blocks(int n_sm);
 // sub-episodes (fem_joinbound.cu): per frequent 2-node episode a bitset of
 // its valid ends and one of its valid starts; skip[c] = 1 where the
 // popcount of their AND is at or below the threshold.
+constexpr int kJoinBoundMaxBins = 32;
 struct JoinBoundArgs {
     const RecInfo *ri;          // per recording: lists and time index
     int n_recs;
@@ -443,7 +444,7 @@ struct JoinBoundArgs {
     const uint32_t *thr;        // per recording
     uint32_t *vbits, *sbits;    // bitsets (cap_words words each)
     int64_t cap_words;
-    int nch;                    // chunks of 1024 events in the longest list
+    int chunk, nch;             // list events per item (a multiple of 32), items of the longest list
     int64_t *base;              // n_recs + 1: first word per recording, total
     uint8_t *skip;
     int or_skip;                // keep flags already set by another bound
