@@ -208,18 +208,20 @@ __device__ __forceinline__ bool g_joins(const uint16_t *ft, const int32_t *fl, c
     return true;
 }
 
-// Partners per frequent episode a of its recording (0 beyond the live count).
+// Partners per frequent episode a of its recording (0 beyond the live count);
+// one warp per episode, its partners tested 32 at a time.
 __global__ void k_g_join_count(const uint16_t *ft, const int32_t *fl, const int32_t *fh, const uint32_t *frec,
                                const int64_t *foff, const int32_t *ctr_prev, int M, int64_t cap, int32_t *cnt) {
     const int64_t F = ctr_prev[1];
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a <= cap; a += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
+    const int lane = threadIdx.x & 31;
+    for (int64_t a = F + t0; a <= cap; a += gs) cnt[a] = 0;
+    for (int64_t a = t0 >> 5; a < F; a += gs >> 5) {
+        const uint32_t r = frec[a];
         int32_t c = 0;
-        if (a < F) {
-            const uint32_t r = frec[a];
-            for (int64_t b = foff[r]; b < foff[r + 1]; ++b)
-                if (g_joins(ft, fl, fh, M, a, b)) ++c;
-        }
-        cnt[a] = c;
+        for (int64_t b = foff[r] + lane; b < foff[r + 1]; b += 32) c += g_joins(ft, fl, fh, M, a, b) ? 1 : 0;
+        c = __reduce_add_sync(0xFFFFFFFFu, c);
+        if (lane == 0) cnt[a] = c;
     }
 }
 
@@ -227,13 +229,17 @@ __global__ void k_g_join_write(const uint16_t *ft, const int32_t *fl, const int3
                                const int64_t *foff, const int32_t *ctr_prev, int M, int64_t cap, const int32_t *pos,
                                uint16_t *ct, int32_t *cl, int32_t *ch, uint32_t *crec, int32_t *ctr) {
     const int64_t F = ctr_prev[1];
-    const int N = M + 1;
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < F; a += (int64_t)gridDim.x * blockDim.x) {
+    const int N = M + 1, lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < F; a += nw) {
         const uint32_t r = frec[a];
-        int64_t o = pos[a];
-        for (int64_t b = foff[r]; b < foff[r + 1]; ++b) {
-            if (!g_joins(ft, fl, fh, M, a, b)) continue;
-            if (o < cap) {
+        int64_t at = pos[a];
+        for (int64_t base = foff[r]; base < foff[r + 1]; base += 32) {
+            const int64_t b = base + lane;
+            const bool ok = b < foff[r + 1] && g_joins(ft, fl, fh, M, a, b);
+            const unsigned bm = __ballot_sync(0xFFFFFFFFu, ok);
+            const int64_t o = at + __popc(bm & ((1u << lane) - 1u));
+            if (ok && o < cap) {
                 for (int k = 0; k < M; ++k) ct[o * N + k] = ft[a * M + k];
                 ct[o * N + M] = ft[b * M + M - 1];
                 for (int k = 0; k < M - 1; ++k) {
@@ -244,7 +250,7 @@ __global__ void k_g_join_write(const uint16_t *ft, const int32_t *fl, const int3
                 ch[o * (N - 1) + M - 1] = fh[b * (M - 1) + M - 2];
                 crec[o] = r;
             }
-            ++o;
+            at += __popc(bm);
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
