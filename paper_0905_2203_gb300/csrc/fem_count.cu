@@ -753,13 +753,13 @@ __device__ __forceinline__ uint32_t dens_lookup(const PrepArgs &a, int rec, int3
 
 __global__ void k_prep(PrepArgs a) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n_cand) return;
-    const int64_t c = a.subset ? a.subset[i] : i;
-    const int rec = a.cand_rec ? (int)a.cand_rec[c] : 0;
-    const int64_t o = a.offs[c];
-    const int64_t N = a.offs[c + 1] - o;
+    const bool in = i < a.n_cand;
+    const int64_t c = in ? (a.subset ? a.subset[i] : i) : 0;
+    const int rec = in && a.cand_rec ? (int)a.cand_rec[c] : 0;
+    const int64_t o = in ? a.offs[c] : 0;
+    const int64_t N = in ? a.offs[c + 1] - o : 0;
     const int64_t eo = o - c;
-    bool bad = (rec < 0 || rec >= a.n_recs || N < 1 || N > FEM_MAX_NODES);
+    bool bad = !in || (rec < 0 || rec >= a.n_recs || N < 1 || N > FEM_MAX_NODES);
     int R = 2;
     int64_t slab = 0;  // sum over nodes of the ring sizes
     int64_t sumhi = 0;
@@ -790,14 +790,15 @@ __global__ void k_prep(PrepArgs a) {
             }
         }
     }
-    if (bad) {
+    if (in && bad) {
         atomicOr(a.status, kStatusInval);
         a.key[i] = 0;
         a.ring[i] = 2;
-        return;
     }
-    int bucket;
-    if (a.mode == 1) {
+    int bucket = 0;
+    if (bad) {
+        // no part in the statistics
+    } else if (a.mode == 1) {
         bucket = kBucketPlain;
     } else if (N == 1) {
         bucket = kBucketN1;
@@ -810,13 +811,39 @@ __global__ void k_prep(PrepArgs a) {
         const int rc = R <= 2 ? 0 : R <= 4 ? 1 : R <= 8 ? 2 : R <= 16 ? 3 : R <= 32 ? 4 : 5;
         bucket = nc * kBucketRing + rc;
     }
-    a.key[i] = bucket * a.n_recs + rec;
-    a.ring[i] = R;
-    atomicMax(&a.bucket_maxR[bucket], R);
-    atomicMax(&a.bucket_maxR[kBuckets + bucket], (int)N);
-    atomicMax(&a.bucket_maxR[2 * kBuckets + bucket], (int)(sumhi > INT32_MAX ? INT32_MAX : sumhi));
-    atomicMax(&a.bucket_maxR[3 * kBuckets + bucket], (int)(slab > INT32_MAX ? INT32_MAX : slab));
-    atomicAdd(a.relevant, relv);
+    const int sum_hi = (int)(sumhi > INT32_MAX ? INT32_MAX : sumhi);
+    const int slab_i = (int)(slab > INT32_MAX ? INT32_MAX : slab);
+    if (!bad) {
+        a.key[i] = bucket * a.n_recs + rec;
+        a.ring[i] = R;
+    }
+    // The buckets' maxima and the sum: a warp whose candidates share a bucket
+    // (all multi-node ones of a local-tracking call do) makes one update of
+    // each; five per candidate on one address took 470 us for 200k.
+    const unsigned good = __ballot_sync(0xFFFFFFFFu, !bad);
+    if (!good) return;
+    const int b0 = __shfl_sync(0xFFFFFFFFu, bucket, __ffs(good) - 1);
+    if (__all_sync(0xFFFFFFFFu, bad || bucket == b0)) {
+        const int mR = __reduce_max_sync(0xFFFFFFFFu, bad ? 0 : R);
+        const int mN = __reduce_max_sync(0xFFFFFFFFu, bad ? 0 : (int)N);
+        const int mS = __reduce_max_sync(0xFFFFFFFFu, bad ? 0 : sum_hi);
+        const int mL = __reduce_max_sync(0xFFFFFFFFu, bad ? 0 : slab_i);
+        if (bad) relv = 0;
+        for (int d = 16; d > 0; d >>= 1) relv += __shfl_down_sync(0xFFFFFFFFu, relv, d);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&a.bucket_maxR[b0], mR);
+            atomicMax(&a.bucket_maxR[kBuckets + b0], mN);
+            atomicMax(&a.bucket_maxR[2 * kBuckets + b0], mS);
+            atomicMax(&a.bucket_maxR[3 * kBuckets + b0], mL);
+            atomicAdd(a.relevant, relv);
+        }
+    } else if (!bad) {
+        atomicMax(&a.bucket_maxR[bucket], R);
+        atomicMax(&a.bucket_maxR[kBuckets + bucket], (int)N);
+        atomicMax(&a.bucket_maxR[2 * kBuckets + bucket], sum_hi);
+        atomicMax(&a.bucket_maxR[3 * kBuckets + bucket], slab_i);
+        atomicAdd(a.relevant, relv);
+    }
 }
 
 // Stable partition by key: blocks of kPartBlock elements.  k_part_count
