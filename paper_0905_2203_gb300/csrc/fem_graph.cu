@@ -1283,8 +1283,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
                 const PairBoundArgs pb{d_ri, n_recs, d_cpre, cpre[n_recs], ub_chunk, d_nt, g->d_thr,
                                        d_uboff, d_blo, d_bhi, nb, hi_max, ub, 0, 0};
                 if (cst == FEM_OK)
-                    cst = pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, mean_window(g->recs, hi_max),
-                                     last_time(g->recs));
+                    cst = pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, last_time(g->recs));
             }
             const uint32_t *ubp = g->prepass ? ub : nullptr;
             k_g_prune_flags<<<gb2, 256, 0, st>>>(gt, glo, ghi, grec, cn, cap2, ubp, d_uboff, d_nt, d_blo, d_bhi, nb,

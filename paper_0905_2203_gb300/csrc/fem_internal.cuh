@@ -474,24 +474,12 @@ constexpr int kPairBoundMaxBins = 8;
 constexpr uint32_t kPairBoundMaxTypes = 1024;
 int pair_bound_chunk(int n_sm, int64_t events);
 int pair_bound(cudaStream_t st, int n_sm, PairBoundArgs a, const std::vector<int32_t> &blo,
-               const std::vector<int32_t> &bhi, uint32_t nt_max, double window, int64_t t_last);
+               const std::vector<int32_t> &bhi, uint32_t nt_max, int64_t t_last);
 inline int64_t last_time(const std::vector<fem_stream *> &recs) {
     int64_t t = 0;
     for (const fem_stream *s : recs) t = std::max<int64_t>(t, s->t_last);
     return t;
 }
-// Events within `hi` ticks after an event, on average over the recordings'
-// events.
-inline double mean_window(const std::vector<fem_stream *> &recs, int64_t hi) {
-    double w = 0, n = 0;
-    for (const fem_stream *s : recs) {
-        const double span = std::max(1.0, (double)s->t_last - (double)s->t_first);
-        w += (double)s->n * ((double)s->n * (double)hi / span);
-        n += (double)s->n;
-    }
-    return n > 0 ? w / n : 0.0;
-}
-
 // Prefix groups of the slots (flags, scan, first slot of each group, and,
 // if in.gmax is set, each recording's largest group) without the item
 // numbering, which depends on the segmentation.

@@ -640,7 +640,7 @@ int MineGroup::gen_level2() {
         pb.nb = nb;
         pb.hi_max = hi_max;
         pb.ub = ub;
-        FEM_TRY(pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, mean_window(recs, hi_max), last_time(recs)));
+        FEM_TRY(pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, last_time(recs)));
         S.kernel_launches++;
     } else {
         for (int r = 0; r < n_recs; ++r) {

@@ -17,12 +17,13 @@
 // 256 types at 25 Hz, 2.6e9 updates: 14.7 ms, 1.7e11 updates/s).  Here a block
 // takes a run of ONE type's event list, so all its updates fall into the
 // type's row of the table (n_types x bins counters), which it keeps in shared
-// memory and adds to the global table once; a warp (or G lanes of it, where
-// windows are short) takes one event and reads the events after it side by
-// side, so the loads are coalesced and no per-thread bitset is needed: the
-// same 20M events take about 4.4 ms, the 1.07M-event recording of 128 types
-// (21 events a window) 165 us instead of 270 us.  It issues on 77-81% of the
-// cycles at 39 registers (6 blocks per SM), the shared-memory pipe is 58% busy.
+// memory and adds to the global table once; eight lanes take one event and
+// read the events after it side by side, so the loads are coalesced and no
+// per-thread bitset is needed.  Whole-call times with 8 lanes an event for
+// every window, with 32 from 12 events on, and before: 20M events from host
+// memory (128 events a window) 6.2, 7.1 and 29.5 ms; 1.07M events of 128 types
+// (21 events) 536, 560 and 870 us.  It issues on about 80% of the cycles at 36
+// registers (6 blocks per SM); the shared-memory pipe is 58% busy.
 #include <algorithm>
 
 #include "fem_internal.cuh"
@@ -33,6 +34,8 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kPbThreads = 256;
+constexpr int kPbLanes = 8;                  // lanes of an event ...
+constexpr unsigned kPbLasts = 0x80808080u;   // ... and the last lane of each group
 constexpr int kPbMinChunk = 256, kPbMaxChunk = 4096;  // list positions per block
 
 // Which bin a distance falls into.  NB = 0: nb adjacent bins of one width (the
@@ -76,8 +79,9 @@ struct Bins<0> {
     }
 };
 
-template <int G, int NB>
+template <int NB>
 __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(PairBoundArgs a) {
+    constexpr int G = kPbLanes;
     extern __shared__ uint32_t s_row[];  // counter of (bin k, type b) at k * nt + b: neighbouring types, other banks
     constexpr int kSide = 32 / G;        // events a warp takes side by side
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -143,17 +147,12 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
                                 b = *py;
                                 bins.add(s_row, x, bj, nt, all);
                                 const unsigned bm = __ballot_sync(kFull, x < all);
-                                if (G == 32) {
-                                    if (!(bm >> 31)) break;
-                                } else {
-                                    constexpr unsigned kLasts = G == 16 ? 0x80008000u : 0x80808080u;
-                                    if (!(bm & kLasts)) break;
-                                    // a finished group waits at the padding
-                                    if (!((bm >> (lane | (G - 1))) & 1u)) {
-                                        pt = tm + n;
-                                        py = ty + n;
-                                        tj = INT32_MAX;
-                                    }
+                                if (!(bm & kPbLasts)) break;
+                                // a finished group waits at the padding
+                                if (!((bm >> (lane | (G - 1))) & 1u)) {
+                                    pt = tm + n;
+                                    py = ty + n;
+                                    tj = INT32_MAX;
                                 }
                             }
                         } else {
@@ -164,12 +163,8 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
                                 const bool win = in && d <= a.hi_max;
                                 if (win) bins.add(s_row + b, d, nt);
                                 const unsigned bm = __ballot_sync(kFull, win);
-                                if (G == 32) {
-                                    if (!(bm >> 31)) break;
-                                } else {
-                                    if (!((bm >> (lane | (G - 1))) & 1u)) j = n;
-                                    if (!__any_sync(kFull, j < n)) break;
-                                }
+                                if (!((bm >> (lane | (G - 1))) & 1u)) j = n;
+                                if (!__any_sync(kFull, j < n)) break;
                             }
                         }
                     }
@@ -187,14 +182,6 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
     }
 }
 
-typedef void (*PairBoundFn)(PairBoundArgs);
-
-template <int G>
-PairBoundFn pick_nb(int nb, bool even) {
-    if (even) return k_pair_bound<G, 0>;
-    return nb <= 2 ? k_pair_bound<G, 2> : nb <= 4 ? k_pair_bound<G, 4> : k_pair_bound<G, 8>;
-}
-
 }  // namespace
 
 // Chunk length (list positions per block): about four blocks per resident
@@ -206,11 +193,10 @@ int pair_bound_chunk(int n_sm, int64_t events) {
     return (int)std::max<int64_t>(kPbMinChunk, std::min<int64_t>(kPbMaxChunk, (c + 255) / 256 * 256));
 }
 
-// blo / bhi: the bins on the host; `window`: events of a look-ahead window on
-// average (weighted by event), which the lanes per event follow; t_last: the
-// last event time of any recording.
+// blo / bhi: the bins on the host; t_last: the last event time of any
+// recording.
 int pair_bound(cudaStream_t st, int n_sm, PairBoundArgs a, const std::vector<int32_t> &blo,
-               const std::vector<int32_t> &bhi, uint32_t nt_max, double window, int64_t t_last) {
+               const std::vector<int32_t> &bhi, uint32_t nt_max, int64_t t_last) {
     if (a.n_items < 1) return FEM_OK;
     // adjacent bins of one width; with m = ceil(2^32 / w) the high word of
     // x * m is x / w exactly while x * (m * w - 2^32) < 2^32, so for every
@@ -221,12 +207,14 @@ int pair_bound(cudaStream_t st, int n_sm, PairBoundArgs a, const std::vector<int
     even = even && t_last + a.hi_max < INT32_MAX;  // the padding's times lie past every window
     a.width = (uint32_t)w;
     a.magic = even ? (uint32_t)((((uint64_t)1 << 32) + w - 1) / w) : 0u;
-    const PairBoundFn f = window < 6.0    ? pick_nb<8>(a.nb, even)
-                          : window < 12.0 ? pick_nb<16>(a.nb, even)
-                                          : pick_nb<32>(a.nb, even);
     const size_t sm = sizeof(uint32_t) * (size_t)nt_max * (size_t)a.nb;  // at most 1024 x 8 words
     const unsigned grid = (unsigned)std::min<int64_t>(a.n_items, (int64_t)n_sm * 64);
-    f<<<grid, kPbThreads, sm, st>>>(a);
+    if (even)
+        k_pair_bound<0><<<grid, kPbThreads, sm, st>>>(a);
+    else if (a.nb <= 4)
+        k_pair_bound<4><<<grid, kPbThreads, sm, st>>>(a);
+    else
+        k_pair_bound<8><<<grid, kPbThreads, sm, st>>>(a);
     FEM_CUDA_TRY(cudaGetLastError());
     return FEM_OK;
 }
