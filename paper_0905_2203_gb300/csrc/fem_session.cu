@@ -13,9 +13,10 @@
 // and starts the greedy from the stored last end.  The tail's counts per type
 // stay on the device, so an append waits for the GPU twice, for the
 // validation and for the new tail's length: ten appends of 100k events with
-// 256 episodes take 2.0 ms, 9.0 with grid-wide tracking throughout.  Ends inside the tail cannot be kept
-// again: their latest start is at most the stored last end (each was either
-// kept, moving the last end to its own time, or refused for that reason).
+// 256 episodes take 2.0 ms, 9.0 with grid-wide tracking throughout.  Ends
+// inside the tail cannot be kept again: their latest start is at most the
+// stored last end (each was either kept, moving the last end to its own time,
+// or refused for that reason).
 #include <algorithm>
 #include <cstring>
 #include <mutex>

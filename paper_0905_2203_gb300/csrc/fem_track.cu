@@ -20,6 +20,9 @@
 //     come in time order, so the window only moves forward;
 //   * the lanes that found a valid predecessor append (t, L) to the node's
 //     entry list in the warp's buffer (ballot + prefix count);
+//   * where the previous node's entries are the shorter side, the lanes take
+//     32 of them instead and look up the events that each one serves with the
+//     stream's per-type time index (inner_by_entries, last_by_entries);
 //   * at the last node the valid ends inside the segment are handed, in time
 //     order, to Algorithm 1 for every entry class of the segment (one class
 //     per lane; the record is that of the other counting kernels, so k_stitch
