@@ -435,6 +435,7 @@ struct MineGroup {
     std::vector<int64_t> c_off;         // host copy of d_coff_rec
 
     int nrec() const { return (int)recs.size(); }
+    bool by_stream = false;             // no room for the list positions: the pair bound without them
     // no candidate's upper bounds add up to more than this
     int64_t span_max() const {
         int32_t h = 0;
@@ -522,6 +523,22 @@ int MineGroup::begin() {
     return finish_candidates();
 }
 
+// Gives back the list positions, which only the pair bound reads (and the
+// graphs captured with them).  Returns whether there were any.
+static bool drop_positions(fem_ctx *ctx, const std::vector<fem_stream *> &recs) {
+    bool any = false;
+    for (auto *s : recs) any = any || s->d_tpos;
+    if (!any) return false;
+    graph_cache_clear(ctx);
+    for (auto *s : recs)
+        if (s->d_tpos) {
+            dev_free(ctx, s->d_tpos, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
+            s->d_tpos = nullptr;
+            s->bytes -= sizeof(int32_t) * s->n;
+        }
+    return true;
+}
+
 int MineGroup::gen_level2() {
     const int n_recs = nrec();
     const int nb = (int)blo.size();
@@ -599,7 +616,7 @@ int MineGroup::gen_level2() {
     for (int r = 0; r < n_recs; ++r) ubp[r] = ub + ub_off[r];
     // by the per-type lists; without room for them (or over 2^30 events) each
     // event looks back over the stream
-    int by_lists = FEM_OK;
+    int by_lists = by_stream ? FEM_ERR_NOMEM : FEM_OK;
     for (int r = 0; r < n_recs && by_lists == FEM_OK; ++r) by_lists = stream_bytype(ctx, recs[r], true);
     if (by_lists != FEM_OK && by_lists != FEM_ERR_NOMEM && by_lists != FEM_ERR_INVAL) return by_lists;
     if (by_lists == FEM_OK) {
@@ -642,6 +659,8 @@ int MineGroup::gen_level2() {
         pb.ub = ub;
         FEM_TRY(pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, last_time(recs)));
         S.kernel_launches++;
+        // little room for the levels: they do without the list positions
+        if (ctx->used.load() > ctx->budget - ctx->budget / 4) drop_positions(ctx, recs);
     } else {
         for (int r = 0; r < n_recs; ++r) {
             const int words = (int)((nth[r] * (uint32_t)nb + 31) / 32);
@@ -797,6 +816,7 @@ int MineGroup::finish_candidates() {
 }
 
 int MineGroup::advance() {
+    track_release(ctx);  // the level's counts are queued: a join may take the entry lists' room
     const int n_recs = nrec();
     const int N = level;
     cudaStream_t st = ctx->stream;
@@ -1056,9 +1076,10 @@ void result_set_stats(fem_result *r, const fem_stats &s) { r->stats = s; }
 
 static int mine_impl(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const std::vector<int32_t> &blo,
                      const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr, int max_size,
-                     fem_result *res) {
+                     fem_result *res, bool by_stream) {
     MineGroup g;
     g.ctx = ctx;
+    g.by_stream = by_stream;
     g.recs = recs;
     for (int r = 0; r < (int)recs.size(); ++r) g.out_rec.push_back(r);
     g.res = res;
@@ -1071,7 +1092,7 @@ static int mine_impl(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
     // path or an alphabet is small enough for the tiled kernel to be the
     // better choice at level 2.
     const fem_tuning &tu = ctx->tuning;
-    bool whole = tu.level_graph != -1 && tu.plain_path != 1 && tu.kernel == 0 && tu.segments == 0 &&
+    bool whole = !by_stream && tu.level_graph != -1 && tu.plain_path != 1 && tu.kernel == 0 && tu.segments == 0 &&
                  tu.lanes_per_cta == 0 && tu.tile_events == 0 && max_size >= 2;
     for (auto *s : recs)
         if (s->n_types < 16) whole = false;
@@ -1140,7 +1161,11 @@ extern "C" int fem_mine_levelwise(fem_ctx *ctx, const fem_stream *const *recs, i
     {
         std::lock_guard<std::mutex> g(ctx->mu);
         cudaSetDevice(ctx->device);
-        st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res);
+        st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res, false);
+        if (st == FEM_ERR_NOMEM && drop_positions(ctx, rv)) {  // once more without the list positions
+            res->lv.assign(n_recs, std::vector<fem_result::Level>(max_size + 1));
+            st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res, true);
+        }
         if (st == FEM_OK) st = sync_status(ctx);
     }
     if (st != FEM_OK) {

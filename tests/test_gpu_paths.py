@@ -274,3 +274,30 @@ def test_one_recording_from_host_memory(fb, ctx, n_cand):
             ctx.count_episodes(st, fb.Cands(offs, bad, lo, hi), keep)
         assert e.value.status == fb.FEM_ERR_INVAL and (keep == 7).all()
         st.free()
+
+
+@pytest.mark.parametrize("recs,budget_mb", [(1, 28), (9, 40)])
+def test_mining_in_little_memory(fb, ctx, mid, recs, budget_mb):
+    """A budget that holds the recordings, their lists and one level, but not
+    the list positions beside them."""
+    s, cfg = mid
+    n = s.n // recs
+    cut = [(s.types[i * n:(i + 1) * n].copy(), s.times[i * n:(i + 1) * n].copy()) for i in range(recs)]
+    thr = [cfg["threshold"] // recs] * recs
+
+    def mine(c):
+        st = [c.load_stream(t, x, s.n_types) for t, x in cut]
+        res = c.mine_levelwise(st, cfg["bins"], thr, 5)
+        out = [np.asarray(a) for r in range(recs) for k in range(1, 6) for a in res.level_arrays(r, k)]
+        res.free()
+        for x in st:
+            x.free()
+        return out
+
+    small = fb.Context(0, hbm_budget_bytes=budget_mb << 20)
+    try:
+        got = mine(small)
+    finally:
+        small.close()
+    want = mine(ctx)
+    assert len(got) == len(want) and all(np.array_equal(a, b) for a, b in zip(got, want))
