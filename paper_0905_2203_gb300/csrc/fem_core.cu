@@ -99,8 +99,8 @@ void pool_release(fem_ctx *ctx) {
     ctx->cached_bytes = 0;
 }
 
-// Gives the entry lists back to the driver unless the call in progress works
-// with them.
+// Gives the entry lists back to the driver unless a launch that reads them is
+// being prepared.
 static bool track_give_back(fem_ctx *ctx) {
     if (ctx->track_held || !ctx->track.p) return false;
     cudaStreamSynchronize(ctx->stream);
@@ -196,18 +196,26 @@ int scratch(fem_ctx *ctx, int slot, size_t bytes, void **p) {
     return FEM_OK;
 }
 
-int track_lists(fem_ctx *ctx, size_t bytes, void **p) {
-    if (!ctx->track.p || ctx->track.cap < bytes) {
-        ctx->track_held = false;
-        track_give_back(ctx);
+int TrackLists::get(size_t bytes, int32_t **p) {
+    release();
+    if (ctx_->track_held) return FEM_ERR_NOMEM;  // (another launch is being prepared with them)
+    if (!ctx_->track.p || ctx_->track.cap < bytes) {
+        track_give_back(ctx_);
         void *q = nullptr;
-        FEM_TRY(dev_alloc(ctx, &q, bytes));
-        std::lock_guard<std::mutex> g(ctx->pool_mu);
-        ctx->track = DevBuf{q, ctx->live[q]};
+        FEM_TRY(dev_alloc(ctx_, &q, bytes));
+        std::lock_guard<std::mutex> g(ctx_->pool_mu);
+        ctx_->track = DevBuf{q, ctx_->live[q]};
     }
-    ctx->track_held = true;
-    *p = ctx->track.p;
+    ctx_->track_held = held_ = true;
+    *p = static_cast<int32_t *>(ctx_->track.p);
     return FEM_OK;
+}
+
+bool TrackLists::keep(const int32_t *p, size_t bytes) {
+    release();
+    if (ctx_->track_held || !p || ctx_->track.p != p || ctx_->track.cap < bytes) return false;
+    ctx_->track_held = held_ = true;
+    return true;
 }
 
 int sync_status(fem_ctx *ctx) {
@@ -618,7 +626,6 @@ int fem::load_stream_unlocked(fem_ctx *ctx, const uint16_t *types, const int32_t
     if (head) n += head->n;
     if (n > (int64_t)INT32_MAX * 4) return FEM_ERR_INVAL;
     *out = nullptr;
-    track_release(ctx);
     cudaSetDevice(ctx->device);
     fem_stream *s = new (std::nothrow) fem_stream();
     if (!s) return FEM_ERR_NOMEM;

@@ -1957,7 +1957,6 @@ static int group_pairs(CountCall &cc, int32_t *d_perm, int64_t ns, bool *use, do
 static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int force_segments) {
     fem_ctx *ctx = cc.ctx;
     const int n_recs = (int)cc.recs.size();
-    track_release(ctx);
     // Local tracking, one warp per (episode, segment), one launch for every
     // multi-node episode: the default (kernel 0) and kernel 7; the last
     // fallback round and the explicit kernel choices 1-3 keep the
@@ -2267,8 +2266,9 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             int blocks = track_nblocks;
             const int64_t n_items = limit > 0 ? std::min(limit, pl.records) : pl.records;
             blocks = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kTrackWarps - 1) / kTrackWarps));
-            void *pb = nullptr;
-            FEM_TRY(track_lists(ctx, track_buf_bytes(blocks, cap, pair_groups), &pb));
+            TrackLists lists(ctx);
+            int32_t *pb = nullptr;
+            FEM_TRY(lists.get(track_buf_bytes(blocks, cap, pair_groups), &pb));
             TrackArgs ta{};
             ta.rinfo = d_ri;
             ta.n_recs = n_recs;
@@ -2321,7 +2321,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
             ta.relaxed = cc.mode == 2;
             ta.skip = nullptr;
             ta.queue = reinterpret_cast<unsigned long long *>(mb + o_q);
-            ta.buf = static_cast<int32_t *>(pb);
+            ta.buf = pb;
             ta.cap = cap;
             ta.rec = rec_base;
             ta.counts = limit > 0 ? nullptr : cc.counts;  // unsegmented episodes: counts written directly
@@ -2956,7 +2956,6 @@ static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t
     }
     cc.plt_ok = n <= kPltMaxCands && s->n >= kPltMinEvents;
     if (cc.plt_ok && !few_by_segments(cc)) return FEM_OK;
-    track_release(ctx);
     const int sb = stream_tindex(ctx, s);
     if (sb == FEM_ERR_NOMEM) return FEM_OK;
     FEM_TRY(sb);
@@ -2986,10 +2985,13 @@ static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t
                  o_ty = carve(2 * nn), o_in = carve(64), o_ct = carve(4 * n), o_s2c = carve(4 * n),
                  o_fl = carve(4 * n), o_gs = carve(4 * (n + 1)), o_fb = carve(4 * n);
     const size_t up = o_in + 64, down = 64 + 4 * (size_t)n;
-    void *pd = nullptr, *pb = nullptr, *pr = nullptr;
-    if (scratch(ctx, kSlotQuick, off, &pd) != FEM_OK ||
-        track_lists(ctx, track_buf_bytes(blocks, s->max_list), &pb) != FEM_OK ||
-        scratch(ctx, kSlotRecords, (size_t)(n * P) * kRecWords * 4, &pr) != FEM_OK)
+    TrackLists lists(ctx);
+    int32_t *pb = nullptr;
+    void *pd = nullptr, *pr = nullptr;
+    const int64_t *seg = nullptr;
+    if (lists.get(track_buf_bytes(blocks, s->max_list), &pb) != FEM_OK || stream_segments(ctx, s, P, &seg) != FEM_OK ||
+        scratch(ctx, kSlotRecords, (size_t)(n * P) * kRecWords * 4, &pr) != FEM_OK ||
+        scratch(ctx, kSlotQuick, off, &pd) != FEM_OK)
         return FEM_OK;
     if (ctx->stage_bytes < std::max(up, down)) {
         if (ctx->stage) cudaFreeHost(ctx->stage);
@@ -3002,8 +3004,6 @@ static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t
         }
         ctx->stage_bytes = want;
     }
-    const int64_t *seg = nullptr;
-    FEM_TRY(stream_segments(ctx, s, P, &seg));
     *used = true;
     cudaStream_t st = ctx->stream;
     char *d = static_cast<char *>(pd), *h = static_cast<char *>(ctx->stage);
@@ -3039,7 +3039,7 @@ static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t
     ta.slot2cand = s2c;
     ta.relaxed = mode == 2;
     ta.queue = &info->queue;
-    ta.buf = static_cast<int32_t *>(pb);
+    ta.buf = pb;
     ta.cap = std::max<int64_t>(s->max_list, 1);
     ta.rec = static_cast<int32_t *>(pr);
     ta.counts = cc.counts;
@@ -3048,6 +3048,7 @@ static int count_quick(fem_ctx *ctx, fem_stream *s, const fem_cands *c, uint32_t
     ta.ibase = info->ibase;
     ta.last_mode = tu.track_last;
     FEM_TRY(launch_track(st, blocks, ta, false));
+    lists.release();
     if (P > 1) {
         k_stitch<<<(unsigned)((n + kStitchWarps - 1) / kStitchWarps), kStitchWarps * 32, 0, st>>>(
             ta.rec, ta.rinfo, s2c, nullptr, 0, (int)n, cc.counts, fb, &info->fb_count, &info->n_live, kStitchSplit);
@@ -3154,7 +3155,6 @@ __global__ void k_append_n1(const int32_t *__restrict__ cand, int n_slots, int n
 int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCount &c, fem_stats *stats, bool *used) {
     *used = false;
     cudaStream_t st = ctx->stream;
-    track_release(ctx);
     const int64_t m = fs->n, n_new = m - n_tail;
     // events of one type in the longest span (see few_by_segments)
     const double span = std::max(1.0, (double)fs->t_last - (double)fs->t_first);
@@ -3176,9 +3176,11 @@ int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCou
     const size_t free_b = track_room(ctx);
     while (blocks > 1 && track_buf_bytes(blocks, fs->max_list) > free_b / 4) blocks = (blocks + 1) / 2;
     if (track_buf_bytes(blocks, fs->max_list) + (size_t)items * kRecWords * 4 > free_b / 2) return FEM_OK;
-    void *pb = nullptr, *pr = nullptr, *pt = nullptr;
+    TrackLists lists(ctx);
+    int32_t *pb = nullptr;
+    void *pr = nullptr, *pt = nullptr;
     // table: [queue][RecInfo][segment starts]
-    if (track_lists(ctx, track_buf_bytes(blocks, fs->max_list), &pb) != FEM_OK ||
+    if (lists.get(track_buf_bytes(blocks, fs->max_list), &pb) != FEM_OK ||
         scratch(ctx, kSlotRecords, (size_t)std::max<int64_t>(items, 1) * kRecWords * 4, &pr) != FEM_OK ||
         scratch(ctx, kSlotRecTab, 512 + sizeof(int64_t) * (kStitchSplit + 1), &pt) != FEM_OK)
         return FEM_OK;
@@ -3210,7 +3212,7 @@ int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCou
         ta.chi = c.hi;
         ta.slot2cand = c.slots;
         ta.queue = reinterpret_cast<unsigned long long *>(tab);
-        ta.buf = static_cast<int32_t *>(pb);
+        ta.buf = pb;
         ta.cap = std::max<int64_t>(fs->max_list, 1);
         ta.rec = static_cast<int32_t *>(pr);
         ta.last_mode = ctx->tuning.track_last;

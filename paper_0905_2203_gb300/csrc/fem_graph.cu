@@ -894,8 +894,9 @@ static size_t graph_sparse_smem(int N, int R) {
     return (size_t)(6 * (nmax - 1) + 2 * (N - 1) * R) * 64 * 4;
 }
 
-static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std::vector<int32_t> &bhi,
-                       const std::vector<uint32_t> &thr, const std::vector<int32_t> &lo_vals) {
+static int build_graph(GraphTail *g, TrackLists &lists, const std::vector<int32_t> &blo,
+                       const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr,
+                       const std::vector<int32_t> &lo_vals) {
     fem_ctx *ctx = g->ctx;
     cudaStream_t st = ctx->stream;
     const int n_recs = g->n_recs, L = g->max_size, first = g->first;
@@ -1036,9 +1037,7 @@ static int build_graph(GraphTail *g, const std::vector<int32_t> &blo, const std:
     FEM_TRY(g->get(&rec, (size_t)g->cap_threads * kRecWords));
     FEM_TRY(g->get(&g->d_maxP, 1));
     if (g->track) {
-        void *tb = nullptr;
-        FEM_TRY(track_lists(ctx, track_buf_bytes(g->track_nblocks, g->track_cap), &tb));
-        g->tbuf = static_cast<int32_t *>(tb);
+        FEM_TRY(lists.get(track_buf_bytes(g->track_nblocks, g->track_cap), &g->tbuf));
         FEM_TRY(g->get(&g->tqueue, 1));
         FEM_TRY(g->get(&g->tg_gidx, cap + 2));
         FEM_TRY(g->get(&g->tg_gstart, cap + 2));
@@ -1541,14 +1540,12 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
         while (cap < pairs / 4 && cap < (1 << 20)) cap <<= 1;
     }
     GraphTail *g = nullptr;
-    track_release(ctx);
+    TrackLists lists(ctx);
     auto it = ctx->graphs.find(key);
     if (it != ctx->graphs.end() && it->second->cap >= cap_need &&
         (!it->second->track ||
-         (it->second->tbuf == ctx->track.p &&
-          ctx->track.cap >= track_buf_bytes(it->second->track_nblocks, it->second->track_cap)))) {
+         lists.keep(it->second->tbuf, track_buf_bytes(it->second->track_nblocks, it->second->track_cap)))) {
         g = it->second;
-        ctx->track_held = g->track;
     } else {
         if (it != ctx->graphs.end()) {
             delete it->second;
@@ -1570,7 +1567,7 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
             ng->coarse = coarse;
             ng->coarse_min = 0;
             ng->cap = cap;
-            st = build_graph(ng.get(), blo, bhi, thr, lo_vals);
+            st = build_graph(ng.get(), lists, blo, bhi, thr, lo_vals);
             if (st != FEM_ERR_NOMEM || cap == cap_need) break;
             cap = cap_need;  // no room for the guess
         }

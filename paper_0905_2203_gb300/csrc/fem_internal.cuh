@@ -201,8 +201,8 @@ struct fem_ctx {
     fem_tuning tuning{};
     fem_stats last{};
     std::map<int, fem::DevBuf> scratch;  // slot -> buffer (grown on demand)
-    fem::DevBuf track;                   // per-warp entry lists of the local-tracking kernel (track_lists)
-    bool track_held = false;             // the call in progress works with them
+    fem::DevBuf track;                   // per-warp entry lists of the local-tracking kernel (TrackLists)
+    bool track_held = false;             // a launch that reads them is being prepared
     std::map<std::string, fem::TuneVal> tune;  // autotuner cache
     std::map<std::string, fem::GraphTail *> graphs;  // captured mining graphs
     std::map<std::string, int64_t> graph_cap;        // candidate capacity a graph key needed last time
@@ -280,14 +280,30 @@ int dev_alloc(fem_ctx *ctx, void **p, size_t bytes);
 void dev_free(fem_ctx *ctx, void *p, size_t bytes);
 // Scratch slot of at least `bytes` (contents undefined).
 int scratch(fem_ctx *ctx, int slot, size_t bytes, void **p);
-// The context's per-warp entry lists, at least `bytes`: one buffer for every
-// counting launch and mining graph of the context (their work is ordered on
-// its stream; each launch writes what it reads).  Grown exactly; a call that
-// begins lets go of it (track_release), and an allocation that finds no room
-// then takes it back.  A captured graph remembers the pointer and is captured
-// again when the buffer has moved.
-int track_lists(fem_ctx *ctx, size_t bytes, void **p);
-inline void track_release(fem_ctx *ctx) { ctx->track_held = false; }
+// The context's per-warp entry lists: one buffer for every counting launch and
+// mining graph of the context (their work is ordered on its stream; each
+// launch writes what it reads), grown exactly.  An object of this class keeps
+// them while a launch that reads them is prepared and queued; at any other time
+// an allocation that finds no room takes them back (and waits for the stream
+// first).  A captured graph remembers the pointer and is captured again when
+// the buffer has moved.
+class TrackLists {
+  public:
+    explicit TrackLists(fem_ctx *c) : ctx_(c) {}
+    ~TrackLists() { release(); }
+    TrackLists(const TrackLists &) = delete;
+    TrackLists &operator=(const TrackLists &) = delete;
+    int get(size_t bytes, int32_t **p);            // at least `bytes`
+    bool keep(const int32_t *p, size_t bytes);     // whether they are still p and hold `bytes`
+    void release() {
+        if (held_) ctx_->track_held = false;
+        held_ = false;
+    }
+
+  private:
+    fem_ctx *ctx_;
+    bool held_ = false;
+};
 // Budget left for those lists: what is free and what they hold.
 inline size_t track_room(const fem_ctx *ctx) {
     const size_t used = ctx->used.load() - ctx->track.cap;

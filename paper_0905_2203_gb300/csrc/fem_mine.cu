@@ -816,7 +816,6 @@ int MineGroup::finish_candidates() {
 }
 
 int MineGroup::advance() {
-    track_release(ctx);  // the level's counts are queued: a join may take the entry lists' room
     const int n_recs = nrec();
     const int N = level;
     cudaStream_t st = ctx->stream;
