@@ -415,6 +415,8 @@ struct AppendCount {
     const int32_t *lo, *hi;
     const int32_t *slots;        // the multi-node ones [n_slots], then the
     int n_slots, n_singles;      // 1-node ones [n_singles]
+    const int64_t *h_offs;       // the offsets and types on the host
+    const uint16_t *h_types;
     int64_t sumhi;               // largest sum of an episode's upper bounds
     const int32_t *tail_cnt;     // tail events per type
     uint32_t *counts;            // added to
@@ -423,8 +425,8 @@ struct AppendCount {
     int *fb_count;               // (zeroed here)
     unsigned long long *relevant;  // relevant events of all candidates (zeroed here)
 };
-// *used = false (nothing launched): the spans hold too many events of a type
-// to cut the recording, or the lists have no room.  Does not wait.
+// *used = false (nothing launched): the recording cannot be cut and counting
+// grid-wide is the shorter way, or the lists have no room.
 int count_appended(fem_ctx *ctx, fem_stream *fs, int64_t n_tail, const AppendCount &c, fem_stats *stats, bool *used);
 
 // Persistent grid of the local-tracking kernel on this device (blocks), the

@@ -9,14 +9,14 @@
 // reach back to: the events at or after t_last - max sum(hi).  An append
 // counts the tail followed by the new events by local tracking, one warp per
 // (episode, segment of the new events) (fem_track.cu; grid-wide, fem_plt.cu,
-// where spans are too wide to cut), takes only the ends among the new events,
-// and starts the greedy from the stored last end.  The tail's counts per type
-// stay on the device, so an append waits for the GPU twice, for the
-// validation and for the new tail's length: ten appends of 100k events with
-// 256 episodes take 2.0 ms, 9.0 with grid-wide tracking throughout.  Ends
-// inside the tail cannot be kept again: their latest start is at most the
-// stored last end (each was either kept, moving the last end to its own time,
-// or refused for that reason).
+// where they can be cut too little for that to be the shorter way), takes only
+// the ends among the new events, and starts the greedy from the stored last
+// end.  The tail's counts per type stay on the device, so an append waits for
+// the GPU twice, for the validation and for the new tail's length: ten appends
+// of 100k events with 256 episodes take 2.0 ms, 9.0 with grid-wide tracking
+// throughout.  Ends inside the tail cannot be kept again: their latest start is
+// at most the stored last end (each was either kept, moving the last end to its
+// own time, or refused for that reason).
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -43,6 +43,8 @@ struct fem_session {
     int32_t *d_fb = nullptr;         // candidates that overflowed [n_cand]
     int32_t *d_slots = nullptr;      // multi-node candidates, then 1-node ones [n_cand]
     int n_slots = 0;                 // multi-node candidates
+    std::vector<int64_t> h_offs;     // the candidates' offsets and types on the host
+    std::vector<uint16_t> h_types;
     int64_t seen = 0;                // events appended so far
 };
 
@@ -188,6 +190,8 @@ extern "C" int fem_session_create(fem_ctx *ctx, const fem_cands *c, uint32_t n_t
         delete s;
         return st;
     }
+    s->h_offs.swap(offs);
+    s->h_types.swap(ty);
     *out = s;
     return FEM_OK;
 }
@@ -223,6 +227,8 @@ extern "C" int fem_session_append(fem_session *s, const uint16_t *types, const i
         ac.slots = s->d_slots;
         ac.n_slots = s->n_slots;
         ac.n_singles = (int)s->n_cand - s->n_slots;
+        ac.h_offs = s->h_offs.data();
+        ac.h_types = s->h_types.data();
         ac.sumhi = s->span_max;
         ac.tail_cnt = tail_cnt;
         ac.counts = s->d_counts;

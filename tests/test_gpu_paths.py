@@ -301,3 +301,29 @@ def test_mining_in_little_memory(fb, ctx, mid, recs, budget_mb):
         small.close()
     want = mine(ctx)
     assert len(got) == len(want) and all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("n_cand,chunk,n_types,grid", [(8, 100_000, 2, True), (8, 5_000, 2, False),
+                                                       (40, 60_000, 60, False)])
+def test_wide_appends_take_the_shorter_way(fb, ctx, n_cand, chunk, n_types, grid):
+    """Appends whose spans hold too many events of a type to cut the chunk: few
+    episodes over long lists are counted grid-wide (no launch over work items),
+    short lists by one warp an episode; counts are the oracle's either way."""
+    ty, tm = synth.tiny_random_stream(79, 2 * chunk, n_types, 20 * chunk)
+    wide = 10 * n_types * 12  # twelve events of a type per edge
+    r = synth.Rng(80, n_cand)
+    offs = np.arange(0, 4 * n_cand + 1, 4, dtype=np.int64)
+    ct = r.integers(0, n_types - 1, 4 * n_cand).astype(np.uint16)
+    lo = (r.integers(0, 1, 3 * n_cand) * wide // 2).astype(np.int32)
+    hi = (lo + wide).astype(np.int32)
+    sess = ctx.session(fb.Cands(offs, ct, lo, hi), n_types)
+    try:
+        for a in (0, chunk):
+            sess.append(ty[a:a + chunk], tm[a:a + chunk])
+            assert (ctx.last_stats()["sparse_launches"] == 0) == grid
+        got = sess.counts().astype(np.int64)
+    finally:
+        sess.close()
+    n = min(len(ty), 2 * chunk)
+    want = oracle_counts(ty[:n], tm[:n], offs, ct, lo, hi)
+    assert np.array_equal(got, want) and want.max() > 0
