@@ -115,13 +115,40 @@ static bool track_give_back(fem_ctx *ctx) {
     return true;
 }
 
+PositionsHold::PositionsHold(const std::vector<fem_stream *> &recs) : recs_(recs) {
+    for (auto *s : recs_) ++s->tpos_holds;
+}
+
+void PositionsHold::release() {
+    for (auto *s : recs_) --s->tpos_holds;
+    recs_.clear();
+}
+
+void drop_positions(fem_ctx *ctx, fem_stream *s) {
+    if (!s->d_tpos || s->tpos_holds > 0) return;
+    graph_cache_drop(ctx, s);
+    dev_free(ctx, s->d_tpos, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
+    s->d_tpos = nullptr;
+    s->bytes -= sizeof(int32_t) * s->n;
+    auto &v = ctx->with_tpos;
+    v.erase(std::remove(v.begin(), v.end(), s), v.end());
+}
+
+// Takes back what is only kept for later calls: the entry lists, then the list
+// positions.  Returns whether anything came back.
+static bool give_back(fem_ctx *ctx) {
+    if (track_give_back(ctx)) return true;
+    const std::vector<fem_stream *> with = ctx->with_tpos;
+    for (auto *s : with) drop_positions(ctx, s);
+    return ctx->with_tpos.size() < with.size();
+}
+
 int dev_alloc(fem_ctx *ctx, void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~size_t(255);
-    if (ctx->used.load() + bytes > ctx->budget &&
-        (!track_give_back(ctx) || ctx->used.load() + bytes > ctx->budget))
-        return FEM_ERR_NOMEM;
+    while (ctx->used.load() + bytes > ctx->budget)
+        if (!give_back(ctx)) return FEM_ERR_NOMEM;
     {
         std::lock_guard<std::mutex> g(ctx->pool_mu);
         auto it = ctx->cached.lower_bound(bytes);
@@ -140,8 +167,9 @@ int dev_alloc(fem_ctx *ctx, void **p, size_t bytes) {
         cudaGetLastError();
         pool_release(ctx);
         e = cudaMalloc(p, bytes);
-        if (e == cudaErrorMemoryAllocation && track_give_back(ctx)) {
+        while (e == cudaErrorMemoryAllocation && give_back(ctx)) {
             cudaGetLastError();
+            pool_release(ctx);
             e = cudaMalloc(p, bytes);
         }
     }
@@ -713,7 +741,7 @@ void fem::stream_free_unlocked(fem_stream *s) {
     coarse_free(ctx, s);
     if (s->d_toff) dev_free(ctx, s->d_toff, sizeof(int64_t) * (s->n_types + 1));
     if (s->d_ttime) dev_free(ctx, s->d_ttime, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
-    if (s->d_tpos) dev_free(ctx, s->d_tpos, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
+    drop_positions(ctx, s);
     if (s->d_tidx) dev_free(ctx, s->d_tidx, sizeof(int32_t) * (size_t)s->n_types * (size_t)(s->tcells + 1));
     delete s;
 }

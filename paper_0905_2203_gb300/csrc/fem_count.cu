@@ -1651,6 +1651,7 @@ int stream_bytype(fem_ctx *ctx, fem_stream *s, bool pos) {
     if (pos) {
         s->d_tpos = static_cast<int32_t *>(p3);
         s->bytes += sizeof(int32_t) * n;
+        ctx->with_tpos.push_back(s);
     }
     return FEM_OK;
 }

@@ -1479,12 +1479,18 @@ void graph_cache_clear(fem_ctx *ctx) {
     ctx->graphs.clear();
 }
 
-void graph_cache_forget(fem_ctx *ctx, const fem_stream *s) {
+// forget: every graph over s, with the capacity it needed; otherwise those that
+// read list positions (their level 2 bounds the pairs).
+static void graph_cache_erase(fem_ctx *ctx, const fem_stream *s, bool forget) {
     for (auto it = ctx->graphs.begin(); it != ctx->graphs.end();) {
         bool uses = false;
+        if (!forget && it->second->first > 2) {
+            ++it;
+            continue;
+        }
         for (auto *r : it->second->recs) uses = uses || r == s;
         if (uses) {
-            ctx->graph_cap.erase(it->first);
+            if (forget) ctx->graph_cap.erase(it->first);
             delete it->second;
             it = ctx->graphs.erase(it);
         } else {
@@ -1492,6 +1498,10 @@ void graph_cache_forget(fem_ctx *ctx, const fem_stream *s) {
         }
     }
 }
+
+void graph_cache_forget(fem_ctx *ctx, const fem_stream *s) { graph_cache_erase(ctx, s, true); }
+
+void graph_cache_drop(fem_ctx *ctx, const fem_stream *s) { graph_cache_erase(ctx, s, false); }
 
 namespace {
 
@@ -1541,6 +1551,7 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
     }
     GraphTail *g = nullptr;
     TrackLists lists(ctx);
+    const PositionsHold positions(recs);
     auto it = ctx->graphs.find(key);
     if (it != ctx->graphs.end() && it->second->cap >= cap_need &&
         (!it->second->track ||

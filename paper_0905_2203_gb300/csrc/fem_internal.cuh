@@ -203,6 +203,7 @@ struct fem_ctx {
     std::map<int, fem::DevBuf> scratch;  // slot -> buffer (grown on demand)
     fem::DevBuf track;                   // per-warp entry lists of the local-tracking kernel (TrackLists)
     bool track_held = false;             // a launch that reads them is being prepared
+    std::vector<fem_stream *> with_tpos; // recordings that keep list positions
     std::map<std::string, fem::TuneVal> tune;  // autotuner cache
     std::map<std::string, fem::GraphTail *> graphs;  // captured mining graphs
     std::map<std::string, int64_t> graph_cap;        // candidate capacity a graph key needed last time
@@ -245,6 +246,7 @@ struct fem_stream {
     int64_t *d_toff = nullptr;    // per-type event lists (built on first use): offsets [n_types + 1]
     int32_t *d_ttime = nullptr;   // times grouped by type, ascending within a type [n]
     int32_t *d_tpos = nullptr;    // stream position of every list entry [n] (built on request)
+    int tpos_holds = 0;           // steps at work that read them (PositionsHold)
     int64_t max_list = 0;         // longest per-type list (the largest frequency)
     // Per-type time index (built on first use, after the lists): cells of
     // 2^tshift ticks from t_first; d_tidx[a * (tcells + 1) + c] is the
@@ -304,6 +306,26 @@ class TrackLists {
     fem_ctx *ctx_;
     bool held_ = false;
 };
+// List positions (stream_bytype with `pos`) are read by the level-2 pair bound
+// alone and kept for the recording's next mining call: an allocation that finds
+// no room takes them back, with the mining graphs captured on them, from every
+// recording that no object of this class holds.  A step holds its recordings
+// from before it asks for their positions until the launch that reads them is
+// queued (a captured graph: until it has run).
+class PositionsHold {
+  public:
+    explicit PositionsHold(const std::vector<fem_stream *> &recs);
+    ~PositionsHold() { release(); }
+    PositionsHold(const PositionsHold &) = delete;
+    PositionsHold &operator=(const PositionsHold &) = delete;
+    void release();
+
+  private:
+    std::vector<fem_stream *> recs_;
+};
+// Gives the positions of a recording that is not held back (if it has any).
+void drop_positions(fem_ctx *ctx, fem_stream *s);
+
 // Budget left for those lists: what is free and what they hold.
 inline size_t track_room(const fem_ctx *ctx) {
     const size_t used = ctx->used.load() - ctx->track.cap;
@@ -576,6 +598,7 @@ int run_graph_tail(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const st
                    TailResult *out, bool *used);
 void graph_cache_clear(fem_ctx *ctx);
 void graph_cache_forget(fem_ctx *ctx, const fem_stream *s);
+void graph_cache_drop(fem_ctx *ctx, const fem_stream *s);  // those that read its list positions
 // Stream load without taking the context lock (caller holds it or owns the
 // context exclusively).
 // Events in two parts: np device-resident ones, then n.

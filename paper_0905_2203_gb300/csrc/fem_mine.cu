@@ -435,7 +435,7 @@ struct MineGroup {
     std::vector<int64_t> c_off;         // host copy of d_coff_rec
 
     int nrec() const { return (int)recs.size(); }
-    bool by_stream = false;             // no room for the list positions: the pair bound without them
+    bool once = false;                  // the recordings are mined once: list positions go back after the bound
     // no candidate's upper bounds add up to more than this
     int64_t span_max() const {
         int32_t h = 0;
@@ -523,22 +523,6 @@ int MineGroup::begin() {
     return finish_candidates();
 }
 
-// Gives back the list positions, which only the pair bound reads (and the
-// graphs captured with them).  Returns whether there were any.
-static bool drop_positions(fem_ctx *ctx, const std::vector<fem_stream *> &recs) {
-    bool any = false;
-    for (auto *s : recs) any = any || s->d_tpos;
-    if (!any) return false;
-    graph_cache_clear(ctx);
-    for (auto *s : recs)
-        if (s->d_tpos) {
-            dev_free(ctx, s->d_tpos, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
-            s->d_tpos = nullptr;
-            s->bytes -= sizeof(int32_t) * s->n;
-        }
-    return true;
-}
-
 int MineGroup::gen_level2() {
     const int n_recs = nrec();
     const int nb = (int)blo.size();
@@ -616,7 +600,15 @@ int MineGroup::gen_level2() {
     for (int r = 0; r < n_recs; ++r) ubp[r] = ub + ub_off[r];
     // by the per-type lists; without room for them (or over 2^30 events) each
     // event looks back over the stream
-    int by_lists = by_stream ? FEM_ERR_NOMEM : FEM_OK;
+    RecInfo *d_ri;
+    int64_t *d_cpre, *d_uboff;
+    uint32_t *d_ntp;
+    FEM_TRY(tmp.get(&d_ri, n_recs));
+    FEM_TRY(tmp.get(&d_cpre, n_recs + 1));
+    FEM_TRY(tmp.get(&d_uboff, n_recs + 1));
+    FEM_TRY(tmp.get(&d_ntp, n_recs));
+    PositionsHold positions(recs);
+    int by_lists = FEM_OK;
     for (int r = 0; r < n_recs && by_lists == FEM_OK; ++r) by_lists = stream_bytype(ctx, recs[r], true);
     if (by_lists != FEM_OK && by_lists != FEM_ERR_NOMEM && by_lists != FEM_ERR_INVAL) return by_lists;
     if (by_lists == FEM_OK) {
@@ -634,13 +626,6 @@ int MineGroup::gen_level2() {
             ri[r].freq = recs[r]->d_freq;
             recinfo_lists(ri[r], recs[r]);
         }
-        RecInfo *d_ri;
-        int64_t *d_cpre, *d_uboff;
-        uint32_t *d_ntp;
-        FEM_TRY(tmp.get(&d_ri, n_recs));
-        FEM_TRY(tmp.get(&d_cpre, n_recs + 1));
-        FEM_TRY(tmp.get(&d_uboff, n_recs + 1));
-        FEM_TRY(tmp.get(&d_ntp, n_recs));
         FEM_CUDA_TRY(cudaMemcpyAsync(d_ri, ri.data(), sizeof(RecInfo) * n_recs, cudaMemcpyHostToDevice, st));
         FEM_CUDA_TRY(cudaMemcpyAsync(d_cpre, cpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
         FEM_CUDA_TRY(cudaMemcpyAsync(d_uboff, ub_off.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
@@ -659,9 +644,13 @@ int MineGroup::gen_level2() {
         pb.ub = ub;
         FEM_TRY(pair_bound(st, ctx->n_sm, pb, blo, bhi, nt_max, last_time(recs)));
         S.kernel_launches++;
-        // little room for the levels: they do without the list positions
-        if (ctx->used.load() > ctx->budget - ctx->budget / 4) drop_positions(ctx, recs);
+        positions.release();
+        // (little room for the levels: they are cut by what is free)
+        if (once || ctx->used.load() > ctx->budget - ctx->budget / 4)
+            for (auto *s : recs) drop_positions(ctx, s);
     } else {
+        positions.release();
+        for (auto *s : recs) drop_positions(ctx, s);
         for (int r = 0; r < n_recs; ++r) {
             const int words = (int)((nth[r] * (uint32_t)nb + 31) / 32);
             int threads = std::min(256, (int)(48 * 1024 / (4 * words)) / 32 * 32);
@@ -1055,6 +1044,7 @@ MineGroup *mg_create(fem_ctx *ctx, fem_stream *s, const std::vector<int32_t> &bl
     g->bhi = bhi;
     g->thr = {thr};
     g->max_size = max_size;
+    g->once = true;
     return g;
 }
 int mg_begin(MineGroup *g) { return g->begin(); }
@@ -1075,10 +1065,9 @@ void result_set_stats(fem_result *r, const fem_stats &s) { r->stats = s; }
 
 static int mine_impl(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const std::vector<int32_t> &blo,
                      const std::vector<int32_t> &bhi, const std::vector<uint32_t> &thr, int max_size,
-                     fem_result *res, bool by_stream) {
+                     fem_result *res) {
     MineGroup g;
     g.ctx = ctx;
-    g.by_stream = by_stream;
     g.recs = recs;
     for (int r = 0; r < (int)recs.size(); ++r) g.out_rec.push_back(r);
     g.res = res;
@@ -1091,7 +1080,7 @@ static int mine_impl(fem_ctx *ctx, const std::vector<fem_stream *> &recs, const 
     // path or an alphabet is small enough for the tiled kernel to be the
     // better choice at level 2.
     const fem_tuning &tu = ctx->tuning;
-    bool whole = !by_stream && tu.level_graph != -1 && tu.plain_path != 1 && tu.kernel == 0 && tu.segments == 0 &&
+    bool whole = tu.level_graph != -1 && tu.plain_path != 1 && tu.kernel == 0 && tu.segments == 0 &&
                  tu.lanes_per_cta == 0 && tu.tile_events == 0 && max_size >= 2;
     for (auto *s : recs)
         if (s->n_types < 16) whole = false;
@@ -1160,11 +1149,7 @@ extern "C" int fem_mine_levelwise(fem_ctx *ctx, const fem_stream *const *recs, i
     {
         std::lock_guard<std::mutex> g(ctx->mu);
         cudaSetDevice(ctx->device);
-        st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res, false);
-        if (st == FEM_ERR_NOMEM && drop_positions(ctx, rv)) {  // once more without the list positions
-            res->lv.assign(n_recs, std::vector<fem_result::Level>(max_size + 1));
-            st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res, true);
-        }
+        st = mine_impl(ctx, rv, blo, bhi, thr, max_size, res);
         if (st == FEM_OK) st = sync_status(ctx);
     }
     if (st != FEM_OK) {

@@ -60,11 +60,13 @@ struct fem_server {
 
 namespace {
 
-// Device memory a job is expected to hold: its stream (6 B per event plus
-// padding), level-2 candidate arrays and the pair-bound table (both at most
-// quadratic in the alphabet), and a fixed allowance for the rest.
+// Device memory a job is expected to hold: its stream, level-2 candidate arrays
+// and the pair-bound table (both at most quadratic in the alphabet), and a
+// fixed allowance for the rest (level-wise arrays, segment records, entry
+// lists).
 size_t estimate_job_bytes(int64_t n, uint32_t n_types, int nb) {
-    // stream (6 B/event) + per-type lists (4 B/event kept, 8 B/event while built)
+    // per event: the stream 6 B, the per-type lists 4 B, their time index 3 to
+    // 6 B, and until the pair bound has been queued the list positions, 4 B
     const size_t stream = (size_t)(n + fem::kPadEvents) * 18;
     const size_t pairs = (size_t)n_types * n_types * (size_t)std::max(nb, 1);
     return stream + pairs * 48 + (size_t)16 * 1024 * 1024;

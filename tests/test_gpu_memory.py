@@ -50,3 +50,78 @@ def test_recounts_of_an_append_find_the_entry_lists_room(fb):
     want, _ = oracle.count_many(ty, tm, *cands)
     assert np.array_equal(got, want.astype(np.int64))
     assert again > 50
+
+
+def poisson_types(seed, n, n_types, per):
+    """n events of n_types types at 5 to 20 units of rate, `per` ticks apart on
+    average, sorted, no repeated (type, time)."""
+    r = np.random.default_rng(seed)
+    p = np.random.default_rng(7).uniform(5, 20, n_types)
+    ty = r.choice(n_types, n, p=p / p.sum())
+    key = np.unique(np.sort(r.integers(0, n * per, n)) * 65536 + ty)
+    return (key % 65536).astype(np.uint16), (key // 65536).astype(np.int32)
+
+
+def test_a_served_job_has_the_list_positions_room_after_level_2(fb):
+    """A lone job whose third level needs, beside the recording, its lists and
+    their index, more than what the budget leaves while the list positions
+    (4 bytes an event) are kept; they are read by level 2 alone."""
+    ty, tm = poisson_types(1, 4_080_000, 60, 83)
+    bins, thr = [(0, 500), (500, 1000), (1000, 1500), (1500, 2000)], 8000
+    srv = fb.Server(0, hbm_budget_bytes=128 << 20, max_jobs=2)
+    try:
+        res, _ = srv.wait(srv.submit(ty, tm, 60, bins, thr, 3), 120_000)
+        got = [np.asarray(a) for k in (1, 2, 3) for a in res.level_arrays(0, k)]
+        res.free()
+    finally:
+        srv.close()
+    ctx = fb.Context(0)
+    st = ctx.load_stream(ty, tm, 60)
+    res = ctx.mine_levelwise([st], bins, [thr], 3)
+    want = [np.asarray(a) for k in (1, 2, 3) for a in res.level_arrays(0, k)]
+    res.free()
+    st.free()
+    ctx.close()
+    assert all(np.array_equal(a, b) for a, b in zip(got, want)) and len(want[9]) > 0
+
+
+@pytest.mark.parametrize("host_path", [False, True])
+def test_loads_find_the_list_positions_room(fb, host_path):
+    """Recordings arrive after a recording of 2M events was mined: as many find
+    room as when it was only counted (mining keeps 8 MB of list positions for
+    the next call, fourteen of the arriving recordings), and mined again it
+    gives the same result."""
+    a, b = poisson_types(2, 2_000_000, 60, 83), poisson_types(3, 100_000, 60, 83)
+    bins = [(0, 500), (500, 1000)]
+
+    def mine(ctx, s):
+        res = ctx.mine_levelwise([s], bins, [20_000], 3)
+        out = [np.asarray(x) for k in (1, 2, 3) for x in res.level_arrays(0, k)]
+        res.free()
+        return out
+
+    def room(ctx):
+        got = []
+        with pytest.raises(fb.FemError) as e:
+            while len(got) < 1000:
+                got.append(ctx.load_stream(*b, 60))
+        assert e.value.status == fb.FEM_ERR_NOMEM
+        for x in got:
+            x.free()
+        return len(got)
+
+    ctx = fb.Context(0, hbm_budget_bytes=80 << 20)
+    s = ctx.load_stream(*a, 60)
+    ctx.count_episodes(s, fb.Cands(*random_cands(5, 300, 60, 3, bins)))
+    counted = room(ctx)
+    ctx.close()
+    ctx = fb.Context(0, hbm_budget_bytes=80 << 20)
+    if host_path:
+        ctx.set_tuning(level_graph=-1)
+    s = ctx.load_stream(*a, 60)
+    first = mine(ctx, s)
+    mined = room(ctx)
+    again = mine(ctx, s)
+    ctx.close()
+    assert mined >= counted - 7
+    assert all(np.array_equal(x, y) for x, y in zip(first, again))
