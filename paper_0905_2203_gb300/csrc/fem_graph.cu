@@ -758,13 +758,32 @@ struct FLevel {
 
 // Layout of the results the graph's last node writes to mapped host memory:
 // the status word, the counters, the per-recording offsets, the relevant-
-// event sums, then per level its frequent set (capacity-sized regions).
+// event sums, then the levels' frequent sets one after another, as long as
+// they fit.  The buffer holds every level at full capacity up to kPackRoom;
+// beyond that (a capacity of 2^20 candidates over 16 levels would pin 1.4 GB,
+// 0.4 s, for sets that are a thousandth of it) a set that finds no room is read
+// from the graph's own arrays instead.
+constexpr int64_t kPackRoom = (int64_t)64 << 20;
 struct PackLayout {
     int64_t o_ctr, o_coff, o_coff2, o_rel;  // byte offsets
     int64_t o_skip3;                        // level 3: candidates per recording the join bound dropped
-    int64_t o_lvl[FEM_MAX_NODES + 1];       // per level: types, then lo, hi, rec, counts
-    int64_t fcap[FEM_MAX_NODES + 1];        // per level capacity
+    int64_t o_levels, end;                  // the frequent sets, the buffer's end
 };
+
+// A level's region from byte `at`: types, lo, hi, rec, counts, each 8-byte
+// aligned; returns the byte after it.
+struct PackLevel {
+    int64_t types, lo, hi, rec, counts;
+};
+__host__ __device__ inline int64_t pack_level(int N, int64_t F, int64_t at, PackLevel *p) {
+    const int64_t e = (4 * F * (N - 1) + 7) / 8 * 8, c = (4 * F + 7) / 8 * 8;
+    p->types = at;
+    p->lo = at + (2 * F * N + 7) / 8 * 8;
+    p->hi = p->lo + e;
+    p->rec = p->hi + e;
+    p->counts = p->rec + c;
+    return p->counts + c;
+}
 
 __device__ __forceinline__ void pack_copy(char *dst, const char *src, int64_t bytes, int64_t t0, int64_t stride) {
     // 4-byte words (every region is a multiple of 4 bytes and 8-byte aligned)
@@ -784,23 +803,23 @@ __global__ void k_g_pack(const int *status, const int32_t *ctr, const int64_t *c
     pack_copy(out + lay.o_coff2, reinterpret_cast<const char *>(coff2), 8 * (int64_t)(n_recs + 1), t0, gs);
     pack_copy(out + lay.o_rel, reinterpret_cast<const char *>(rel), 8 * (int64_t)(L + 1), t0, gs);
     if (skip3) pack_copy(out + lay.o_skip3, reinterpret_cast<const char *>(skip3), 8 * (int64_t)n_recs, t0, gs);
+    int64_t at = lay.o_levels;
     for (int N = first; N <= L; ++N) {
-        const int64_t Fn = ctr[N * kCtr + 1], fc = lay.fcap[N];
+        const int64_t Fn = ctr[N * kCtr + 1];
+        PackLevel p;
+        const int64_t to = pack_level(N, Fn, at, &p);
+        if (to > lay.end) return;  // (no room for this set and those after it)
+        at = to;
         const FLevel f = F[N];
-        char *o = out + lay.o_lvl[N];
-        const int64_t tb = ((2 * fc * N) + 7) / 8 * 8, eb = 4 * fc * (N - 1);
-        // types: 2-byte entries, copied as bytes pairs
-        {
-            const uint16_t *s = f.types;
-            uint16_t *d = reinterpret_cast<uint16_t *>(o);
-            for (int64_t i = t0; i < Fn * N; i += gs) d[i] = s[i];
-        }
+        // types: 2-byte entries
+        uint16_t *d = reinterpret_cast<uint16_t *>(out + p.types);
+        for (int64_t i = t0; i < Fn * N; i += gs) d[i] = f.types[i];
         if (N > 1) {
-            pack_copy(o + tb, reinterpret_cast<const char *>(f.lo), 4 * Fn * (N - 1), t0, gs);
-            pack_copy(o + tb + eb, reinterpret_cast<const char *>(f.hi), 4 * Fn * (N - 1), t0, gs);
+            pack_copy(out + p.lo, reinterpret_cast<const char *>(f.lo), 4 * Fn * (N - 1), t0, gs);
+            pack_copy(out + p.hi, reinterpret_cast<const char *>(f.hi), 4 * Fn * (N - 1), t0, gs);
         }
-        pack_copy(o + tb + 2 * eb, reinterpret_cast<const char *>(f.rec), 4 * Fn, t0, gs);
-        pack_copy(o + tb + 2 * eb + 4 * fc, reinterpret_cast<const char *>(f.counts), 4 * Fn, t0, gs);
+        pack_copy(out + p.rec, reinterpret_cast<const char *>(f.rec), 4 * Fn, t0, gs);
+        pack_copy(out + p.counts, reinterpret_cast<const char *>(f.counts), 4 * Fn, t0, gs);
     }
 }
 
@@ -1126,13 +1145,13 @@ static int build_graph(GraphTail *g, TrackLists &lists, const std::vector<int32_
         lay.o_coff2 = take(8 * (int64_t)(n_recs + 1));
         lay.o_rel = take(8 * (int64_t)(L + 1));
         lay.o_skip3 = take(8 * (int64_t)std::max(n_recs, 1));
-        for (int N = first; N <= L; ++N) {
-            const int64_t fc = N == 1 ? std::max<int64_t>(tot1, 1) : cap;
-            lay.fcap[N] = fc;
-            const int64_t tb = ((2 * fc * N) + 7) / 8 * 8, eb = 4 * fc * (N - 1);
-            lay.o_lvl[N] = take(tb + 2 * eb + 8 * fc);
+        lay.o_levels = o;
+        for (int N = first; N <= L && o - lay.o_levels < kPackRoom; ++N) {
+            PackLevel p;
+            o = pack_level(N, N == 1 ? std::max<int64_t>(tot1, 1) : cap, o, &p);
         }
-        g->out_bytes = (size_t)o;
+        lay.end = std::min(o, lay.o_levels + kPackRoom);
+        g->out_bytes = (size_t)lay.end;
         // the mapped result buffer of an earlier graph of the context, when
         // large enough (pinning a large buffer costs more than a launch)
         if (ctx->pinned && ctx->pinned_bytes >= g->out_bytes) {
@@ -1654,6 +1673,7 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
     for (int N = std::max(first, 2); N <= max_size; ++N) out->relevant += (double)rel[N];
     // results
     out->levels.clear();
+    int64_t at = g->lay.o_levels;
     for (int N = first; N <= max_size; ++N) {
         const int32_t *c = &ctr[(size_t)N * kCtr];
         TailLevel tl;
@@ -1668,19 +1688,34 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
                 tl.skipped.assign(sk, sk + n_recs);
             }
         }
-        const int64_t Fn = c[1], fc = g->lay.fcap[N];
-        const char *o = ho + g->lay.o_lvl[N];
-        const int64_t tb = ((2 * fc * N) + 7) / 8 * 8, eb = 4 * fc * (N - 1);
-        const uint16_t *ty = reinterpret_cast<const uint16_t *>(o);
-        const int32_t *lo = reinterpret_cast<const int32_t *>(o + tb);
-        const int32_t *hi = reinterpret_cast<const int32_t *>(o + tb + eb);
-        const uint32_t *rc = reinterpret_cast<const uint32_t *>(o + tb + 2 * eb);
-        const uint32_t *ct = reinterpret_cast<const uint32_t *>(o + tb + 2 * eb + 4 * fc);
-        tl.types.assign(ty, ty + Fn * N);
-        tl.lo.assign(lo, lo + Fn * (N - 1));
-        tl.hi.assign(hi, hi + Fn * (N - 1));
-        tl.rec.assign(rc, rc + Fn);
-        tl.counts.assign(ct, ct + Fn);
+        const int64_t Fn = c[1], Fe = Fn * (N - 1);
+        PackLevel p;
+        at = pack_level(N, Fn, at, &p);
+        if (at <= g->lay.end) {
+            const uint16_t *ty = reinterpret_cast<const uint16_t *>(ho + p.types);
+            const int32_t *lo = reinterpret_cast<const int32_t *>(ho + p.lo);
+            const int32_t *hi = reinterpret_cast<const int32_t *>(ho + p.hi);
+            const uint32_t *rc = reinterpret_cast<const uint32_t *>(ho + p.rec);
+            const uint32_t *ct = reinterpret_cast<const uint32_t *>(ho + p.counts);
+            tl.types.assign(ty, ty + Fn * N);
+            tl.lo.assign(lo, lo + Fe);
+            tl.hi.assign(hi, hi + Fe);
+            tl.rec.assign(rc, rc + Fn);
+            tl.counts.assign(ct, ct + Fn);
+        } else {  // no room in the packed results
+            const FLevel &f = g->F[N];
+            tl.types.resize(Fn * N);
+            tl.lo.resize(Fe);
+            tl.hi.resize(Fe);
+            tl.rec.resize(Fn);
+            tl.counts.resize(Fn);
+            FEM_TRY(copy_out(ctx, tl.types.data(), f.types, 2 * Fn * N, 0));
+            FEM_TRY(copy_out(ctx, tl.lo.data(), f.lo, 4 * Fe, 0));
+            FEM_TRY(copy_out(ctx, tl.hi.data(), f.hi, 4 * Fe, 0));
+            FEM_TRY(copy_out(ctx, tl.rec.data(), f.rec, 4 * Fn, 0));
+            FEM_TRY(copy_out(ctx, tl.counts.data(), f.counts, 4 * Fn, 0));
+            FEM_CUDA_TRY(cudaStreamSynchronize(st));
+        }
         out->levels.push_back(std::move(tl));
         if ((N >= 2 && c[0] == 0) || Fn == 0) break;
     }

@@ -125,3 +125,31 @@ def test_loads_find_the_list_positions_room(fb, host_path):
     ctx.close()
     assert mined >= counted - 7
     assert all(np.array_equal(x, y) for x, y in zip(first, again))
+
+
+def test_frequent_sets_larger_than_the_packed_results(fb):
+    """Frequent pairs of 256 recordings that pass the 64 MB of mapped results
+    are read from the device arrays: the host-driven path's sets, level by
+    level."""
+    n_types, bins = 60, [(0, 2000), (2000, 4000), (4000, 6000), (6000, 8000)]
+    data = [poisson_types(100 + r, 1200, n_types, 10) for r in range(256)]
+    ctx = fb.Context(0)
+    st = [ctx.load_stream(t, x, n_types) for t, x in data]
+
+    def mine():
+        res = ctx.mine_levelwise(st, bins, [0] * len(st), 2)
+        out = [res.level_arrays(r, k) for r in range(len(st)) for k in (1, 2)]
+        tails = res.stats()["graph_tails"]
+        res.free()
+        return out, tails
+
+    try:
+        got, tails = mine()
+        ctx.set_tuning(level_graph=-1)
+        want, _ = mine()
+    finally:
+        ctx.close()
+    assert tails == 1
+    assert sum(len(x[4]) for x in want[1::2]) * 20 > 64 << 20
+    for a, b in zip(got, want):
+        assert all(np.array_equal(x, y) for x, y in zip(a, b))
