@@ -214,8 +214,13 @@ struct fem_ctx {
     // in use to its size; `cached` holds free blocks by size.
     std::mutex pool_mu;
     std::unordered_map<void *, size_t> live;
-    std::multimap<size_t, void *> cached;
+    struct Parked {
+        void *p;
+        uint64_t at;              // allocations made when it was parked
+    };
+    std::multimap<size_t, Parked> cached;
     size_t cached_bytes = 0;
+    uint64_t n_allocs = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     void *stage = nullptr;        // pinned staging of small counting calls
     size_t stage_bytes = 0;
