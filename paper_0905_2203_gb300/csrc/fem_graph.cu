@@ -1535,6 +1535,25 @@ struct Level2In {
 
 }  // namespace
 
+// Capacity of the first capture for several recordings: a quarter of all
+// ordered pairs x bins, within 2^20 and a sixteenth of the budget (a candidate
+// takes about 400 bytes and 24 a level), unless the last calls of this shape
+// (recordings, pairs of types, levels) needed half of kSmallCap at most.  An
+// overflow costs a second capture and the first run (8 recordings of 20k events
+// with 17,727 candidates: 3.5 ms with room for them, 11.7 ms from 4096); room
+// that nothing needs costs 0.2 to 1.2 ms (4 to 16 levels): the buffers, and the
+// single-block kernels that a small level is made for (8 recordings of 5000
+// events mined again, 8 levels: 660 us without them, 420 with).
+constexpr int64_t kSmallCap = 4096;
+
+static int64_t first_capacity(const fem_ctx *ctx, const std::string &shape, int64_t pairs, int max_size, int64_t cap) {
+    const auto seen = ctx->graph_seen.find(shape);
+    if (seen != ctx->graph_seen.end() && 2 * seen->second <= kSmallCap) return cap;
+    const int64_t room = (int64_t)(ctx->budget / 16 / (size_t)(400 + 24 * max_size));
+    while (cap < pairs / 4 && cap < (1 << 20) && 2 * cap <= room) cap <<= 1;
+    return cap;
+}
+
 // Runs levels first..max_size through the cached (or newly captured) graph.
 // *grow: a level had more candidates than the graph's capacity and nothing
 // else went wrong; the next call captures a larger one.
@@ -1553,20 +1572,19 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
     const bool jb_on = ctx->tuning.prepass == 0 || ctx->tuning.prepass == 1;
     const std::string key = graph_key(recs, blo, bhi, thr, max_size, first, prepass, coarse + 2 * (jb_on ? 1 : 0),
                                       ctx->tuning.kernel, ctx->tuning.track_last);
-    int64_t cap = 4096;
+    int64_t cap = kSmallCap;
     auto hint = ctx->graph_cap.find(key);
     const int64_t want = std::max<int64_t>(cap_min, hint != ctx->graph_cap.end() ? hint->second : 0);
     while (cap < want && cap < kMaxCap) cap <<= 1;
     if (cap < want) return FEM_OK;
-    // Several recordings: a quarter of all ordered pairs x bins to begin with
-    // (within 2^20; about 800 bytes a candidate), so that level 2 seldom
-    // overflows and the deepest level needs one larger capture at most; one
-    // recording starts at 4096, where the single-block kernels do its levels.
     const int64_t cap_need = cap;
+    std::string shape;
     if (n_recs >= kManyRecs) {
         int64_t pairs = 0;
         for (auto *s : recs) pairs += (int64_t)s->n_types * (s->n_types - 1) * (int64_t)blo.size();
-        while (cap < pairs / 4 && cap < (1 << 20)) cap <<= 1;
+        shape = std::to_string(n_recs) + '/' + std::to_string(pairs) + '/' + std::to_string(max_size) + '/' +
+                std::to_string(first);
+        cap = first_capacity(ctx, shape, pairs, max_size, cap);
     }
     GraphTail *g = nullptr;
     TrackLists lists(ctx);
@@ -1638,13 +1656,19 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
     const int64_t *coff2 = reinterpret_cast<const int64_t *>(ho + g->lay.o_coff2);
     const unsigned long long *rel = reinterpret_cast<const unsigned long long *>(ho + g->lay.o_rel);
     bool flagged = false, other = false;
-    int64_t need = 0;
+    int64_t need = 0, peak = 1;
     for (int N = std::max(first, 2); N <= max_size; ++N) {
         const int32_t *c = &ctr[(size_t)N * kCtr];
         if (c[2] != 0 || c[3] != 0) flagged = true;
         if ((c[2] & ~(kFlagCap | kFlagFreq)) != 0 || c[3] != 0) other = true;
         if (c[2] & kFlagCap) need = std::max<int64_t>(need, (int64_t)c[5] + 1);
         if (c[2] & kFlagFreq) need = std::max<int64_t>(need, 2 * g->cap);
+        peak = std::max<int64_t>(peak, c[0]);
+    }
+    if (!shape.empty()) {
+        if (ctx->graph_seen.size() >= 64) ctx->graph_seen.clear();
+        int64_t &seen = ctx->graph_seen[shape];
+        seen = std::max({seen / 2, peak, std::min(need, kMaxCap) / 2});
     }
     if (flagged) {
         // a capacity overflow grows the next capture, for several recordings
@@ -1720,6 +1744,11 @@ static int run_graph_once(fem_ctx *ctx, const std::vector<fem_stream *> &recs, c
         if ((N >= 2 && c[0] == 0) || Fn == 0) break;
     }
     *used = true;
+    // room that nothing needed: the next call is captured for what it was
+    if (!shape.empty() && g->cap > kFusedCap && cap_need == kSmallCap && 2 * ctx->graph_seen[shape] <= kSmallCap) {
+        ctx->graphs.erase(key);
+        delete g;
+    }
     return FEM_OK;
 }
 

@@ -207,6 +207,7 @@ struct fem_ctx {
     std::map<std::string, fem::TuneVal> tune;  // autotuner cache
     std::map<std::string, fem::GraphTail *> graphs;  // captured mining graphs
     std::map<std::string, int64_t> graph_cap;        // candidate capacity a graph key needed last time
+    std::map<std::string, int64_t> graph_seen;       // largest level of calls of a shape (first_capacity)
     std::string tune_path;                     // JSON file backing the cache ("" = memory only)
     // Allocation cache: freed device blocks kept for reuse (all of a
     // context's work is ordered on its stream, so a block freed after its

@@ -327,3 +327,38 @@ def test_wide_appends_take_the_shorter_way(fb, ctx, n_cand, chunk, n_types, grid
     n = min(len(ty), 2 * chunk)
     want = oracle_counts(ty[:n], tm[:n], offs, ct, lo, hi)
     assert np.array_equal(got, want) and want.max() > 0
+
+
+def test_captures_follow_what_calls_of_a_shape_needed(fb):
+    """Eight short recordings: after a first call that needed little, the next
+    is captured with the single-block kernels of small levels (fewer launches);
+    one that needs far more is captured again; results are the host-driven
+    path's throughout."""
+    n_types, bins = 60, [(0, 50), (50, 100), (100, 150), (150, 200)]
+    ctx = fb.Context(0)
+
+    def mine(st, thr):
+        res = ctx.mine_levelwise(st, bins, [thr] * 8, 3)
+        out = [res.level(r, N) for r in range(8) for N in (1, 2, 3)]
+        stats = res.stats()
+        res.free()
+        return out, stats
+
+    try:
+        launches = []
+        for seed, thr in ((0, 60), (1, 60), (2, 4), (3, 60), (4, 4)):
+            st = [ctx.load_stream(*synth.tiny_random_stream(0xCC0 + 16 * seed + i, 5000 + i, n_types, 100_000), n_types)
+                  for i in range(8)]
+            (a, s), (b, _) = mine(st, thr), mine(st, thr)
+            launches.append(s["kernel_launches"])
+            ctx.set_tuning(level_graph=-1)
+            h, _ = mine(st, thr)
+            ctx.reset_tuning()
+            assert a == h and b == h and s["graph_tails"] == 1
+            if thr == 4:
+                assert sum(len(c) for _, c in h[1::3]) > 4096
+            for x in st:
+                x.free()
+        assert launches[1] < launches[0]
+    finally:
+        ctx.close()
