@@ -362,3 +362,37 @@ def test_captures_follow_what_calls_of_a_shape_needed(fb):
         assert launches[1] < launches[0]
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("force", [0, 2])
+@pytest.mark.parametrize("rare,wide", [(1, 100_000), (3, 900), (40, 340), (40, 3_000), (700, 330)])
+def test_entries_that_serve_many_events(fb, ctx, rare, wide, force):
+    """A rare type followed by frequent ones at a wide edge: intervals of 15 to
+    5,000 events, cut by the next entry or by the edge, at both ends of a
+    chunk of entries; three to five nodes."""
+    n, n_types = 30_000, 6
+    ty, tm = synth.tiny_random_stream(95, n, n_types, 20 * n)
+    r = synth.Rng(96, rare)
+    ty = np.where(ty == 0, 1, ty)
+    ty[r.integers(0, len(ty) // 3, rare)] = 0
+    ok = np.concatenate([[True], np.diff(tm.astype(np.int64)) > 0])
+    ty, tm = ty[ok].astype(np.uint16), tm[ok]
+    n_cand = 120
+    sizes = r.integers(3, 5, n_cand)
+    offs = np.zeros(n_cand + 1, np.int64)
+    offs[1:] = np.cumsum(sizes)
+    ct = r.integers(1, n_types - 1, int(offs[-1])).astype(np.uint16)
+    ct[offs[:-1]] = 0
+    lo = r.integers(0, 30, int(offs[-1]) - n_cand).astype(np.int32)
+    hi = (lo + 1 + r.integers(0, wide, lo.size)).astype(np.int32)
+    hi[offs[:-1] - np.arange(n_cand)] += wide
+    want = oracle_counts(ty, tm, offs, ct, lo, hi)
+    st = ctx.load_stream(ty, tm, n_types)
+    ctx.set_tuning(track_last=force)
+    try:
+        got = ctx.count_episodes(st, fb.Cands(offs, ct, lo, hi)).astype(np.int64)
+    finally:
+        ctx.reset_tuning()
+    assert np.array_equal(got, want), np.nonzero(got != want)[0][:5]
+    assert want.max() > 0
+    st.free()
