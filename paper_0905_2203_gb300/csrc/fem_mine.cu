@@ -600,13 +600,12 @@ int MineGroup::gen_level2() {
     for (int r = 0; r < n_recs; ++r) ubp[r] = ub + ub_off[r];
     // by the per-type lists; without room for them (or over 2^30 events) each
     // event looks back over the stream
-    RecInfo *d_ri;
-    int64_t *d_cpre, *d_uboff;
-    uint32_t *d_ntp;
-    FEM_TRY(tmp.get(&d_ri, n_recs));
-    FEM_TRY(tmp.get(&d_cpre, n_recs + 1));
-    FEM_TRY(tmp.get(&d_uboff, n_recs + 1));
-    FEM_TRY(tmp.get(&d_ntp, n_recs));
+    // the bound's table in one copy: recordings, first items, rows, types
+    const size_t o_cpre = sizeof(RecInfo) * n_recs, o_uboff = o_cpre + 8 * (n_recs + 1),
+                 o_nt = o_uboff + 8 * (n_recs + 1);
+    std::vector<char> tab_h(o_nt + 4 * (size_t)n_recs);
+    char *tab;
+    FEM_TRY(tmp.get(&tab, tab_h.size()));
     PositionsHold positions(recs);
     int by_lists = FEM_OK;
     for (int r = 0; r < n_recs && by_lists == FEM_OK; ++r) by_lists = stream_bytype(ctx, recs[r], true);
@@ -614,8 +613,9 @@ int MineGroup::gen_level2() {
     if (by_lists == FEM_OK) {
         PairBoundArgs pb{};
         pb.chunk = pair_bound_chunk(ctx->n_sm, events);
-        std::vector<int64_t> cpre(n_recs + 1, 0);
-        std::vector<RecInfo> ri(n_recs);
+        RecInfo *ri = reinterpret_cast<RecInfo *>(tab_h.data());
+        int64_t *cpre = reinterpret_cast<int64_t *>(tab_h.data() + o_cpre);
+        cpre[0] = 0;
         for (int r = 0; r < n_recs; ++r) {
             const bool any = prev.h_off[r + 1] - prev.h_off[r] >= 2;
             cpre[r + 1] = cpre[r] + (any ? (recs[r]->n + pb.chunk - 1) / pb.chunk : 0);
@@ -626,17 +626,16 @@ int MineGroup::gen_level2() {
             ri[r].freq = recs[r]->d_freq;
             recinfo_lists(ri[r], recs[r]);
         }
-        FEM_CUDA_TRY(cudaMemcpyAsync(d_ri, ri.data(), sizeof(RecInfo) * n_recs, cudaMemcpyHostToDevice, st));
-        FEM_CUDA_TRY(cudaMemcpyAsync(d_cpre, cpre.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
-        FEM_CUDA_TRY(cudaMemcpyAsync(d_uboff, ub_off.data(), 8 * (n_recs + 1), cudaMemcpyHostToDevice, st));
-        FEM_CUDA_TRY(cudaMemcpyAsync(d_ntp, nth.data(), 4 * n_recs, cudaMemcpyHostToDevice, st));
-        pb.ri = d_ri;
+        std::copy(ub_off.begin(), ub_off.end(), reinterpret_cast<int64_t *>(tab_h.data() + o_uboff));
+        std::copy(nth.begin(), nth.end(), reinterpret_cast<uint32_t *>(tab_h.data() + o_nt));
+        FEM_CUDA_TRY(cudaMemcpyAsync(tab, tab_h.data(), tab_h.size(), cudaMemcpyHostToDevice, st));
+        pb.ri = reinterpret_cast<RecInfo *>(tab);
         pb.n_recs = n_recs;
-        pb.cpre = d_cpre;
+        pb.cpre = reinterpret_cast<int64_t *>(tab + o_cpre);
         pb.n_items = cpre[n_recs];
-        pb.nt = d_ntp;
+        pb.nt = reinterpret_cast<uint32_t *>(tab + o_nt);
         pb.thr = d_thr;
-        pb.ub_off = d_uboff;
+        pb.ub_off = reinterpret_cast<int64_t *>(tab + o_uboff);
         pb.blo = d_blo;
         pb.bhi = d_bhi;
         pb.nb = nb;

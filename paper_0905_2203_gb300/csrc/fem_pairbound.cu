@@ -36,7 +36,15 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kPbThreads = 256;
 constexpr int kPbLanes = 8;                  // lanes of an event ...
 constexpr unsigned kPbLasts = 0x80808080u;   // ... and the last lane of each group
+constexpr int kPbWarps = kPbThreads / 32;
 constexpr int kPbMinChunk = 256, kPbMaxChunk = 4096;  // list positions per block
+
+// A warp's share of a chunk, at most its lanes and a multiple of the events it
+// takes side by side.
+__host__ __device__ constexpr int pair_bound_batch(int chunk) {
+    const int b = chunk / kPbWarps;
+    return b >= 32 ? 32 : b <= 32 / kPbLanes ? 32 / kPbLanes : b / (32 / kPbLanes) * (32 / kPbLanes);
+}
 
 // Which bin a distance falls into.  NB = 0: nb adjacent bins of one width (the
 // usual case), found by one multiplication; the newest-event condition is
@@ -85,6 +93,7 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
     extern __shared__ uint32_t s_row[];  // counter of (bin k, type b) at k * nt + b: neighbouring types, other banks
     constexpr int kSide = 32 / G;        // events a warp takes side by side
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int batch = pair_bound_batch(a.chunk);  // list positions a warp takes at a time
     Bins<NB> bins(a);
     const int32_t all = a.nb * (int32_t)a.width;  // (NB = 0) the windows' whole width
     for (int64_t item = blockIdx.x; item < a.n_items; item += gridDim.x) {
@@ -114,12 +123,12 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
             if (ri.freq[E] > a.thr[r]) {
                 for (int w = threadIdx.x; w < words; w += kPbThreads) s_row[w] = 0;
                 __syncthreads();
-                for (int base = p + warp * 32; base < p1; base += kPbThreads) {
+                for (int base = p + warp * batch; base < p1; base += kPbWarps * batch) {
                     const int q = base + lane;
                     const int32_t t = q < p1 ? tl[q] : 0;
                     const int32_t at = q < p1 ? tp[q] : 0;
                     const uint32_t gap = q < p1 && q + 1 < te ? (uint32_t)(tl[q + 1] - t) : 0xFFFFFFFFu;
-                    const int cnt = min(32, p1 - base);
+                    const int cnt = min(batch, p1 - base);
                     for (int e = 0; e < cnt; e += kSide) {
                         const int src = e + lane / G;  // below 32: e is a multiple of kSide
                         const int32_t ti = __shfl_sync(kFull, t, src);
@@ -187,9 +196,17 @@ __global__ void __launch_bounds__(kPbThreads, NB == 0 ? 6 : 4) k_pair_bound(Pair
 // Chunk length (list positions per block): about four blocks per resident
 // one over all recordings, so that the last wave is short, between 256 (a
 // batch of 32 events per warp) and 4096 (the row's flush is then under 1% of
-// the updates).
+// the updates).  Fewer events than fill the resident blocks that way are dealt
+// out over them, down to 4 events per warp: with chunks of 256, 5000 events of
+// 500 types (eight uneven bins, 50 events in their windows) make 20 blocks of
+// 25 rows each: the whole mining call takes 402 us, 163 with chunks of 32.
 int pair_bound_chunk(int n_sm, int64_t events) {
-    const int64_t c = events / ((int64_t)n_sm * 8 * 4);
+    const int64_t resident = (int64_t)n_sm * 8;
+    if (events < resident * kPbMinChunk) {
+        const int64_t c = (events / resident + 31) / 32 * 32;
+        return (int)std::max<int64_t>(32, std::min<int64_t>(kPbMinChunk, c));
+    }
+    const int64_t c = events / (resident * 4);
     return (int)std::max<int64_t>(kPbMinChunk, std::min<int64_t>(kPbMaxChunk, (c + 255) / 256 * 256));
 }
 

@@ -396,3 +396,34 @@ def test_entries_that_serve_many_events(fb, ctx, rare, wide, force):
     assert np.array_equal(got, want), np.nonzero(got != want)[0][:5]
     assert want.max() > 0
     st.free()
+
+
+@pytest.mark.parametrize("host_path", [False, True])
+@pytest.mark.parametrize("bins", ["eight", "overlap", "gaps"])
+@pytest.mark.parametrize("n,n_types", [(33, 16), (700, 300), (5000, 900), (41_000, 500)])
+def test_pair_bound_over_few_events_of_many_types(fb, ctx, n, n_types, bins, host_path):
+    """Chunks of 32 list positions and four events a warp: lists of a few
+    events, chunks that end inside one."""
+    ty, tm = synth.tiny_random_stream(33, n, n_types, 3 * n)
+    bl, thr = PAIR_BINS[bins], max(1, n // (2 * n_types))
+    freq = np.bincount(ty, minlength=n_types)
+    keep = np.nonzero(freq > thr)[0]
+    ub = np.zeros((n_types, n_types, len(bl)), np.int64)
+    for k, (lo, hi) in enumerate(bl):  # pairs of (b event, type) with an event of it in the window
+        first = np.searchsorted(tm, tm.astype(np.int64) - hi, side="left")
+        last = np.searchsorted(tm, tm.astype(np.int64) - lo, side="left")
+        for j in range(len(tm)):
+            ub[np.unique(ty[first[j]:last[j]]), ty[j], k] += 1
+    pairs = np.zeros((n_types, n_types), bool)
+    pairs[np.ix_(keep, keep)] = True
+    np.fill_diagonal(pairs, False)
+    kept = int((pairs[:, :, None] & (ub > thr)).sum())
+    st = ctx.load_stream(ty, tm, n_types)
+    ctx.set_tuning(level_graph=-1 if host_path else 0)
+    try:
+        res = ctx.mine_levelwise([st], bl, [thr], 2)
+    finally:
+        ctx.reset_tuning()
+    assert res.stats()["candidates_counted"] == kept
+    res.free()
+    st.free()
