@@ -138,6 +138,25 @@ void drop_positions(fem_ctx *ctx, fem_stream *s) {
     v.erase(std::remove(v.begin(), v.end(), s), v.end());
 }
 
+void drop_lists(fem_ctx *ctx, fem_stream *s) {
+    graph_cache_forget(ctx, s);
+    drop_positions(ctx, s);
+    const size_t nt = s->n_types;
+    if (s->d_tidx) {
+        const size_t b = sizeof(int32_t) * nt * (size_t)(s->tcells + 1);
+        dev_free(ctx, s->d_tidx, b);
+        s->d_tidx = nullptr;
+        s->bytes -= b;
+    }
+    if (s->d_ttime) {
+        dev_free(ctx, s->d_toff, sizeof(int64_t) * (nt + 1));
+        dev_free(ctx, s->d_ttime, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
+        s->d_toff = nullptr;
+        s->d_ttime = nullptr;
+        s->bytes -= sizeof(int64_t) * (nt + 1) + sizeof(int32_t) * s->n;
+    }
+}
+
 // Takes back what is only kept for later calls: the entry lists, then the list
 // positions.  Returns whether anything came back.
 static bool give_back(fem_ctx *ctx) {
@@ -754,10 +773,7 @@ void fem::stream_free_unlocked(fem_stream *s) {
     for (auto &kv : s->dens) dev_free(ctx, kv.second, sizeof(uint32_t) * s->n_types);
     for (auto &kv : s->segs) dev_free(ctx, kv.second, sizeof(int64_t) * (kv.first + 1));
     coarse_free(ctx, s);
-    if (s->d_toff) dev_free(ctx, s->d_toff, sizeof(int64_t) * (s->n_types + 1));
-    if (s->d_ttime) dev_free(ctx, s->d_ttime, sizeof(int32_t) * std::max<int64_t>(s->n, 1));
-    drop_positions(ctx, s);
-    if (s->d_tidx) dev_free(ctx, s->d_tidx, sizeof(int32_t) * (size_t)s->n_types * (size_t)(s->tcells + 1));
+    drop_lists(ctx, s);
     delete s;
 }
 

@@ -1857,7 +1857,7 @@ struct CountCall {
     int64_t n_edges = 0;                 // entries of lo
     int mode = 0;                        // 0 exact, 1 plain, 2 relaxed
     double seg_div = 1.0;                // fallback rounds divide the segment count
-    bool force_tiled = false;            // last fallback round: tiled kernel, one segment
+    bool force_tiled = false;            // last fallback round, or no room for lists: tiled kernel
     int64_t sumhi = -1;                  // largest sum of an episode's upper bounds (-1: not known)
     bool plt_ok = false;                 // grid-wide local tracking may count this call (or its recounts)
     fem_stats stats{};
@@ -2009,7 +2009,7 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
     for (int r = 0; r < n_recs; ++r) {
         nt_h[r] = cc.recs[r]->n_types;
         if (track) continue;  // window densities size rings; local tracking keeps none
-        FEM_TRY(stream_densities(ctx, cc.recs[r], lov));
+        if (!cc.force_tiled) FEM_TRY(stream_densities(ctx, cc.recs[r], lov));  // (all at once, by the lists)
         for (size_t j = 0; j < lov.size(); ++j) {
             uint32_t *d = nullptr;
             FEM_TRY(stream_density(ctx, cc.recs[r], lov[j], &d));
@@ -2752,7 +2752,7 @@ static int run_count(CountCall &cc, const int32_t *subset, int64_t n_sub, int fo
     const int kern = cc.ctx->tuning.kernel;
     bool plt = kern >= 4 && kern <= 6;
     cc.plt_ok = false;
-    if (kern == 0 && n_sub <= kPltMaxCands && cc.mode != 1 && force_segments == 0) {
+    if (kern == 0 && !cc.force_tiled && n_sub <= kPltMaxCands && cc.mode != 1 && force_segments == 0) {
         int64_t nmax = 0;
         bool lists = true;
         for (auto *r : cc.recs) {
@@ -3120,19 +3120,32 @@ static int count_entry(fem_ctx *ctx, const fem_stream *const *recs, int n_recs, 
         ctx->last = cc.stats;
         return FEM_OK;
     };
-    if (n_recs == 1) {
-        bool used = false;
-        FEM_TRY(count_quick(ctx, cc.recs[0], c, counts, out_is_device, mode, cc, &used));
-        if (used) return finish();
+    auto count_all = [&]() -> int {
+        if (n_recs == 1 && !cc.force_tiled) {
+            bool used = false;
+            FEM_TRY(count_quick(ctx, cc.recs[0], c, counts, out_is_device, mode, cc, &used));
+            if (used) return FEM_OK;
+        }
+        FEM_TRY(stage_candidates(ctx, c, cc, n_recs > 1 ? rec_id : nullptr, n_recs));
+        void *pc = nullptr;
+        FEM_TRY(scratch(ctx, kSlotCounts, 4 * c->n_cand, &pc));
+        cc.counts = static_cast<uint32_t *>(pc);
+        FEM_TRY(run_count(cc, nullptr, c->n_cand, 0));
+        FEM_TRY(copy_out(ctx, counts, cc.counts, 4 * c->n_cand, out_is_device));
+        FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        return FEM_OK;
+    };
+    int st = count_all();
+    if (st == FEM_ERR_NOMEM && ctx->tuning.kernel == 0 && mode != 1) {
+        // the recordings' lists fitted, but not what counting over them takes:
+        // once more without them, by the tiled kernel
+        for (auto *r : cc.recs) drop_lists(ctx, r);
+        cc.stats = fem_stats{};
+        cc.count_ms = 0.f;
+        cc.force_tiled = true;
+        st = count_all();
     }
-    FEM_TRY(stage_candidates(ctx, c, cc, n_recs > 1 ? rec_id : nullptr, n_recs));
-    void *pc = nullptr;
-    FEM_TRY(scratch(ctx, kSlotCounts, 4 * c->n_cand, &pc));
-    cc.counts = static_cast<uint32_t *>(pc);
-    FEM_TRY(run_count(cc, nullptr, c->n_cand, 0));
-    FEM_TRY(copy_out(ctx, counts, cc.counts, 4 * c->n_cand, out_is_device));
-    FEM_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    return finish();
+    return st == FEM_OK ? finish() : st;
 }
 
 // Appended events: 1-node episodes (cand[n_slots ..]) gain their type's new

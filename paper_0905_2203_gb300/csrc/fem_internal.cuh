@@ -331,6 +331,9 @@ class PositionsHold {
 };
 // Gives the positions of a recording that is not held back (if it has any).
 void drop_positions(fem_ctx *ctx, fem_stream *s);
+// Gives back a recording's lists with their positions and time index, and the
+// mining graphs captured on it; no launch that reads them is being prepared.
+void drop_lists(fem_ctx *ctx, fem_stream *s);
 
 // Budget left for those lists: what is free and what they hold.
 inline size_t track_room(const fem_ctx *ctx) {

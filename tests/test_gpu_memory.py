@@ -153,3 +153,30 @@ def test_frequent_sets_larger_than_the_packed_results(fb):
     assert sum(len(x[4]) for x in want[1::2]) * 20 > 64 << 20
     for a, b in zip(got, want):
         assert all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+def test_counts_wherever_the_recording_fits(fb):
+    """Once a budget holds a recording of 1M events and its candidates, every
+    larger one counts: room for the per-type lists or their time index but not
+    for what counting over them takes is no reason to refuse."""
+    ty, tm = poisson_types(4, 1_000_000, 60, 83)
+    r = np.random.default_rng(5)
+    offs = np.concatenate([[0], np.cumsum(r.integers(2, 6, 200))]).astype(np.int64)
+    ct = r.integers(0, 60, int(offs[-1])).astype(np.uint16)
+    lo = (r.integers(0, 4, len(ct) - 200) * 500).astype(np.int32)
+    cands = offs, ct, lo, (lo + 500).astype(np.int32)
+    want, _ = oracle.count_many(ty, tm, *cands)
+    done = []
+    for kb in range(7_500, 24_000, 500):
+        ctx = fb.Context(0, hbm_budget_bytes=kb << 10)
+        try:
+            st = ctx.load_stream(ty, tm, 60)
+            got = ctx.count_episodes(st, fb.Cands(*cands)).astype(np.int64)
+            assert np.array_equal(got, want.astype(np.int64)), kb
+            done.append(kb)
+        except fb.FemError as e:
+            assert e.status == fb.FEM_ERR_NOMEM
+        finally:
+            ctx.close()
+    assert done == list(range(done[0], 24_000, 500)), done
+    assert done[0] <= 12_000  # (6 MB; its lists and their index take 8 MB more)
