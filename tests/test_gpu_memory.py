@@ -180,3 +180,27 @@ def test_counts_wherever_the_recording_fits(fb):
             ctx.close()
     assert done == list(range(done[0], 24_000, 500)), done
     assert done[0] <= 12_000  # (6 MB; its lists and their index take 8 MB more)
+
+
+def test_pair_bound_without_room_for_list_positions(fb):
+    """13 MB hold a recording of 1M events (6 MB) and its lists (4 MB), not
+    their positions (4 MB): the pair bound looks back over the stream instead
+    and drops the same candidates."""
+    ty, tm = poisson_types(6, 1_000_000, 60, 83)
+    bins, thr = [(0, 500), (500, 1000), (1000, 1500)], 3_000
+
+    def mine(budget):
+        ctx = fb.Context(0, hbm_budget_bytes=budget)
+        try:
+            res = ctx.mine_levelwise([ctx.load_stream(ty, tm, 60)], bins, [thr], 2)
+            out = [np.asarray(x) for k in (1, 2) for x in res.level_arrays(0, k)]
+            stats = res.stats()
+            res.free()
+            return out, stats
+        finally:
+            ctx.close()
+
+    (got, a), (want, b) = mine(13 << 20), mine(0)
+    assert all(np.array_equal(x, y) for x, y in zip(got, want))
+    assert a["candidates_pruned"] == b["candidates_pruned"] > 0
+    assert a["graph_tails"] == 0 and b["graph_tails"] == 1

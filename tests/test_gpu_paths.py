@@ -427,3 +427,75 @@ def test_pair_bound_over_few_events_of_many_types(fb, ctx, n, n_types, bins, hos
     assert res.stats()["candidates_counted"] == kept
     res.free()
     st.free()
+
+
+JOIN_BINS = {
+    "five": [(6 * k, 6 * k + 6) for k in range(5)],
+    "eight": [(4 * k, 4 * k + 4) for k in range(8)],
+    "gaps": [(3, 9), (14, 15), (20, 31)],
+    "overlap": [(0, 12), (5, 30), (29, 31)],
+    "overlap_six": [(0, 12), (2, 5), (5, 30), (8, 9), (29, 31), (30, 33)],
+}
+
+
+@pytest.mark.parametrize("bins", sorted(JOIN_BINS))
+@pytest.mark.parametrize("recs", [1, 3])
+def test_join_bound_over_any_bins(fb, ctx, recs, bins):
+    """Level 3 with the join bound over five and more, gapped and overlapping
+    bins: the oracle miner's sets, and fewer exact counts than without it."""
+    n_types, bl = 16, JOIN_BINS[bins]
+    thr = [{"five": 27, "eight": 19, "overlap": 60}.get(bins, 15)] * recs
+    data = []
+    for i in range(recs):
+        ty, tm = synth.tiny_random_stream(0xB1 + i, 2600 + 64 * i, n_types, 5200)
+        first = tm[ty == 0].astype(np.int64)  # a planted chain 0 -> 1 -> 2, seven ticks each
+        key = np.unique(np.concatenate([tm.astype(np.int64) * 16 + ty, (first + 7) * 16 + 1, (first + 14) * 16 + 2]))
+        data.append(((key % 16).astype(np.uint16), (key // 16).astype(np.int32)))
+    st = [ctx.load_stream(ty, tm, n_types) for ty, tm in data]
+
+    def mine():
+        res = ctx.mine_levelwise(st, bl, thr, 3)
+        out = [res.level(r, N) for r in range(recs) for N in (1, 2, 3)]
+        stats = res.stats()
+        res.free()
+        return out, stats
+
+    mine()  # (the first run may find a level larger than its capture)
+    got, bounded = mine()
+    ctx.set_tuning(prepass=2)
+    try:
+        mine()
+        plain, exact = mine()
+    finally:
+        ctx.reset_tuning()
+    for r, (ty, tm) in enumerate(data):
+        want = oracle.mine_levelwise(ty, tm, n_types, bl, thr[r], 3)
+        for N in (1, 2, 3):
+            assert list(zip(*got[3 * r + N - 1])) == want[N], (r, N)
+    assert plain == got
+    assert bounded["graph_tails"] == exact["graph_tails"] == 1 and len(got[2][0]) > 0
+    assert bounded["candidates_counted"] < exact["candidates_counted"]
+    for s in st:
+        s.free()
+
+
+@pytest.mark.parametrize("hi,route", [(20, "segments"), (700, "recounts"), (9_000, "grid")])
+def test_few_episodes_routes(fb, ctx, hi, route):
+    """At most 256 episodes over more than 2^20 events, half of them ten times
+    denser: segments; segments with episodes that run out of entry classes in
+    the dense half and are counted again; grid-wide at once."""
+    n, n_types = 1_100_000, 8
+    r = np.random.default_rng(12)
+    tm = np.cumsum(r.integers(1, np.where(np.arange(n) < n // 2, 200, 20))).astype(np.int32)
+    ty = r.integers(0, n_types, n).astype(np.uint16)
+    offs = np.arange(0, 4 * 30 + 1, 4, dtype=np.int64)
+    ct = r.integers(0, n_types, 4 * 30).astype(np.uint16)
+    lo = (r.integers(0, 2, 3 * 30) * hi // 2).astype(np.int32)
+    up = np.full(3 * 30, hi, np.int32)
+    st = ctx.load_stream(ty, tm, n_types)
+    got = ctx.count_episodes(st, fb.Cands(offs, ct, lo, up)).astype(np.int64)
+    s = ctx.last_stats()
+    st.free()
+    assert np.array_equal(got, oracle_counts(ty, tm, offs, ct, lo, up)) and got.max() > 0
+    assert (s["sparse_launches"] == 0) == (route == "grid")
+    assert (s["fallback_recounts"] > 0) == (route == "recounts")
