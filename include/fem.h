@@ -182,7 +182,14 @@ typedef struct {
 
 /* Creates a context on CUDA device `device`.
  *   hbm_budget_bytes  upper bound on device memory the context may hold
- *                     (streams + scratch); 0 = 90% of the device's free memory
+ *                     (streams + scratch); 0 = 90% of the device's free memory.
+ *                     The context keeps scratch for later calls, also after a
+ *                     stream is freed: per-warp entry lists (at most a quarter
+ *                     of the budget), list positions of mined streams (4 bytes
+ *                     an event) and freed blocks (at most a quarter of the
+ *                     budget and 8 GB).  A call that finds no room takes them
+ *                     back; other users of the GPU get them with
+ *                     fem_ctx_destroy
  *   cuda_stream       a cudaStream_t to run on, or NULL for a stream the
  *                     context creates and owns
  * On success *out owns the context; free it with fem_ctx_destroy. */

@@ -852,9 +852,9 @@ __global__ void k_prep(PrepArgs a) {
 // first key-k element goes, and k_part_scatter assigns stable positions: each
 // of the block's warps takes a contiguous part, counts its keys, starts after
 // the warps before it and walks its elements 32 at a time (equal keys of a
-// step ranked by a match).  One warp per block walked all 4096 alone, a chain
-// of 128 steps: the lists of 1M events took 86 us and a gather of 8 us, those
-// of 20M events 243 and 117 us; now 20 and 289 us, times written directly.
+// step ranked by a match), a chain of 16 steps.  The lists of 1M events take
+// 20 us, those of 20M events 289 us (one warp per block, 128 steps, and the
+// times gathered after it: 94 and 360 us).
 constexpr int kPartBlock = 4096;
 constexpr int kPartWarps = 8;
 
@@ -1031,9 +1031,8 @@ int scan_exclusive(cudaStream_t st, int32_t *data, int64_t m, int32_t *tmp, int3
 //
 // One block per boundary: its threads take the up to 8193 places side by side
 // (coalesced reads) and reduce to the largest gap, the first place among
-// equal ones.  One thread per boundary walked them one after another, a chain
-// of 8193 loads that held the whole launch: 360-560 us for a 1M-event
-// recording cut into 130 segments.
+// equal ones (one thread per boundary, a chain of 8193 loads: 360-560 us for a
+// 1M-event recording cut into 130 segments).
 constexpr int kSegThreads = 256;
 
 // `base` is added to every boundary (a part of a recording that starts there).
@@ -1891,8 +1890,9 @@ constexpr int64_t kPltMinEvents = 1 << 20;
 // recording, first node, second node and first edge, so that one item tracks
 // the common two-node prefix once for all of its episodes.  That prefix is the
 // longest step (every event of two types; later nodes run over the few
-// entries left): 200k episodes of 2-8 nodes, 60 types, 4M events, 14 episodes
-// a group.  The sort (three or four partition passes) and its two host reads
+// entries left): of 200k episodes of 2-8 nodes over 60 types and four bins
+// twelve share one on average, and with a new group every kTrackPairMax slots
+// an item holds seven; two-node episodes are items of their own.  The sort (three or four partition passes) and its two host reads
 // cost 0.4 ms: for sets of at least kPairMinSlots episodes and kPairMinWork
 // relevant events (about 2.5 ms of counting).
 constexpr int64_t kPairMinSlots = 1 << 14;
@@ -2168,8 +2168,8 @@ static int count_core(CountCall &cc, const int32_t *subset, int64_t n_work, int 
                 work += (double)c * (double)cc.recs[r]->n;
             }
             seg_len = std::max(1.0, work / desired) / seg_mult;
-            // an item is a whole group: four items' worth of segments per
-            // group keep the launch's tail short
+            // an item is a whole group: kTrackPairCut items' worth of segments
+            // per group keep the launch's tail short
             if (pl.track && pair_groups) seg_len /= kTrackPairCut * pair_avg;
         } else {
             const size_t sm = tiled_smem_rt(pl.nclass, K, pl.R, T);

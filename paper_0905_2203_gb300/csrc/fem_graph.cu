@@ -463,10 +463,10 @@ __global__ void __launch_bounds__(1024, 1)
 // for local tracking and levels that one block keeps fast: the join (N >= 3;
 // level 2's candidates are there already), the CSR index, the prefix groups
 // (N >= 3), the segmentation by the largest of them, the segment starts, the
-// item numbering and the work counter.  As eleven launches these took longer
-// than the counting they prepare: a level of a mid-size recording has some
-// twenty candidates (mining 1.07M events, 128 types, six levels: 700 -> 539
-// us; a 5k-event recording, four levels: 360 -> 291 us).
+// item numbering and the work counter.  A level of a mid-size recording has
+// some twenty candidates, and the launches that prepare it would outlast their
+// counting (mining 1.07M events, 128 types, six levels: 539 us, with eleven
+// launches a level 700; a 5k-event recording, four levels: 291 and 360 us).
 struct SmallLevel {
     int N;
     const uint16_t *ft;              // level N - 1's frequent set (N >= 3)

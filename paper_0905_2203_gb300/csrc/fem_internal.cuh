@@ -87,13 +87,15 @@ constexpr int kTrackWarps = 8;           // warps per block
 constexpr int kTrackMaxBlocksPerSm = 6;  // resident blocks per SM the grid asks for (40 registers)
 constexpr int kTrackGroupMax = 64;       // episodes per prefix group (a new group every 64 slots)
 // Groups of a common two-node prefix: episodes per group and segments per
-// group (this times its episodes).  200k episodes over 4M events, (16, 12):
-// (8, 4) 122 ms, (16, 4) 148, (8, 12) 96, (16, 12) 99, (32, 12) 101,
-// (16, 40) 97: a group of frequent chains outlasts the launch when cut coarsely.
+// group (this times its episodes): a group of frequent chains outlasts the
+// launch when cut coarsely.  200k episodes over 4M events: with 12, groups of 8
+// 73.3 ms, of 16 74.1, of 32 80.7 (a set whose episodes share their prefix more
+// often gains from the longer ones); with an earlier state of the kernel (16, 4)
+// 148 ms, (16, 12) 99, (16, 40) 97.
 constexpr int kTrackPairMax = 16;
 constexpr double kTrackPairCut = 12.0;
 constexpr int kTrackMinSeg = 8192;       // shortest segment (events) of a local-tracking item
-constexpr int kTrackEntryRatio = 2;      // last node by entries when events > this x entries
+constexpr int kTrackEntryRatio = 2;      // a node by entries when its events > this x entries
 constexpr int kTrackEntrySlots = 2;      // entries per lane of the entry-driven last node step
 struct TrackArgs {
     const RecInfo *rinfo;

@@ -79,8 +79,7 @@ __global__ void k_jb_base(JoinBoundArgs a) {
 // that of its first frequent bin.  64 recordings of 60 types (55M events, four
 // bins): 12 ms bin by bin, 8 ms so; one 1.07M-event recording 72 -> 51 us, with
 // chunks of a 64th of the longest list (2048 events: 212 us, too few items).
-// NB: bins held in registers (0: in shared
-// memory, up to 32).
+// NB: bins held in registers (0: in shared memory, up to 32).
 template <int NB>
 __global__ void __launch_bounds__(256, 6) k_jb_bits(JoinBoundArgs a) {
     __shared__ int32_t s_lo[kJoinBoundMaxBins], s_hi[kJoinBoundMaxBins];

@@ -243,8 +243,8 @@ __device__ __forceinline__ bool joins(const uint16_t *ft, const int32_t *fl, con
     return true;
 }
 
-// One warp per alpha, its partners tested 32 at a time: a thread per alpha
-// walked them one by one (3000 frequent pairs: 324 us for the write).
+// One warp per alpha, its partners tested 32 at a time (a thread per alpha:
+// 324 us for the write of 3000 frequent pairs' candidates).
 __global__ void k_join_count(const uint16_t *ft, const int32_t *fl, const int32_t *fh, const uint32_t *frec,
                              const int64_t *f_off, int M, int64_t F, int32_t *cnt) {
     const int lane = threadIdx.x & 31;

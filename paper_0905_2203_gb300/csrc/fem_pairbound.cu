@@ -19,11 +19,11 @@
 // type's row of the table (n_types x bins counters), which it keeps in shared
 // memory and adds to the global table once; eight lanes take one event and
 // read the events after it side by side, so the loads are coalesced and no
-// per-thread bitset is needed.  Whole-call times with 8 lanes an event for
-// every window, with 32 from 12 events on, and before: 20M events from host
-// memory (128 events a window) 6.2, 7.1 and 29.5 ms; 1.07M events of 128 types
-// (21 events) 536, 560 and 870 us.  It issues on about 80% of the cycles at 36
-// registers (6 blocks per SM); the shared-memory pipe is 58% busy.
+// per-thread bitset is needed.  Mining calls by this kernel, with 32 lanes an
+// event from 12 events on, and by the look-back: 20M events from host memory
+// (128 events a window) 6.1, 7.1 and 29.5 ms; 1.07M events of 128 types (21
+// events) 536, 560 and 870 us.  At 36 registers (6 blocks per SM) it issues on
+// 67% of the cycles over the latter.
 #include <algorithm>
 
 #include "fem_internal.cuh"
