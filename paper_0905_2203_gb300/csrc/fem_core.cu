@@ -219,14 +219,18 @@ void dev_free(fem_ctx *ctx, void *p, size_t bytes) {
     }
     ctx->used -= sz;
     const size_t limit = pool_limit(ctx);
-    for (auto i = ctx->cached.begin(); ctx->cached_bytes + sz > limit && i != ctx->cached.end();) {
-        if (ctx->n_allocs - i->second.at < kPoolStale) {
-            ++i;
-            continue;
+    if (ctx->cached_bytes + sz > limit && ctx->n_allocs - ctx->parked_from >= kPoolStale) {
+        ctx->parked_from = ctx->n_allocs;
+        for (auto i = ctx->cached.begin(); i != ctx->cached.end();) {
+            if (ctx->cached_bytes + sz <= limit || ctx->n_allocs - i->second.at < kPoolStale) {
+                ctx->parked_from = std::min(ctx->parked_from, i->second.at);
+                ++i;
+                continue;
+            }
+            cudaFree(i->second.p);
+            ctx->cached_bytes -= i->first;
+            i = ctx->cached.erase(i);
         }
-        cudaFree(i->second.p);
-        ctx->cached_bytes -= i->first;
-        i = ctx->cached.erase(i);
     }
     if (ctx->cached_bytes + sz <= limit) {
         ctx->cached.emplace(sz, fem_ctx::Parked{p, ctx->n_allocs});

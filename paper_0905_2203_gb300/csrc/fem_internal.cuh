@@ -224,6 +224,7 @@ struct fem_ctx {
     std::multimap<size_t, Parked> cached;
     size_t cached_bytes = 0;
     uint64_t n_allocs = 0;
+    uint64_t parked_from = 0;     // no parked block is older than this
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     void *stage = nullptr;        // pinned staging of small counting calls
     size_t stage_bytes = 0;
